@@ -1,5 +1,6 @@
 // C ABI of the library (include/molt.h): argument validation, workspace
 // layout, TMA tensor maps and the launch sequence of each entry point.
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <cstring>
@@ -111,6 +112,24 @@ molt_status make_tmap(CUtensorMap* m, CUtensorMapDataType dt, int elem_bytes, co
   return MOLT_OK;
 }
 
+// bf16 matrix `rows` x `panels * 64` seen as [panel, row, 64]: boxes of 64 rows of
+// two neighbouring panels, panel after panel in shared memory.  Rows are
+// row_bytes apart, panels panel_bytes.
+molt_status make_tmap_panels(CUtensorMap* m, const void* base, uint64_t rows, uint64_t panels, uint64_t row_bytes,
+                             uint64_t panel_bytes) {
+  auto fn = encode_fn();
+  if (!fn) return fail(MOLT_ERR_CUDA, "cuTensorMapEncodeTiled entry point unavailable");
+  cuuint64_t dims[3] = {kBK, rows, panels};
+  cuuint64_t strides[2] = {row_bytes, panel_bytes};
+  cuuint32_t box[3] = {kBK, 64, 2};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(MOLT_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
+  return MOLT_OK;
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 inline size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -128,8 +147,70 @@ int choose_splits(int64_t Tcap, int64_t V, int n_sm) {
   return static_cast<int>(S);
 }
 
+// Backward over chunks (lmhead_bwd_chunk.cu): whether a call of this size takes
+// it, and what it needs of the workspace.  n_t, n_v, n_h, chunk_t and chunk_v
+// count 256-row tiles.
+struct ChunkPlan {
+  bool use = false;
+  int64_t n_t = 0, n_v = 0, n_h = 0, chunk_t = 0, chunk_v = 0, max_chunks = 0;
+  int64_t panel_rows = 0, buf_panels = 0;   // of one chunk buffer: token rows of a panel, 64-column panels
+  int n_buf = 0;
+  bool one_token_chunk = false;
+  int64_t g_rows() const { return n_buf * buf_panels * panel_rows; }
+  size_t g_bytes() const { return use ? static_cast<size_t>(g_rows()) * kBK * 2 : 0; }
+  int64_t ctl_words() const { return use ? kChunkCtlHead + 2 * max_chunks : 0; }
+  int64_t turn_words() const { return use ? (n_t + n_v) * n_h * 16 : 0; }
+};
+// T is the call's row count; the rows with a gradient, at most as many, are
+// known on the device only.
+//
+// Which calls: against the kernels that hold g in one cluster (or CTA), this one
+// is 1.3 to 2.6 times faster from H = 640 on at any T (T = 700, H = 896, V =
+// 19000: 88 against 126 us; T = 16384, H = 4096, V = 151936: 38.0 against 54.4
+// ms), and for 256 < H < 640 from about 512 rows on (T = 2000, H = 320, V =
+// 19000: 108 against 163 us; but T = 64, H = 320, V = 100000: 170 against 82 us).
+// At H = 256 a logit tile is four K blocks and its epilogue and store are most of
+// it: the cluster kernel is up to 1.6 times faster (T = 300, V = 150000: 177
+// against 296 us), except on the smallest calls, where both wait for their chains
+// of tiles and this one's is shorter (T = 512, V = 4096: 26 against 31 us).
+//
+// Chunk size: 16 x 16 tiles (4096 x 4096) in two buffers drain least; measured on
+// T = 16384, H = 4096, V = 151936: 38.8 ms, against 40.5 for 8 x 16 in four, 39.5
+// for 12 x 20, 41.2 for 32 x 8.  With few tiles or a short H a chunk holds too
+// little between a tile and what it waits for, and more, smaller buffers are
+// faster (T = 5003, H = 320, V = 50257: 0.71 ms with 8 x 16 in four, 0.94 with 16
+// x 16; T = 3000, H = 1024, V = 32000: 0.40 with 16 x 8 in four, 0.49).  Up to
+// 1024 rows the vocabulary is cut into about eight chunks, so that dH, whose tiles
+// are few and as long as a chunk, spreads over the SMs.
+ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
+  ChunkPlan p;
+  if (T <= 0 || !(H >= 640 || (H > 256 && T >= 512) || (T <= 1024 && V <= 4096))) return p;
+  p.n_t = (T + 255) / 256;
+  p.n_v = (V + 255) / 256;
+  p.n_h = (H + 255) / 256;
+  p.chunk_t = 16;
+  p.chunk_v = 16;
+  if (p.n_t <= 4)
+    p.chunk_v = std::max<int64_t>(4, std::min<int64_t>(32, (p.n_v + 7) / 8));
+  else if (H < 1024)
+    p.chunk_t = 8;
+  else if (p.n_t * p.n_v < 2560)
+    p.chunk_v = 8;
+  const int64_t n_tc = (p.n_t + p.chunk_t - 1) / p.chunk_t, n_vc = (p.n_v + p.chunk_v - 1) / p.chunk_v;
+  const int64_t tiles = p.n_t * p.n_v + (p.n_t * n_vc + p.n_v * n_tc) * p.n_h;
+  p.use = tiles < (int64_t(1) << 30);   // claimed with a 32-bit counter
+  p.max_chunks = n_tc * n_vc;
+  const int64_t ct = std::min(p.n_t, p.chunk_t), cv = std::min(p.n_v, p.chunk_v);
+  p.panel_rows = ct * 256;
+  p.buf_panels = cv * 4;
+  // all buffers together stay at 64 MB, half of L2
+  p.n_buf = static_cast<int>(std::min<int64_t>(8, std::max<int64_t>(2, 512 / (ct * cv))));
+  p.one_token_chunk = n_tc == 1;
+  return p;
+}
+
 struct Layout {
-  size_t counts, row_map, pos, tok_p, b_p, adv_p, h_p, part, zx, lse, coef, tile_flag, tile_list, red, dh32, turns;
+  size_t counts, row_map, pos, tok_p, b_p, adv_p, h_p, part, zx, lse, coef, tile_flag, tile_list, red, dh32, turns, g, ctl;
   size_t lp_p, ent_p, ecoef, mu, gate_p;
   size_t live_map, live_of, h_l, tok_l, lse_l, coef_l, ecoef_l, mu_l, total;
 };
@@ -178,7 +259,12 @@ Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = 
   L.tile_list = take(ntile * 4);
   L.red = take(ntile * kRedSlots * 8);
   L.dh32 = with_bwd ? take(static_cast<size_t>(Tcap) * H * 4) : o;
-  L.turns = (with_bwd && det) ? take(static_cast<size_t>(turn_layout(Tcap, H, V).words) * 4) : kNoRegion;
+  const ChunkPlan cp = chunk_plan(T, H, V);
+  L.turns = (with_bwd && det)
+                ? take(static_cast<size_t>(cp.use ? cp.turn_words() : turn_layout(Tcap, H, V).words) * 4)
+                : kNoRegion;
+  L.g = with_bwd ? take(cp.g_bytes()) : o;
+  L.ctl = with_bwd ? take(static_cast<size_t>(cp.ctl_words()) * 4) : o;
   L.lp_p = with_bwd ? take(Tcap * 4) : o;
   L.ent_p = with_bwd ? take(Tcap * 4) : o;
   L.ecoef = with_bwd ? take(Tcap * 4) : o;
@@ -217,7 +303,7 @@ Layout vp_loss_layout(int64_t T) {
   L.red = take(ntile * kRedSlots * 8);
   L.live_map = take(Tcap * 4);
   L.live_of = take(Tcap * 4);
-  L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.dh32 = L.lp_p = L.ent_p = L.ecoef = L.mu = L.gate_p =
+  L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.dh32 = L.g = L.ctl = L.lp_p = L.ent_p = L.ecoef = L.mu = L.gate_p =
       L.h_l = L.tok_l = L.lse_l = L.coef_l = L.ecoef_l = L.mu_l = o;
   L.turns = kNoRegion;
   L.total = o + 256;
@@ -227,7 +313,7 @@ Layout vp_loss_layout(int64_t T) {
 // Workspace of one shard's backward (molt_vp_backward): the rows with a
 // gradient, packed (hidden, token, lse, m c / D), and the fp32 dhidden
 // accumulator by backward row.
-Layout vp_backward_layout(int64_t T, int64_t H) {
+Layout vp_backward_layout(int64_t T, int64_t H, int64_t V) {
   const int64_t Tcap = round_tiles(T);
   const int64_t ntile = Tcap / kTileM;
   Layout L{};
@@ -246,6 +332,9 @@ Layout vp_backward_layout(int64_t T, int64_t H) {
   L.lse_l = take(Tcap * 4);
   L.coef_l = take(Tcap * 4);
   L.dh32 = take(static_cast<size_t>(Tcap) * H * 4);
+  const ChunkPlan cp = chunk_plan(T, H, V);
+  L.g = take(cp.g_bytes());
+  L.ctl = take(static_cast<size_t>(cp.ctl_words()) * 4);
   L.row_map = L.pos = L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.coef = L.tile_flag = L.red =
       L.lp_p = L.ent_p = L.ecoef = L.mu = L.gate_p = L.ecoef_l = L.mu_l = o;
   L.turns = kNoRegion;
@@ -272,6 +361,8 @@ Workspace carve(void* base, const Layout& L) {
   w.red = reinterpret_cast<double*>(p + L.red);
   w.dh32 = reinterpret_cast<float*>(p + L.dh32);
   w.turns = L.turns != kNoRegion ? reinterpret_cast<uint32_t*>(p + L.turns) : nullptr;
+  w.g = reinterpret_cast<uint16_t*>(p + L.g);
+  w.ctl = reinterpret_cast<uint32_t*>(p + L.ctl);
   w.lp_p = reinterpret_cast<float*>(p + L.lp_p);
   w.ent_p = reinterpret_cast<float*>(p + L.ent_p);
   w.ecoef = reinterpret_cast<float*>(p + L.ecoef);
@@ -479,18 +570,68 @@ molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int3
   return MOLT_OK;
 }
 
-// Zero the backward's fp32 reduce-add targets on stream s: the dhidden
-// accumulator, the deterministic schedule's turn counters and, unless the call
-// accumulates into it, dW.
+// Zero what the backward adds to on stream s: the dhidden accumulator, the
+// chunk counters, the deterministic schedule's turn counters and, unless the
+// call accumulates into it or stores it whole, dW.
 molt_status zero_backward_targets(const Workspace& w, int64_t T, int64_t H, int64_t V, bool det, float* dW_out,
                                   int accumulate_dW, cudaStream_t s) {
   const int64_t Tcap = round_tiles(T);
+  const ChunkPlan cp = chunk_plan(T, H, V);
   MOLT_CUDA(cudaMemsetAsync(w.dh32, 0, static_cast<size_t>(Tcap) * H * sizeof(float), s), "memset dh32");
+  if (cp.use) MOLT_CUDA(cudaMemsetAsync(w.ctl, 0, static_cast<size_t>(cp.ctl_words()) * 4, s), "memset counters");
   if (det) {
-    const TurnLayout tl = turn_layout(Tcap, H, V);
-    MOLT_CUDA(cudaMemsetAsync(w.turns, 0, static_cast<size_t>(tl.words) * 4, s), "memset turns");
+    const int64_t words = cp.use ? cp.turn_words() : turn_layout(Tcap, H, V).words;
+    MOLT_CUDA(cudaMemsetAsync(w.turns, 0, static_cast<size_t>(words) * 4, s), "memset turns");
   }
-  if (!accumulate_dW) MOLT_CUDA(cudaMemsetAsync(dW_out, 0, static_cast<size_t>(V) * H * sizeof(float), s), "memset dW");
+  if (!accumulate_dW && !(cp.use && cp.one_token_chunk))
+    MOLT_CUDA(cudaMemsetAsync(dW_out, 0, static_cast<size_t>(V) * H * sizeof(float), s), "memset dW");
+  return MOLT_OK;
+}
+
+// The backward over chunks: as run_backward.
+molt_status run_backward_chunk(const DeviceInfo* di, const ChunkPlan& cp, const uint16_t* W, int64_t T, int64_t H,
+                               int64_t V, const Workspace& w, bool det, int det_clusters, bool with_ecoef,
+                               float* dW_out, int accumulate_dW, cudaStream_t stream) {
+  const int64_t Tcap = round_tiles(T);
+  const auto bf16 = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  const auto f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  const uint64_t g_rows = cp.g_rows();
+  ChunkMaps m;
+  MOLT_TRY(make_tmap(&m.h128, bf16, 2, w.h_l, Tcap, H, kBK, 128));
+  MOLT_TRY(make_tmap(&m.w128, bf16, 2, W, V, H, kBK, 128));
+  MOLT_TRY(make_tmap(&m.g128, bf16, 2, w.g, g_rows, kBK, kBK, 128));
+  MOLT_TRY(make_tmap(&m.g32, bf16, 2, w.g, g_rows, kBK, kBK, 32));
+  MOLT_TRY(make_tmap_panels(&m.h64x2, w.h_l, Tcap, H / kBK, H * 2, kBK * 2));
+  MOLT_TRY(make_tmap_panels(&m.w64x2, W, V, H / kBK, H * 2, kBK * 2));
+  MOLT_TRY(make_tmap_panels(&m.g64x2, w.g, cp.panel_rows, g_rows / cp.panel_rows, kBK * 2, cp.panel_rows * kBK * 2));
+  MOLT_TRY(make_tmap(&m.dh, f32, 4, w.dh32, Tcap, H, 32, 32));
+  MOLT_TRY(make_tmap(&m.dw, f32, 4, dW_out, V, H, 32, 32));
+  ChunkArgs a{};
+  a.tok_p = w.tok_l;
+  a.lse = w.lse_l;
+  a.coef = w.coef_l;
+  if (with_ecoef) {
+    a.ecoef = w.ecoef_l;
+    a.mu = w.mu_l;
+  }
+  a.counts = w.counts;
+  a.V = static_cast<int>(V);
+  a.H = static_cast<int>(H);
+  a.n_buf = cp.n_buf;
+  a.chunk_t = static_cast<int>(cp.chunk_t);
+  a.chunk_v = static_cast<int>(cp.chunk_v);
+  a.buf_panels = static_cast<int>(cp.buf_panels);
+  a.panel_rows = static_cast<int>(cp.panel_rows);
+  a.store_dw = cp.one_token_chunk && !accumulate_dW;
+  a.max_t = static_cast<int>(cp.n_t);
+  a.max_chunks = static_cast<int>(cp.max_chunks);
+  a.ctl = w.ctl;
+  a.det_turns = det ? w.turns : nullptr;
+  a.err = di->status;
+  const int ctas = det_clusters > 0 ? 4 * det_clusters : di->n_sm;
+  ev_start(3, stream);
+  MOLT_LAUNCH(launch_lmhead_bwd_chunk(m, a, ctas, stream), "lmhead backward");
+  ev_stop(3, stream);
   return MOLT_OK;
 }
 
@@ -503,6 +644,9 @@ molt_status zero_backward_targets(const Workspace& w, int64_t T, int64_t H, int6
 molt_status run_backward(const DeviceInfo* di, const uint16_t* W, int64_t T, int64_t H, int64_t V,
                          const Workspace& w, bool det, int n_det, bool with_ecoef, float* dW_out, int accumulate_dW,
                          bool zeroed, cudaStream_t stream) {
+  if (!zeroed) MOLT_TRY(zero_backward_targets(w, T, H, V, det, dW_out, accumulate_dW, stream));
+  if (const ChunkPlan cp = chunk_plan(T, H, V); cp.use)
+    return run_backward_chunk(di, cp, W, T, H, V, w, det, n_det, with_ecoef, dW_out, accumulate_dW, stream);
   const int64_t Tcap = round_tiles(T);
   const bool pair_bwd = (H % 128) == 0;   // the cluster backward
   CUtensorMap tm_wz, tm_wn, tm_dh, tm_dw;
@@ -520,7 +664,6 @@ molt_status run_backward(const DeviceInfo* di, const uint16_t* W, int64_t T, int
   MOLT_TRY(make_tmap(&tm_h64, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w.h_l, Tcap, H, kBK, 64));
   MOLT_TRY(make_tmap(&tm_dh, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w.dh32, Tcap, H, 32, 32));
   MOLT_TRY(make_tmap(&tm_dw, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dW_out, V, H, 32, 32));
-  if (!zeroed) MOLT_TRY(zero_backward_targets(w, T, H, V, det, dW_out, accumulate_dW, stream));
   const TurnLayout tl = turn_layout(Tcap, H, V);
   BwdArgs ba{};
   ba.tok_p = w.tok_l;
@@ -1036,7 +1179,7 @@ molt_status molt_vp_loss(const float* partials, int n_shards, const float* behav
 
 size_t molt_vp_backward_workspace_bytes(int64_t T, int64_t H, int64_t V_shard) {
   if (check_shape(T, H, V_shard) != MOLT_OK) return 0;
-  return vp_backward_layout(T, H).total;
+  return vp_backward_layout(T, H, V_shard).total;
 }
 
 molt_status molt_vp_backward(const uint16_t* hidden, const uint16_t* W_shard, const int32_t* tokens,
@@ -1059,7 +1202,7 @@ molt_status molt_vp_backward(const uint16_t* hidden, const uint16_t* W_shard, co
       MOLT_CUDA(cudaMemsetAsync(dW_shard_out, 0, V_shard * H * sizeof(float), stream), "memset dW");
     return MOLT_OK;
   }
-  const Layout L = vp_backward_layout(T, H);
+  const Layout L = vp_backward_layout(T, H, V_shard);
   Scratch sc;
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);

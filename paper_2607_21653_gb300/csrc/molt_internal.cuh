@@ -43,6 +43,9 @@ struct Workspace {
   float* ecoef_l;       // [Tcap] entropy-bonus coefficient (extended objective)
   float* mu_l;          // [Tcap]
   uint32_t* turns;      // deterministic schedule: abort word + turn counters, or nullptr
+  // backward over chunks
+  uint16_t* g;          // chunk buffers of the softmax gradient (bf16 bits)
+  uint32_t* ctl;        // tile counter, abort word, per-chunk counters
   // extended objective (loss call only)
   float* lp_p;          // [Tcap] packed log-probs
   float* ent_p;         // [Tcap] packed entropies
@@ -86,6 +89,35 @@ struct BwdArgs {
   uint32_t* det_abort;       // deterministic: set once any turn wait gives up (zeroed per call)
   uint32_t* det_dh_turns;    // deterministic: [token quads, H jobs, 32] counters, blocks done
   uint32_t* det_dw_turns;    // deterministic: [vocab blocks, H jobs, 32] counters, quads done
+  unsigned* err;
+};
+
+// backward over chunks of the tokens x vocabulary plane (lmhead_bwd_chunk.cu)
+constexpr int kChunkCtlHead = 64;    // control words before the per-chunk counters:
+                                     // [0] next tile, [1] set once any wait gives up
+struct ChunkMaps {                   // bf16 maps have 64-column (128-byte) boxes
+  CUtensorMap h128, w128;            // packed hidden rows and W, 128 rows
+  CUtensorMap g128, g32;             // chunk buffers: 64-column panels of token rows; g32 stores
+  CUtensorMap h64x2, w64x2, g64x2;   // as [column box or panel, row, 64]: 64 rows of two boxes side by side
+  CUtensorMap dh, dw;                // fp32 targets, 32 x 32 boxes
+};
+struct ChunkArgs {
+  const int32_t* tok_p;
+  const float* lse;
+  const float* coef;
+  const float* ecoef;        // or nullptr
+  const float* mu;
+  const int32_t* counts;     // counts[3] = rows
+  int V, H;
+  int chunk_t, chunk_v;      // a chunk's tiles of tokens and vocab, at most
+  int n_buf;                 // chunk buffers (>= 2)
+  int buf_panels;            // 64-column panels of one buffer
+  int panel_rows;            // token rows of one panel (128 bytes each)
+  int store_dw;              // dW is stored, not added to (one token chunk)
+  int max_t;                 // token tiles of the call's capacity
+  int max_chunks;
+  uint32_t* ctl;             // zeroed: kChunkCtlHead words, then tiles stored and tiles read per chunk
+  uint32_t* det_turns;       // reproducible sums: zeroed [token tiles + vocab tiles, H tiles, 16] counters, or nullptr
   unsigned* err;
 };
 
@@ -162,6 +194,8 @@ void note_launches(int n);
 cudaError_t launch_lmhead_bwd_quad(const CUtensorMap& tm_hz, const CUtensorMap& tm_wz, const CUtensorMap& tm_h,
                                    const CUtensorMap& tm_w_n, const CUtensorMap& tm_dh, const CUtensorMap& tm_dw,
                                    const BwdArgs& a, int n_sm, cudaStream_t s);
+// lmhead_bwd_chunk.cu
+cudaError_t launch_lmhead_bwd_chunk(const ChunkMaps& m, const ChunkArgs& a, int n_ctas, cudaStream_t s);
 // lmhead_bwd.cu
 cudaError_t launch_lmhead_bwd(const CUtensorMap& tm_h, const CUtensorMap& tm_w_z, const CUtensorMap& tm_w_n,
                               const CUtensorMap& tm_dh, const CUtensorMap& tm_dw, const BwdArgs& a, int grid,

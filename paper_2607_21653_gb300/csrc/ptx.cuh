@@ -113,6 +113,13 @@ __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* m, uint32_t
                "r"(src), "r"(x), "r"(y)
                : "memory");
 }
+// store of a shared-memory box to global memory
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, uint32_t src, int32_t x, int32_t y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(m)),
+               "r"(src), "r"(x), "r"(y)
+               : "memory");
+}
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void bulk_wait_group_read() {
@@ -142,6 +149,9 @@ __device__ __forceinline__ uint32_t ld_relaxed_gpu(const uint32_t* p) {
 }
 __device__ __forceinline__ void st_release_gpu(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void red_add_release_gpu(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 // Bounded wait until the counter *turn (raised by other CTAs with release
 // stores) reaches `target`.  Gives up at once when this CTA or the call has
@@ -342,6 +352,9 @@ __device__ __forceinline__ void st_shared_cluster_v4(uint32_t cluster_addr, uint
                "r"(d)
                : "memory");
 }
+__device__ __forceinline__ void st_shared_cluster_u32(uint32_t cluster_addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ void fence_proxy_async_cluster() {
   asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
 }
@@ -352,6 +365,13 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* m, uint32_t bar_cluster,
+                                                 int32_t x, int32_t y, int32_t z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster), "r"(x), "r"(y), "r"(z)
       : "memory");
 }
 // TMEM allocation / MMA / commit for a CTA pair (cta_group::2): allocation and
@@ -374,6 +394,26 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, 
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// four products in a row, the operands' descriptors advancing by a_step and b_step
+// (their low words; the offsets stay inside the address field): one statement, so
+// that nothing is scheduled between the products
+__device__ __forceinline__ void umma4_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t a_step,
+                                                uint32_t b_step, uint32_t idesc, uint32_t accumulate) {
+  const uint32_t a0 = static_cast<uint32_t>(adesc), ah = static_cast<uint32_t>(adesc >> 32);
+  const uint32_t b0 = static_cast<uint32_t>(bdesc), bh = static_cast<uint32_t>(bdesc >> 32);
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 a0, a1, a2, a3, b0, b1, b2, b3;\n\t"
+      "setp.ne.b32 p, %11, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"
+      "mov.b64 a0, {%1, %5};\n\tmov.b64 a1, {%2, %5};\n\tmov.b64 a2, {%3, %5};\n\tmov.b64 a3, {%4, %5};\n\t"
+      "mov.b64 b0, {%6, %10};\n\tmov.b64 b1, {%7, %10};\n\tmov.b64 b2, {%8, %10};\n\tmov.b64 b3, {%9, %10};\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a0, b0, %12, p;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a1, b1, %12, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a2, b2, %12, q;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], a3, b3, %12, q;\n}" ::"r"(d_tmem),
+      "r"(a0), "r"(a0 + a_step), "r"(a0 + 2 * a_step), "r"(a0 + 3 * a_step), "r"(ah), "r"(b0), "r"(b0 + b_step),
+      "r"(b0 + 2 * b_step), "r"(b0 + 3 * b_step), "r"(bh), "r"(accumulate), "r"(idesc)
       : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem]^T for a CTA pair: A is read from TMEM (each CTA

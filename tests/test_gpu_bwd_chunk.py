@@ -1,0 +1,75 @@
+"""The backward over chunks (csrc/lmhead_bwd_chunk.cu) where its tile list can go
+wrong: one row, tiles and chunks with remainders in both directions, a last H
+tile of 64 to 192 columns, one and several token chunks (dW stored or added to),
+a call without any gradient row, and the lines of the rule that chooses it."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2607_21653_gb300 as molt  # noqa: E402
+from oracle import molt_oracle as O  # noqa: E402
+from workloads import random_problem  # noqa: E402
+
+from parity import assert_grad_close, assert_loss_close, behavior_from_oracle, bf, np_, t  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    molt.build()
+    molt.load()
+
+
+def _run(args, **kw):
+    out = molt.policy_loss_fwd_bwd_ex(*args, 0.2, 0.28, **kw)
+    torch.cuda.synchronize()
+    assert molt.device_status() == 0
+    return out
+
+
+# (1, 640, 1): one row, one column; (257, 704, 513): remainders of one row, column
+# and a 192-column H tile; (512, 320, 4097): the rule's least T for this H, a
+# 64-column H tile; (1024, 256, 4096): the largest call the rule takes at H = 256;
+# (2049, 640, 2100): two token chunks of 8 tiles at most; (4200, 1088, 4400): two
+# chunks in both directions, a 64-column H tile
+@pytest.mark.parametrize("T,H,V", [(1, 640, 1), (257, 704, 513), (512, 320, 4097), (1024, 256, 4096),
+                                   (2049, 640, 2100), (4200, 1088, 4400)])
+def test_chunk_backward_matches_oracle(T, H, V):
+    rng = np.random.default_rng(T + H + V)
+    h, W, x, m = random_problem(rng, T, H, V, mask_frac=0.1 if T > 1 else 0.0, w_std=0.05)
+    m[-1] = 1
+    adv = rng.standard_normal(T).astype(np.float32)
+    h64, W64 = O.widen_bf16(h), O.widen_bf16(W)
+    b = behavior_from_oracle(h64, W64, x, 0.3, 0.2, 0.28, T)
+    ref = O.policy_loss(h64, W64, x, b.astype(np.float64), adv.astype(np.float64), m, 0.2, 0.28)
+    ref["_adv"] = adv.astype(np.float64)
+    args = (bf(h), bf(W), t(x), t(b), t(adv), t(m))
+    out = _run(args)
+    assert_loss_close(float(out["loss"].item()), ref)
+    assert_grad_close(np_(out["dhidden"]), ref["dH"], "dhidden")
+    assert_grad_close(np_(out["dW"]), ref["dW"], "dW")
+    # added onto the caller's dW instead of stored
+    dW0 = torch.randn(V, H, device="cuda", generator=torch.Generator(device="cuda").manual_seed(T))
+    acc = dW0.clone()
+    _run(args, dW=acc, accumulate_dW=True)
+    assert_grad_close(np_(acc - dW0), ref["dW"], "dW accumulated")
+    # the entropy term, whose gradient has no oracle slice of its own here: the
+    # plain gradient is what is left of it at coefficient 0 and the term is linear
+    e1, e2 = (_run(args, entropy_coef=c) for c in (0.01, 0.02))
+    d1, d2 = (np_(e["dW"]) - np_(out["dW"]) for e in (e1, e2))
+    if V > 1:
+        assert np.abs(d2 - 2 * d1).max() <= 2e-2 * np.abs(d2).max() + 2e-2 * np.abs(ref["dW"]).max()
+    # no row with a gradient: everything 0, dW included, whatever it held
+    dW = torch.full((V, H), float("nan"), device="cuda")
+    zero = _run((*args[:4], torch.zeros_like(args[4]), args[5]), dW=dW)
+    assert (np_(zero["dW"]) == 0).all() and (np_(zero["dhidden"]) == 0).all()
+    if H % 128 == 0:
+        det = [_run(args, deterministic=True, det_clusters=n) for n in (0, 0, 4)]
+        assert_grad_close(np_(det[0]["dW"]), ref["dW"], "dW deterministic")
+        for o in det[1:]:
+            for k in ("dW", "dhidden"):
+                np.testing.assert_array_equal(np_(o[k]).view(np.uint8), np_(det[0][k]).view(np.uint8), err_msg=k)
