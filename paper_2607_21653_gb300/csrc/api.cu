@@ -136,17 +136,6 @@ inline size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
 int64_t round_tiles(int64_t T) { return ((T + kTileM - 1) / kTileM) * kTileM; }
 
-// vocab splits of the forward pass: enough units for ~16 waves of CTAs when
-// every row is active, never more splits than vocab tiles
-int choose_splits(int64_t Tcap, int64_t V, int n_sm) {
-  const int64_t n_vt = (V + kFwdBN - 1) / kFwdBN;
-  const int64_t n_mt = Tcap / kTileM;
-  int64_t S = (16 * static_cast<int64_t>(n_sm) + n_mt - 1) / n_mt;
-  if (S < 1) S = 1;
-  if (S > n_vt) S = n_vt;
-  return static_cast<int>(S);
-}
-
 // Backward over chunks (lmhead_bwd_chunk.cu): whether a call of this size takes
 // it, and what it needs of the workspace.  n_t, n_v, n_h, chunk_t and chunk_v
 // count 256-row tiles.
@@ -251,7 +240,7 @@ Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = 
   L.b_p = take(Tcap * 4);
   L.adv_p = take(Tcap * 4);
   L.h_p = take(Tcap * H * 2);
-  L.part = take(static_cast<size_t>(S) * Tcap * 16);
+  L.part = take(static_cast<size_t>(kFwdParts) * S * Tcap * 16);
   L.zx = take(Tcap * 4);
   L.lse = take(Tcap * 4);
   L.coef = take(Tcap * 4);
@@ -561,6 +550,7 @@ molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int3
   fa.H = static_cast<int>(H);
   fa.n_split = S;
   fa.n_vtiles = static_cast<int>((V + kFwdBN - 1) / kFwdBN);
+  fa.next_unit = w.counts + 4;
   fa.part = w.part;
   fa.zx = w.zx;
   fa.err = di->status;
@@ -782,7 +772,7 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
     return MOLT_OK;
   }
   const int64_t Tcap = round_tiles(T);
-  const int S = choose_splits(Tcap, V, di->n_sm);
+  const int S = forward_splits(Tcap, H, V, di->n_sm);
   // deterministic schedule: n_det clusters (a multiple of 4), all resident at
   // once, whose reduce-adds take turns
   int n_det = det ? lmhead_bwd_quad_det_clusters(di->n_sm) : 0;
@@ -801,7 +791,7 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
   const Workspace w = carve(sc.ptr, L);
   CUtensorMap tm_h, tm_w;
   MOLT_TRY(make_tmap(&tm_h, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w.h_p, Tcap, H, kBK, kTileM));
-  MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, V, H, kBK, kFwdBN));
+  MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, V, H, kBK, 128));
   // the backward's targets are zeroed on the side lane while the forward runs;
   // the caller's stream waits for them before the backward, or on any early
   // return before the workspace is released
@@ -827,14 +817,14 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
   if (token_loss_out) MOLT_CUDA(cudaMemsetAsync(token_loss_out, 0, T * sizeof(float), stream), "memset token loss");
   ev_start(2, stream);
   if (opts) {
-    MOLT_LAUNCH(launch_merge_stats_ex(static_cast<int>(Tcap), static_cast<int>(V), S, w, logp_out, entropy_out,
+    MOLT_LAUNCH(launch_merge_stats_ex(static_cast<int>(Tcap), static_cast<int>(V), kFwdParts * S, w, logp_out, entropy_out,
                                     di->status, stream),
               "merge");
     MOLT_LAUNCH(launch_seq_gate(static_cast<int>(T), static_cast<int>(Tcap), ex, w, di->status, stream), "gate");
     MOLT_LAUNCH(launch_loss_rows_ex(static_cast<int>(Tcap), denom, clip_lo, clip_hi, ex, w, token_loss_out, stream),
               "loss rows");
   } else {
-    MOLT_LAUNCH(launch_merge(true, static_cast<int>(Tcap), static_cast<int>(V), S, denom, clip_lo, clip_hi, w,
+    MOLT_LAUNCH(launch_merge(true, static_cast<int>(Tcap), static_cast<int>(V), kFwdParts * S, denom, clip_lo, clip_hi, w,
                            logp_out, entropy_out, token_loss_out, di->status, stream),
               "merge");
   }
@@ -874,6 +864,17 @@ int device_sm_count() {
   molt_status st;
   const DeviceInfo* di = device_info(&st);
   return di ? di->n_sm : 1;
+}
+
+// Enough units for 24 waves of CTA pairs when every row is active, so that the
+// last wave is a small part of the whole, but at least 64 K blocks to a unit as
+// long as four waves are left (at H = 320 a tile is five K blocks, and handing
+// over a unit costs about as much), and never more splits than vocab tiles.
+int forward_splits(int64_t Tcap, int64_t H, int64_t V, int n_sm) {
+  const int64_t n_vt = (V + kFwdBN - 1) / kFwdBN, n_mt = (Tcap + 255) / 256, pairs = n_sm / 2;
+  auto waves = [&](int64_t w) { return (w * pairs + n_mt - 1) / n_mt; };
+  const int64_t S = std::min(waves(24), std::max(waves(4), n_vt * (H / kBK) / 64));
+  return static_cast<int>(std::max<int64_t>(1, std::min(S, n_vt)));
 }
 
 molt_status encode_tmap_2d(CUtensorMap* m, CUtensorMapDataType dt, int elem_bytes, const void* base, uint64_t rows,
@@ -1007,7 +1008,7 @@ size_t molt_token_logprobs_workspace_bytes(int64_t T, int64_t H, int64_t V) {
   const DeviceInfo* di = device_info(&st);
   const int n_sm = di ? di->n_sm : 152;
   const int64_t Tcap = round_tiles(T);
-  return layout(T, H, V, choose_splits(Tcap > 0 ? Tcap : kTileM, V, n_sm), false).total;
+  return layout(T, H, V, forward_splits(Tcap > 0 ? Tcap : kTileM, H, V, n_sm), false).total;
 }
 
 size_t molt_policy_loss_workspace_bytes(int64_t T, int64_t H, int64_t V) {
@@ -1016,7 +1017,7 @@ size_t molt_policy_loss_workspace_bytes(int64_t T, int64_t H, int64_t V) {
   const DeviceInfo* di = device_info(&st);
   const int n_sm = di ? di->n_sm : 152;
   const int64_t Tcap = round_tiles(T);
-  return layout(T, H, V, choose_splits(Tcap > 0 ? Tcap : kTileM, V, n_sm), true).total;
+  return layout(T, H, V, forward_splits(Tcap > 0 ? Tcap : kTileM, H, V, n_sm), true).total;
 }
 
 size_t molt_policy_loss_workspace_bytes_ex(int64_t T, int64_t H, int64_t V, const molt_loss_options* opts) {
@@ -1027,7 +1028,7 @@ size_t molt_policy_loss_workspace_bytes_ex(int64_t T, int64_t H, int64_t V, cons
   const DeviceInfo* di = device_info(&st);
   const int n_sm = di ? di->n_sm : 152;
   const int64_t Tcap = round_tiles(T);
-  return layout(T, H, V, choose_splits(Tcap > 0 ? Tcap : kTileM, V, n_sm), true, det).total;
+  return layout(T, H, V, forward_splits(Tcap > 0 ? Tcap : kTileM, H, V, n_sm), true, det).total;
 }
 
 molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, const int32_t* tokens,
@@ -1042,19 +1043,19 @@ molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, c
   const DeviceInfo* di = device_info(&st);
   if (!di) return st;
   const int64_t Tcap = round_tiles(T);
-  const int S = choose_splits(Tcap, V, di->n_sm);
+  const int S = forward_splits(Tcap, H, V, di->n_sm);
   const Layout L = layout(T, H, V, S, false);
   Scratch sc;
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
   CUtensorMap tm_h, tm_w;
   MOLT_TRY(make_tmap(&tm_h, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w.h_p, Tcap, H, kBK, kTileM));
-  MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, V, H, kBK, kFwdBN));
+  MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, V, H, kBK, 128));
   MOLT_TRY(run_forward(di, hidden, tokens, mask, nullptr, nullptr, T, H, V, S, w, tm_h, tm_w, stream));
   MOLT_CUDA(cudaMemsetAsync(logp_out, 0, T * sizeof(float), stream), "memset logp");
   if (entropy_out) MOLT_CUDA(cudaMemsetAsync(entropy_out, 0, T * sizeof(float), stream), "memset entropy");
   ev_start(2, stream);
-  MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
+  MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), kFwdParts * S, 0.0, 0.f, 0.f, w, logp_out,
                          entropy_out, nullptr, di->status, stream),
             "merge");
   ev_stop(2, stream);
@@ -1108,18 +1109,18 @@ molt_status molt_vp_partials(const uint16_t* hidden, const uint16_t* W_shard, co
   const DeviceInfo* di = device_info(&st);
   if (!di) return st;
   const int64_t Tcap = round_tiles(T);
-  const int S = choose_splits(Tcap, V_shard, di->n_sm);
+  const int S = forward_splits(Tcap, H, V_shard, di->n_sm);
   const Layout L = layout(T, H, V_shard, S, false);
   Scratch sc;
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
   CUtensorMap tm_h, tm_w;
   MOLT_TRY(make_tmap(&tm_h, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w.h_p, Tcap, H, kBK, kTileM));
-  MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W_shard, V_shard, H, kBK, kFwdBN));
+  MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W_shard, V_shard, H, kBK, 128));
   MOLT_TRY(run_forward(di, hidden, tokens, mask, nullptr, nullptr, T, H, V_shard, S, w, tm_h, tm_w, stream,
                        static_cast<int>(v_begin)));
   ev_start(2, stream);
-  MOLT_LAUNCH(launch_vp_local(static_cast<int>(T), static_cast<int>(Tcap), static_cast<int>(V_shard), S, w,
+  MOLT_LAUNCH(launch_vp_local(static_cast<int>(T), static_cast<int>(Tcap), static_cast<int>(V_shard), kFwdParts * S, w,
                               reinterpret_cast<float4*>(partials_out), stream),
               "shard statistics");
   ev_stop(2, stream);

@@ -2,21 +2,37 @@
 // actor's recomputed log-probabilities of the generated tokens, plus entropy).
 //
 // z = h W^T is never written to global memory.  Each work unit is one tile of
-// 128 packed token rows times one contiguous split of the vocabulary.  For
-// every 256-column vocab tile of the split, the tensor cores accumulate the
-// 128 x 256 fp32 logit tile in TMEM (K = H in 64-element steps fed by TMA), and
-// the epilogue warps fold it into per-row running statistics:
+// 256 packed token rows times one contiguous split of the vocabulary.  For
+// every 256-column vocab tile of the split, the tensor cores of a CTA pair
+// accumulate the 256 x 256 fp32 logit tile in TMEM (128 rows in each CTA; K = H
+// in 64-element steps fed by TMA), and the epilogue warps fold it into per-row
+// running statistics:
 //   m = running max, s = sum exp(z - m), q = sum exp(z - m) (z - m)
-// and pick the target logit z[x].  The split's (m, s, q) go to a small
-// workspace; a row-level merge kernel combines the splits into
+// and pick the target logit z[x].  The split's (m, s, q), one set for each
+// column half, go to a small workspace; a row-level merge kernel combines them
+// into
 //   lse = m + log s,  logp = z[x] - lse,  entropy = log s - q / s.
 //
-// Roles (192 threads, one CTA per SM, persistent over units):
-//   warp 0      TMA producer (one lane): h tile [128 x 64] + W tile [256 x 64]
-//               per stage, 128-byte swizzle, 4-stage ring
-//   warp 1      MMA issuer (one lane): tcgen05.mma kind::f16, M=128 N=256 K=16,
-//               double-buffered accumulators (2 x 256 TMEM columns)
-//   warps 2-5   epilogue: each thread owns one TMEM lane = one token row
+// What bounds it: the tensor cores under the board's power cap, so the bytes
+// moved per product count as much as the time they take.  A pair loads 64 bytes
+// of operands per clock and SM at full rate where a single CTA's 128 x 256 tile
+// loads 96.  Units are taken 16 token tiles at a time, all of them on one vocab
+// split before the next, so that W comes from HBM once per 4096 rows and the
+// pairs in flight read the same W tiles.  Measured in a loop at the power cap
+// (T = 32768, H = 4096, V = 151936): 22.98 ms, 1.78 PFLOP/s, against 25.44 ms for
+// 128 x 256 tiles on single CTAs; with groups of 8, 32 and 76 token tiles 23.20,
+// 24.73 and 27.04 ms.  T = 1031: 0.90 against 1.72 ms (W came from HBM once per
+// 128 rows); T = 5003, H = 320, V = 50257: 0.162 against 0.174 ms.
+//
+// Roles per CTA (384 threads; clusters of two CTAs, persistent, units claimed
+// from a counter):
+//   warps 0, 11  TMA producers: h tile [128 x 64] and W tile [128 x 64] of this
+//                CTA per stage, 128-byte swizzle, 7-stage ring
+//   warp 1       MMA issuer (even CTA): tcgen05.mma cta_group::2 kind::f16, M=256
+//                N=256 K=16, double-buffered accumulators (2 x 256 TMEM columns)
+//   warps 2-9    epilogue, two per TMEM lane quarter: each thread owns one TMEM
+//                lane = one token row, and 128 of the 256 columns
+//   warp 10      even CTA: claims units and hands them to every role of both CTAs
 #include <atomic>
 #include <cstdint>
 #include <cuda.h>
@@ -28,19 +44,22 @@
 namespace molt {
 namespace {
 
-constexpr int kStages = 4;
-constexpr int kABytes = kTileM * kBK * 2;        // 16 KB
-constexpr int kBBytes = kFwdBN * kBK * 2;        // 32 KB
-constexpr int kStageBytes = kABytes + kBBytes;   // 48 KB
-constexpr int kThreads = 192;
+constexpr int kStages = 7;
+constexpr int kHalf = 128 * kBK * 2;             // one operand's half of a stage, 16 KB
+constexpr int kStageBytes = 2 * kHalf;           // 32 KB per CTA
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 128 + 32 * kEpiWarps;
 constexpr int kSmemBytes = kStages * kStageBytes + 1024;
-constexpr uint32_t kIdesc = idesc_bf16_f32(kTileM, kFwdBN, false, false);
+constexpr int kSlots = 2;                        // units handed from the claiming warp to the other roles
+constexpr int kGroup = 16;                       // token tiles that share a pass over the vocabulary
+constexpr uint32_t kIdesc = idesc_bf16_f32(256, 256, false, false);
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
 __device__ __forceinline__ void split_range(int s, int S, int n_vt, int& vt0, int& vt1) {
-  vt0 = static_cast<int>(static_cast<int64_t>(s) * n_vt / S);
-  vt1 = static_cast<int>(static_cast<int64_t>(s + 1) * n_vt / S);
+  const int per = n_vt / S, more = n_vt - per * S;   // the first `more` splits take one tile more
+  vt0 = s * per + min(s, more);
+  vt1 = vt0 + per + (s < more ? 1 : 0);
 }
 
 // fold 32 logits (all columns valid) into the running (m, s, q2) of one row;
@@ -102,20 +121,34 @@ __device__ __forceinline__ void fold_partial(const float (&v)[32], int nv, float
   }
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+// unit u of the list: 256-row token tile and vocab split
+__device__ __forceinline__ void unit_of(int u, int n_mt, int S, int& mt, int& s) {
+  const int g = u / (kGroup * S);
+  const int r = u - g * kGroup * S;
+  const int g_mt = min(kGroup, n_mt - g * kGroup);
+  s = r / g_mt;
+  mt = g * kGroup + (r - s * g_mt);
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     lmhead_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
                       const FwdArgs a) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[kStages];
-  __shared__ __align__(8) uint64_t empty_bar[kStages];
-  __shared__ __align__(8) uint64_t accf_bar[2];
-  __shared__ __align__(8) uint64_t acce_bar[2];
+  __shared__ __align__(8) uint64_t full_bar[kStages];    // even CTA: both CTAs' bytes land here
+  __shared__ __align__(8) uint64_t empty_bar[kStages];   // both CTAs
+  __shared__ __align__(8) uint64_t accf_bar[2];          // both CTAs: accumulator full
+  __shared__ __align__(8) uint64_t acce_bar[2];          // even CTA: one arrival per epilogue warp of the pair
+  __shared__ __align__(8) uint64_t ufull_bar[kSlots];    // both CTAs: unit index written
+  __shared__ __align__(8) uint64_t uempty_bar[kSlots];   // even CTA: every reader of both CTAs has it
   __shared__ __align__(8) uint64_t done_bar;
+  __shared__ int unit_sh[kSlots];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
 
   const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const bool leader = rank == 0;
   volatile int* abort_flag = &abort_sh;
 
   if (threadIdx.x == 0) {
@@ -125,127 +158,178 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&accf_bar[b]), 1);
-      mbar_init(smem_u32(&acce_bar[b]), 128);
+      mbar_init(smem_u32(&acce_bar[b]), 2 * kEpiWarps);
+    }
+    for (int s = 0; s < kSlots; ++s) {
+      mbar_init(smem_u32(&ufull_bar[s]), 1);
+      // readers: the MMA issuer, four producer warps, every epilogue warp
+      mbar_init(smem_u32(&uempty_bar[s]), 5 + 2 * kEpiWarps);
     }
     mbar_init(smem_u32(&done_bar), 1);
     abort_sh = 0;
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&tmem_base_sh), 512);
-    tmem_relinquish();
+    tmem_alloc_pair(smem_u32(&tmem_base_sh), 512);
+    tmem_relinquish_pair();
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();   // both CTAs' barriers exist before any remote arrival
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
 
   const int n_rows = a.counts[0];
-  const int n_mt = (n_rows + kTileM - 1) / kTileM;
+  const int n_mt = (n_rows + 255) / 256;
   const int S = a.n_split;
   const int n_units = n_mt * S;
   const int kblocks = a.H / kBK;
 
-  if (warp == 0) {
+  // the next unit for a reader of the slot ring (called by one lane); -1 ends
+  // the walk, also after a wait that ran out
+  const uint32_t uempty_lead0 = mapa_shared(smem_u32(&uempty_bar[0]), 0);
+  auto next_unit = [&](uint32_t i) -> int {
+    const uint32_t s = i % kSlots;
+    if (!mbar_wait_cluster(smem_u32(&ufull_bar[s]), (i / kSlots) & 1u, abort_flag, a.err)) return -1;
+    const int u = *reinterpret_cast<volatile int*>(&unit_sh[s]);
+    if (u >= -1) mbar_arrive_cluster_relaxed(uempty_lead0 + s * 8);   // always; orders the arrival after the read
+    return u;
+  };
+
+  if (warp == 0 || warp == 3 + kEpiWarps) {
     if (lane == 0) {
-      prefetch_tmap(&tm_h);
-      prefetch_tmap(&tm_w);
-      uint32_t it = 0;
+      const bool is_a = warp == 0;
+      const CUtensorMap* map = is_a ? &tm_h : &tm_w;
+      prefetch_tmap(map);
+      const uint32_t full_lead0 = mapa_shared(smem_u32(&full_bar[0]), 0);
+      const uint32_t dst0 = smem0 + (is_a ? 0 : kHalf);
+      uint32_t st = 0, ph = 0, n_it = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-        const int mt = u / S, s = u - mt * S;
-        int vt0, vt1;
+      int u = next_unit(0);
+      for (uint32_t ui = 0; u >= 0 && ok; ++ui) {
+        int mt, s, vt0, vt1;
+        unit_of(u, n_mt, S, mt, s);
         split_range(s, S, a.n_vtiles, vt0, vt1);
         for (int vt = vt0; vt < vt1 && ok; ++vt) {
+          const int y = (is_a ? mt : vt) * 256 + static_cast<int>(rank) * 128;
           for (int kb = 0; kb < kblocks; ++kb) {
-            const uint32_t st = it % kStages, ph = (it / kStages) & 1u;
-            if (!mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abort_flag, a.err)) {
-              ok = false;
-              break;
+            if (!(ok = mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abort_flag, a.err))) break;
+            if (is_a && leader) mbar_arrive_expect_tx(smem_u32(&full_bar[st]), 2 * kStageBytes);
+            tma_load_2d_pair(dst0 + st * kStageBytes, map, full_lead0 + st * 8, kb * kBK, y);
+            ++n_it;
+            if (++st == kStages) {
+              st = 0;
+              ph ^= 1u;
             }
-            const uint32_t sa = smem0 + st * kStageBytes;
-            const uint32_t fb = smem_u32(&full_bar[st]);
-            mbar_arrive_expect_tx(fb, kStageBytes);
-            tma_load_2d(sa, &tm_h, fb, kb * kBK, mt * kTileM);
-            tma_load_2d(sa + kABytes, &tm_w, fb, kb * kBK, vt * kFwdBN);
-            ++it;
           }
         }
+        if (ok) u = next_unit(ui + 1);
       }
-      // exit path: every issued copy must land before the CTA's smem goes away
-      const uint32_t first = it > (uint32_t)kStages ? it - kStages : 0u;
-      for (uint32_t j = first; j < it; ++j)
-        mbar_wait_drain(smem_u32(&full_bar[j % kStages]), (j / kStages) & 1u, a.err);
+      if (leader && is_a) {
+        // every copy into both CTAs completes on these barriers: wait for the
+        // last issued stages before the pair may exit
+        const uint32_t first = n_it > (uint32_t)kStages ? n_it - kStages : 0u;
+        for (uint32_t j = first; j < n_it; ++j)
+          mbar_wait_drain(smem_u32(&full_bar[j % kStages]), (j / kStages) & 1u, a.err);
+      }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t it = 0, acc_it = 0;
+    if (lane == 0 && leader) {
+      uint32_t st = 0, ph = 0, acc_it = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-        const int mt = u / S, s = u - mt * S;
-        (void)mt;
-        int vt0, vt1;
+      const uint64_t ad0 = sdesc_sw128(smem0, 16, 1024), bd0 = sdesc_sw128(smem0 + kHalf, 16, 1024);
+      int u = next_unit(0);
+      for (uint32_t ui = 0; u >= 0 && ok; ++ui) {
+        int mt, s, vt0, vt1;
+        unit_of(u, n_mt, S, mt, s);
         split_range(s, S, a.n_vtiles, vt0, vt1);
         for (int vt = vt0; vt < vt1 && ok; ++vt) {
-          const uint32_t buf = acc_it & 1u, aph = (acc_it >> 1) & 1u;
-          if (!mbar_wait(smem_u32(&acce_bar[buf]), aph ^ 1u, abort_flag, a.err)) {
-            ok = false;
-            break;
-          }
+          const uint32_t buf = acc_it & 1u;
+          if (!(ok = mbar_wait(smem_u32(&acce_bar[buf]), ((acc_it >> 1) & 1u) ^ 1u, abort_flag, a.err))) break;
           tc_fence_after();
-          const uint32_t d = tmem_base + buf * kFwdBN;
-          for (int kb = 0; kb < kblocks; ++kb) {
-            const uint32_t st = it % kStages, ph = (it / kStages) & 1u;
-            if (!mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag, a.err)) {
-              ok = false;
-              break;
+          const uint32_t d = tmem_base + buf * 256;
+          auto issue = [&](uint32_t stage, uint32_t accumulate) {
+            umma4_bf16_pair(d, ad0 + stage * (kStageBytes >> 4), bd0 + stage * (kStageBytes >> 4), 2u, 2u, kIdesc,
+                            accumulate);
+            umma_commit_pair_mc(smem_u32(&empty_bar[stage]), 3);
+          };
+          // two stages per turn: one wait of the issuing thread for eight products
+          for (int kb = 0; kb < kblocks; kb += 2) {
+            const bool two = kb + 1 < kblocks;
+            const uint32_t st0 = st;
+            if (!(ok = mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag, a.err))) break;
+            if (++st == kStages) {
+              st = 0;
+              ph ^= 1u;
             }
+            if (two && !(ok = mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag, a.err))) break;
             tc_fence_after();
-            const uint32_t sa = smem0 + st * kStageBytes;
-            const uint64_t ad = sdesc_sw128(sa, 16, 1024);
-            const uint64_t bd = sdesc_sw128(sa + kABytes, 16, 1024);
-#pragma unroll
-            for (int k = 0; k < kBK / 16; ++k)
-              umma_bf16(d, ad + 2u * k, bd + 2u * k, kIdesc, (kb | k) != 0 ? 1u : 0u);
-            umma_commit(smem_u32(&empty_bar[st]));
-            ++it;
+            issue(st0, kb != 0 ? 1u : 0u);
+            if (two) {
+              issue(st, 1u);
+              if (++st == kStages) {
+                st = 0;
+                ph ^= 1u;
+              }
+            }
           }
           if (!ok) break;
-          umma_commit(smem_u32(&accf_bar[buf]));
+          umma_commit_pair_mc(smem_u32(&accf_bar[buf]), 3);
           ++acc_it;
         }
+        if (ok) u = next_unit(ui + 1);
       }
-      umma_commit(smem_u32(&done_bar));
+      umma_commit_pair_mc(smem_u32(&done_bar), 1);
       mbar_wait_drain(smem_u32(&done_bar), 0, a.err);
+    }
+  } else if (warp == 2 + kEpiWarps) {
+    if (lane == 0 && leader) {
+      const uint32_t unit_peer0 = mapa_shared(smem_u32(&unit_sh[0]), 1);
+      const uint32_t ufull_peer0 = mapa_shared(smem_u32(&ufull_bar[0]), 1);
+      for (uint32_t i = 0;; ++i) {
+        // claimed ahead of the slot: the counter's round trip is over when it frees
+        int u = atomicAdd(a.next_unit, 1);
+        if (u >= n_units) u = -1;
+        const uint32_t s = i % kSlots;
+        if (!mbar_wait_cluster(smem_u32(&uempty_bar[s]), ((i / kSlots) & 1u) ^ 1u, abort_flag, a.err)) break;
+        *reinterpret_cast<volatile int*>(&unit_sh[s]) = u;
+        mbar_arrive(smem_u32(&ufull_bar[s]));
+        st_shared_cluster_u32(unit_peer0 + s * 4, static_cast<uint32_t>(u));
+        mbar_arrive_cluster(ufull_peer0 + s * 8);
+        if (u < 0) break;
+      }
     }
   } else {
     // epilogue: warp w may read TMEM lanes [32 (w % 4), 32 (w % 4) + 32)
     const int q = warp & 3;
-    const int r_in_tile = q * 32 + lane;
+    const int hf = (warp - 2) >> 2;
+    const int r_in_tile = static_cast<int>(rank) * 128 + q * 32 + lane;
+    const uint32_t acce_lead0 = mapa_shared(smem_u32(&acce_bar[0]), 0);
     uint32_t acc_it = 0;
     bool ok = true;
-    for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
-      const int mt = u / S, s = u - mt * S;
-      int vt0, vt1;
+    for (uint32_t ui = 0; ok; ++ui) {
+      int u = -1;
+      if (lane == 0) u = next_unit(ui);
+      u = __shfl_sync(0xffffffffu, u, 0);
+      if (u < 0) break;
+      int mt, s, vt0, vt1;
+      unit_of(u, n_mt, S, mt, s);
       split_range(s, S, a.n_vtiles, vt0, vt1);
-      const int row = mt * kTileM + r_in_tile;
+      const int row = mt * 256 + r_in_tile;
       const bool valid = row < n_rows;
       const int x = valid ? a.tok_p[row] : -1;
       float m = -INFINITY, ssum = 0.f, q2 = 0.f, zxv = 0.f;
       bool found = false;
       for (int vt = vt0; vt < vt1; ++vt) {
-        const uint32_t buf = acc_it & 1u, aph = (acc_it >> 1) & 1u;
-        if (!mbar_wait(smem_u32(&accf_bar[buf]), aph, abort_flag, a.err)) {
-          ok = false;
-          break;
-        }
+        const uint32_t buf = acc_it & 1u;
+        if (!(ok = mbar_wait(smem_u32(&accf_bar[buf]), (acc_it >> 1) & 1u, abort_flag, a.err))) break;
         tc_fence_after();
-        const int col0 = vt * kFwdBN;
-        const int ncols = min(kFwdBN, a.V - col0);
+        const int col0 = vt * 256 + hf * 128;
+        const int ncols = min(128, a.V - col0);   // may be <= 0 in the last tile
         const int lx = x - col0;
-        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * kFwdBN;
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * 256 + hf * 128;
 #pragma unroll 1
-        for (int c0 = 0; c0 < kFwdBN; c0 += 32) {
+        for (int c0 = 0; c0 < 128; c0 += 32) {
           if (c0 >= ncols) break;
           float v[32];
           tmem_ld32(taddr + c0, v);
@@ -261,13 +345,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           else
             fold_partial(v, ncols - c0, m, ssum, q2);
         }
+        // every lane's TMEM reads are complete: one arrival per warp hands it back
         tc_fence_before();
-        mbar_arrive(smem_u32(&acce_bar[buf]));
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster_relaxed(acce_lead0 + buf * 8);
         ++acc_it;
       }
       if (!ok) break;
       if (valid) {
-        a.part[static_cast<int64_t>(s) * a.rows_cap + row] = make_float4(m, ssum, q2 * kLn2, 0.f);
+        a.part[static_cast<int64_t>(2 * s + hf) * a.rows_cap + row] = make_float4(m, ssum, q2 * kLn2, 0.f);
         if (found) a.zx[row] = zxv;
       }
     }
@@ -275,10 +361,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();   // no CTA leaves while the other may still touch its memory
   tc_fence_after();
   if (warp == 1) {
     __syncwarp();
-    tmem_dealloc(tmem_base, 512);
+    tmem_dealloc_pair(tmem_base, 512);
   }
 }
 
@@ -297,7 +384,7 @@ cudaError_t launch_lmhead_fwd(const CUtensorMap& tm_h, const CUtensorMap& tm_w, 
     if (e != cudaSuccess) return e;
     attr_set.fetch_or(bit, std::memory_order_release);
   }
-  lmhead_fwd_kernel<<<grid, kThreads, kSmemBytes, s>>>(tm_h, tm_w, a);
+  lmhead_fwd_kernel<<<grid / 2 * 2, kThreads, kSmemBytes, s>>>(tm_h, tm_w, a);
   return cudaGetLastError();
 }
 

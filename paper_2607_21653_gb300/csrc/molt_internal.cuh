@@ -12,20 +12,21 @@ namespace molt {
 
 constexpr int kTileM = 128;   // token rows per tile (TMEM lanes)
 constexpr int kFwdBN = 256;   // vocab columns per forward MMA tile
+constexpr int kFwdParts = 2;  // partial statistics per row and vocab split (one per column half)
 constexpr int kBwdBV = 256;   // vocab columns per backward unit
 constexpr int kBK = 64;       // K elements per 128-byte swizzled row
 
 // Device pointers into one call's workspace (all regions 256-byte aligned).
 struct Workspace {
   int32_t* counts;      // [0] active rows n, [1] backward tiles, [2] rejected sequences,
-                        // [3] rows with a gradient (the backward's rows)
+                        // [3] rows with a gradient (the backward's rows), [4] the forward's next unit
   int32_t* row_map;     // [T]    packed row -> original row
   int32_t* pos_of_row;  // [T]    original row -> packed row or -1
   int32_t* tok_p;       // [Tcap] packed tokens
   float* b_p;           // [Tcap] packed behaviour log-probs
   float* adv_p;         // [Tcap] packed advantages
   uint16_t* h_p;        // [Tcap, H] packed hidden rows (bf16 bits), rows >= n zeroed
-  float4* part;         // [S, Tcap] per-split (max, sum exp, sum exp*(z-max), -)
+  float4* part;         // [kFwdParts S, Tcap] per-split (max, sum exp, sum exp*(z-max), -)
   float* zx;            // [Tcap] target logit
   float* lse;           // [Tcap]
   float* coef;          // [Tcap] m c / D
@@ -65,7 +66,8 @@ struct FwdArgs {
   int V, H;
   int n_split;
   int n_vtiles;
-  float4* part;
+  int32_t* next_unit;   // zeroed
+  float4* part;         // [kFwdParts n_split, rows_cap]
   float* zx;
   unsigned* err;
 };
@@ -137,6 +139,8 @@ void set_last_error(const std::string& msg);
 void timing_event(int k, bool stop, cudaStream_t s);
 unsigned* device_status_word(molt_status* st);   // current device's status word
 int device_sm_count();                           // current device's SM count
+// vocab splits of the forward pass over Tcap packed rows
+int forward_splits(int64_t Tcap, int64_t H, int64_t V, int n_sm);
 molt_status encode_tmap_2d(CUtensorMap* m, CUtensorMapDataType dt, int elem_bytes, const void* base, uint64_t rows,
                            uint64_t cols, uint32_t box_cols, uint32_t box_rows);
 
@@ -153,7 +157,7 @@ cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, cuda
 // tok_shift is subtracted from every token (a vocabulary shard's first column)
 cudaError_t launch_gather(const uint16_t* hidden, const int32_t* tokens, const float* b, const float* adv, int T,
                           int Tcap, int H, const Workspace& ws, int n_sm, cudaStream_t s, int tok_shift = 0);
-cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_split, double denom, float clip_lo, float clip_hi,
+cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
                          const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, unsigned* err,
                          cudaStream_t s);
 cudaError_t launch_finalize(int Tcap, double denom, bool with_ecoef, const Workspace& ws, float* loss_out,
@@ -161,7 +165,7 @@ cudaError_t launch_finalize(int Tcap, double denom, bool with_ecoef, const Works
 // the rows with a gradient (finalize's list) packed into whole tiles for the backward
 cudaError_t launch_live_gather(int H, bool with_ecoef, const Workspace& ws, int n_sm, cudaStream_t s);
 // extended objective: packed stats -> sequence gate -> loss rows
-cudaError_t launch_merge_stats_ex(int Tcap, int V, int n_split, const Workspace& ws, float* logp_out, float* ent_out,
+cudaError_t launch_merge_stats_ex(int Tcap, int V, int n_parts, const Workspace& ws, float* logp_out, float* ent_out,
                                   unsigned* err, cudaStream_t s);
 cudaError_t launch_seq_gate(int T, int Tcap, const LossEx& ex, const Workspace& ws, unsigned* err, cudaStream_t s);
 cudaError_t launch_loss_rows_ex(int Tcap, double denom, float clip_lo, float clip_hi, const LossEx& ex,
@@ -172,7 +176,7 @@ cudaError_t launch_cast_dh(const Workspace& ws, int T, int H, uint16_t* dh_out, 
 // forward's split partials; the merge of all shards' statistics with the Eq. 2
 // terms; the rows of a shard's backward (coef != 0) and their packing; the
 // shard's dhidden contribution in the original order (fp32)
-cudaError_t launch_vp_local(int T, int Tcap, int V_s, int n_split, const Workspace& ws, float4* out, cudaStream_t s);
+cudaError_t launch_vp_local(int T, int Tcap, int V_s, int n_parts, const Workspace& ws, float4* out, cudaStream_t s);
 cudaError_t launch_vp_merge(int T, int Tcap, int n_shards, double denom, float clip_lo, float clip_hi,
                             const float4* parts, const float* b, const float* adv, const Workspace& ws,
                             float* lse_out, float* coef_out, float* logp_out, float* ent_out, float* tokloss_out,
@@ -183,6 +187,7 @@ cudaError_t launch_vp_gather(const uint16_t* hidden, const int32_t* tokens, cons
 cudaError_t launch_vp_dh_out(const Workspace& ws, int T, int H, float* out, int n_sm, cudaStream_t s);
 
 // lmhead_fwd.cu
+// (boxes of 128 rows x kBK columns of the packed hidden rows and of W)
 cudaError_t launch_lmhead_fwd(const CUtensorMap& tm_h, const CUtensorMap& tm_w, const FwdArgs& a, int grid,
                               cudaStream_t s);
 // lmhead_bwd4.cu (clusters of two CTA pairs; H % 128 == 0)

@@ -10,8 +10,10 @@
 // and passes every input and output; the call allocates nothing.
 //
 // Differences from molt_token_logprobs_fwd: no active-row compaction (masked
-// rows are computed and then written as 0), at most kNoAllocMaxSplits vocab
-// splits, and T <= kNoAllocMaxRows.  The same forward kernel does the work.
+// rows are computed and then written as 0), as many vocab splits as the array's
+// kNoAllocParts partial statistics per row of the largest batch leave room for,
+// and T <= kNoAllocMaxRows.  The same forward kernel does the work.
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 #include <string>
@@ -20,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/molt.h"
+#include "merge.cuh"
 #include "molt_internal.cuh"
 #include "ptx.cuh"
 
@@ -27,13 +30,11 @@ namespace molt {
 namespace {
 
 constexpr int kNoAllocMaxRows = MOLT_NOALLOC_MAX_TOKENS;
-constexpr int kNoAllocMaxSplits = 8;
+constexpr int kNoAllocParts = 8;   // at kNoAllocMaxRows rows; smaller batches have room for more
 constexpr size_t kCountsBytes = 256;
-constexpr size_t kPartBytes = static_cast<size_t>(kNoAllocMaxSplits) * kNoAllocMaxRows * sizeof(float4);
+constexpr size_t kPartBytes = static_cast<size_t>(kNoAllocParts) * kNoAllocMaxRows * sizeof(float4);
 constexpr size_t kZxBytes = static_cast<size_t>(kNoAllocMaxRows) * sizeof(float);
 constexpr size_t kScratchBytes = kCountsBytes + kPartBytes + kZxBytes;   // ~4.1 MB
-
-constexpr float kLog2e = 1.4426950408889634f;
 
 }  // namespace
 }  // namespace molt
@@ -59,40 +60,32 @@ __global__ void noalloc_init_kernel(int T, int32_t* counts, float* zx) {
   if (t == 0) {
     counts[0] = T;
     counts[1] = 0;
+    counts[4] = 0;
   }
   if (t < T) zx[t] = 0.f;
 }
 
 // merge the per-split partials of each row into logp and entropy; masked rows
 // are written as 0, active rows with an out-of-range token raise the status flag
-__global__ void noalloc_merge_kernel(int T, int V, int S, int rows_cap, const int32_t* __restrict__ tokens,
-                                     const uint8_t* __restrict__ mask, const float4* __restrict__ part,
-                                     const float* __restrict__ zx, float* __restrict__ logp_out,
-                                     float* __restrict__ ent_out, unsigned* err) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  if (mask != nullptr && mask[t] == 0) {
+__global__ void __launch_bounds__(kMergeThreads)
+    noalloc_merge_kernel(int T, int V, int n_parts, int rows_cap, const int32_t* __restrict__ tokens,
+                         const uint8_t* __restrict__ mask, const float4* __restrict__ part,
+                         const float* __restrict__ zx, float* __restrict__ logp_out, float* __restrict__ ent_out,
+                         unsigned* err) {
+  const int t = blockIdx.x * kTileM + threadIdx.x % kTileM;
+  const bool act = t < T && (mask == nullptr || mask[t] != 0);
+  const RowStats st = merge_row_parts(part, rows_cap, n_parts, t, act);
+  if (threadIdx.x >= kTileM || t >= T) return;
+  if (!act) {
     logp_out[t] = 0.f;
     if (ent_out) ent_out[t] = 0.f;
     return;
   }
-  float M = -INFINITY;
-  for (int s = 0; s < S; ++s) M = fmaxf(M, part[static_cast<int64_t>(s) * rows_cap + t].x);
-  float Ssum = 0.f, Q = 0.f;
-  for (int s = 0; s < S; ++s) {
-    const float4 p = part[static_cast<int64_t>(s) * rows_cap + t];
-    if (p.y > 0.f) {
-      const float d = p.x - M;
-      const float f = ex2_approx(d * kLog2e);
-      Ssum += f * p.y;
-      Q += f * (p.z + d * p.y);
-    }
-  }
   const int x = tokens[t];
   if (x < 0 || x >= V) atomicOr(err, kDevErrTokenRange);
-  const float logS = logf(Ssum);
-  logp_out[t] = zx[t] - (M + logS);
-  if (ent_out) ent_out[t] = logS - Q / Ssum;
+  const float logS = logf(st.S);
+  logp_out[t] = zx[t] - (st.M + logS);
+  if (ent_out) ent_out[t] = logS - st.Q / st.S;
 }
 
 molt_status noalloc_fail(molt_status s, const std::string& msg) {
@@ -153,18 +146,18 @@ extern "C" molt_status molt_token_logprobs_fwd_noalloc(const uint16_t* hidden, c
 
   const int64_t Tcap = ((T + kTileM - 1) / kTileM) * kTileM;
   const int n_vt = static_cast<int>((V + kFwdBN - 1) / kFwdBN);
-  int S = static_cast<int>((16 * static_cast<int64_t>(n_sm) * kTileM + Tcap - 1) / Tcap);
-  if (S < 1) S = 1;
-  if (S > kNoAllocMaxSplits) S = kNoAllocMaxSplits;
-  if (S > n_vt) S = n_vt;
+  // as far as the partials fit
+  const int64_t S = std::max<int64_t>(
+      1, std::min<int64_t>(forward_splits(Tcap, H, V, n_sm),
+                           static_cast<int64_t>(kNoAllocParts) * kNoAllocMaxRows / (kFwdParts * Tcap)));
 
   int32_t* counts = reinterpret_cast<int32_t*>(scratch);
   float4* part = reinterpret_cast<float4*>(scratch + kCountsBytes);
   float* zx = reinterpret_cast<float*>(scratch + kCountsBytes + kPartBytes);
 
   CUtensorMap tm_h, tm_w;
-  MOLT_TRY_STATUS(encode_tmap_2d(&tm_h, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hidden, T, H, kBK, kTileM));
-  MOLT_TRY_STATUS(encode_tmap_2d(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, V, H, kBK, kFwdBN));
+  MOLT_TRY_STATUS(encode_tmap_2d(&tm_h, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hidden, T, H, kBK, 128));
+  MOLT_TRY_STATUS(encode_tmap_2d(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, V, H, kBK, 128));
 
   noalloc_init_kernel<<<static_cast<int>((T + 255) / 256), 256, 0, stream>>>(static_cast<int>(T), counts, zx);
   if ((e = cudaGetLastError()) != cudaSuccess) return noalloc_fail(MOLT_ERR_CUDA, cudaGetErrorString(e));
@@ -175,8 +168,9 @@ extern "C" molt_status molt_token_logprobs_fwd_noalloc(const uint16_t* hidden, c
   fa.rows_cap = static_cast<int>(Tcap);
   fa.V = static_cast<int>(V);
   fa.H = static_cast<int>(H);
-  fa.n_split = S;
+  fa.n_split = static_cast<int>(S);
   fa.n_vtiles = n_vt;
+  fa.next_unit = counts + 4;
   fa.part = part;
   fa.zx = zx;
   fa.err = status_word;
@@ -186,8 +180,8 @@ extern "C" molt_status molt_token_logprobs_fwd_noalloc(const uint16_t* hidden, c
   note_launches(1);
   timing_event(1, true, stream);
   timing_event(2, false, stream);
-  noalloc_merge_kernel<<<static_cast<int>((T + 127) / 128), 128, 0, stream>>>(
-      static_cast<int>(T), static_cast<int>(V), S, static_cast<int>(Tcap), tokens, mask, part, zx, logp_out,
+  noalloc_merge_kernel<<<static_cast<int>((T + kTileM - 1) / kTileM), kMergeThreads, 0, stream>>>(
+      static_cast<int>(T), static_cast<int>(V), static_cast<int>(kFwdParts * S), static_cast<int>(Tcap), tokens, mask, part, zx, logp_out,
       entropy_out, status_word);
   if ((e = cudaGetLastError()) != cudaSuccess) return noalloc_fail(MOLT_ERR_CUDA, cudaGetErrorString(e));
   note_launches(1);

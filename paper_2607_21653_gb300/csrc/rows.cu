@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "merge.cuh"
 #include "molt_internal.cuh"
 #include "ptx.cuh"
 
@@ -194,6 +195,7 @@ __global__ void __launch_bounds__(1024) compact_kernel(const uint8_t* __restrict
     counts[0] = total;
     counts[1] = 0;
     counts[2] = 0;
+    counts[4] = 0;
   }
 }
 
@@ -229,24 +231,27 @@ __global__ void gather_kernel(const uint16_t* __restrict__ hidden, const int32_t
   }
 }
 
-// deterministic 128-thread block sum (fixed tree)
+// barrier of a block's first 128 threads
+__device__ __forceinline__ void sync128() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// deterministic sum over a block's first 128 threads (fixed tree)
 template <typename T>
 __device__ T block128_sum(T v, T* sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
+  sync128();
   T r = (sh[0] + sh[1]) + (sh[2] + sh[3]);
-  __syncthreads();
+  sync128();
   return r;
 }
 __device__ double block128_max(double v, double* sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
+  sync128();
   double r = fmax(fmax(sh[0], sh[1]), fmax(sh[2], sh[3]));
-  __syncthreads();
+  sync128();
   return r;
 }
 
@@ -274,13 +279,12 @@ __device__ __forceinline__ RowLoss surrogate_row(float logp, float b, float A, f
 }
 
 // the tile's fixed-tree partial sums (loss, ratio, entropy, max |log ratio|,
-// clip counts) and its activity flag; every thread of the 128-thread block
-// calls it
+// clip counts) and its activity flag; a block's first 128 threads call it
 __device__ void tile_partials(bool act, const RowLoss& rl, float ent, double* __restrict__ red,
                               int32_t* __restrict__ tile_flag) {
   __shared__ double shd[4];
   __shared__ long long shl[4];
-  const int any = __syncthreads_or(act && rl.coef != 0.f);
+  const long long any = block128_sum<long long>(act && rl.coef != 0.f ? 1 : 0, shl);
   double* r = red + (int64_t)blockIdx.x * kRedSlots;
   const double s_loss = block128_sum<double>(act ? (double)rl.tl : 0.0, shd);
   const double s_ratio = block128_sum<double>(act ? (double)rl.ratio : 0.0, shd);
@@ -301,12 +305,13 @@ __device__ void tile_partials(bool act, const RowLoss& rl, float ent, double* __
   }
 }
 
-// One block of 128 threads per packed tile: merge the per-split online
-// softmax partials of each row into lse, logp and entropy; in loss mode also
+// One block per packed tile of 128 rows (merge_row_parts' threads): merge the
+// per-split online softmax partials of each row into lse, logp and entropy; in
+// loss mode the first 128 threads also form
 // the ratio, the clipped surrogate (Sec. 4.5, PPO form), the Eq. 2 coefficient
 // m c / D, per-tile partial sums and the tile's activity flag.
-__global__ void __launch_bounds__(128) merge_kernel(
-    int loss_mode, int Tcap, int V, int n_split, double denom, float clip_lo, float clip_hi,
+__global__ void __launch_bounds__(kMergeThreads) merge_kernel(
+    int loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
     const int32_t* __restrict__ counts, const int32_t* __restrict__ row_map, const int32_t* __restrict__ tok_p,
     const float* __restrict__ b_p, const float* __restrict__ adv_p, const float4* __restrict__ part,
     const float* __restrict__ zx, float* __restrict__ lse_o, float* __restrict__ coef_o,
@@ -316,30 +321,20 @@ __global__ void __launch_bounds__(128) merge_kernel(
   const int n = counts[0];
   const int n_tiles = (n + kTileM - 1) / kTileM;
   if ((int)blockIdx.x >= n_tiles) return;
-  const int k = blockIdx.x * kTileM + threadIdx.x;
+  const int k = blockIdx.x * kTileM + threadIdx.x % kTileM;
   const bool act = k < n;
+  const RowStats st = merge_row_parts(part, Tcap, n_parts, k, act);
+  if (threadIdx.x >= kTileM) return;
   const double D = denom > 0.0 ? denom : static_cast<double>(n);
   float logp = 0.f, ent = 0.f;
   RowLoss rl{0.f, 0.f, 0.f, 0, 0, 0.0};
   if (act) {
-    float M = -INFINITY;
-    for (int s = 0; s < n_split; ++s) M = fmaxf(M, part[(int64_t)s * Tcap + k].x);
-    float S = 0.f, Q = 0.f;
-    for (int s = 0; s < n_split; ++s) {
-      const float4 p = part[(int64_t)s * Tcap + k];
-      if (p.y > 0.f) {
-        const float d = p.x - M;
-        const float f = ex2_approx(d * kLog2e);
-        S += f * p.y;
-        Q += f * (p.z + d * p.y);
-      }
-    }
-    const float logS = logf(S);
-    const float lse = M + logS;
+    const float logS = logf(st.S);
+    const float lse = st.M + logS;
     const int x = tok_p[k];
     if (x < 0 || x >= V) atomicOr(err, kDevErrTokenRange);
     logp = zx[k] - lse;
-    ent = logS - Q / S;
+    ent = logS - st.Q / st.S;
     lse_o[k] = lse;
     if (loss_mode) rl = surrogate_row(logp, b_p[k], adv_p[k], clip_lo, clip_hi, D);
     const int t = row_map[k];
@@ -366,30 +361,19 @@ __global__ void __launch_bounds__(128) merge_kernel(
 // sum exp(z - M), Q = sum exp(z - M) (z - M), z_x the target logit if the
 // target lies in the shard (tok_p holds the shard-local token) and -inf
 // otherwise.  Masked rows get the empty statistics (-inf, 0, 0, -inf).
-__global__ void vp_local_kernel(int T, int Tcap, int V_s, int n_split, const int32_t* __restrict__ pos,
-                                const int32_t* __restrict__ tok_p, const float4* __restrict__ part,
-                                const float* __restrict__ zx, float4* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  const int k = pos[t];
+__global__ void __launch_bounds__(kMergeThreads) vp_local_kernel(
+    int T, int Tcap, int V_s, int n_parts, const int32_t* __restrict__ pos, const int32_t* __restrict__ tok_p,
+    const float4* __restrict__ part, const float* __restrict__ zx, float4* __restrict__ out) {
+  const int t = blockIdx.x * kTileM + threadIdx.x % kTileM;
+  const int k = t < T ? pos[t] : -1;
+  const RowStats st = merge_row_parts(part, Tcap, n_parts, k, k >= 0);
+  if (threadIdx.x >= kTileM || t >= T) return;
   if (k < 0) {
     out[t] = make_float4(-INFINITY, 0.f, 0.f, -INFINITY);
     return;
   }
-  float M = -INFINITY;
-  for (int s = 0; s < n_split; ++s) M = fmaxf(M, part[(int64_t)s * Tcap + k].x);
-  float S = 0.f, Q = 0.f;
-  for (int s = 0; s < n_split; ++s) {
-    const float4 p = part[(int64_t)s * Tcap + k];
-    if (p.y > 0.f) {
-      const float d = p.x - M;
-      const float f = ex2_approx(d * kLog2e);
-      S += f * p.y;
-      Q += f * (p.z + d * p.y);
-    }
-  }
   const int xl = tok_p[k];
-  out[t] = make_float4(M, S, Q, (xl >= 0 && xl < V_s) ? zx[k] : -INFINITY);
+  out[t] = make_float4(st.M, st.S, st.Q, (xl >= 0 && xl < V_s) ? zx[k] : -INFINITY);
 }
 
 // One block of 128 threads per packed tile of active rows: merge the shards'
@@ -600,7 +584,7 @@ __global__ void __launch_bounds__(128) loss_rows_ex_kernel(
     ecoef_o[k] = ecoef;
     mu_o[k] = mu;
   }
-  const int any = __syncthreads_or(coef != 0.f || ecoef != 0.f);
+  const long long any = block128_sum<long long>(coef != 0.f || ecoef != 0.f ? 1 : 0, shl);
   double* rr = red + (int64_t)blockIdx.x * kRedSlots;
   const double s_loss = block128_sum<double>(act ? (double)tl : 0.0, shd);
   const double s_ratio = block128_sum<double>(act ? (double)ratio : 0.0, shd);
@@ -873,22 +857,22 @@ cudaError_t launch_gather(const uint16_t* hidden, const int32_t* tokens, const f
   return cudaGetLastError();
 }
 
-cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_split, double denom, float clip_lo, float clip_hi,
+cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
                          const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, unsigned* err,
                          cudaStream_t s) {
   const int blocks = Tcap / kTileM;
-  merge_kernel<<<blocks, kTileM, 0, s>>>(loss_mode ? 1 : 0, Tcap, V, n_split, denom, clip_lo, clip_hi, ws.counts,
+  merge_kernel<<<blocks, kMergeThreads, 0, s>>>(loss_mode ? 1 : 0, Tcap, V, n_parts, denom, clip_lo, clip_hi, ws.counts,
                                           ws.row_map, ws.tok_p, ws.b_p, ws.adv_p, ws.part, ws.zx, ws.lse, ws.coef,
                                           ws.tile_flag, ws.red, logp_out, ent_out, tokloss_out, nullptr, nullptr,
                                           err);
   return cudaGetLastError();
 }
 
-cudaError_t launch_merge_stats_ex(int Tcap, int V, int n_split, const Workspace& ws, float* logp_out, float* ent_out,
+cudaError_t launch_merge_stats_ex(int Tcap, int V, int n_parts, const Workspace& ws, float* logp_out, float* ent_out,
                                   unsigned* err, cudaStream_t s) {
   const int blocks = Tcap / kTileM;
   if (blocks == 0) return cudaSuccess;
-  merge_kernel<<<blocks, kTileM, 0, s>>>(0, Tcap, V, n_split, 0.0, 0.f, 0.f, ws.counts, ws.row_map, ws.tok_p, ws.b_p,
+  merge_kernel<<<blocks, kMergeThreads, 0, s>>>(0, Tcap, V, n_parts, 0.0, 0.f, 0.f, ws.counts, ws.row_map, ws.tok_p, ws.b_p,
                                           ws.adv_p, ws.part, ws.zx, ws.lse, ws.coef, ws.tile_flag, ws.red, logp_out,
                                           ent_out, nullptr, ws.lp_p, ws.ent_p, err);
   return cudaGetLastError();
@@ -930,10 +914,10 @@ cudaError_t launch_live_gather(int H, bool with_ecoef, const Workspace& ws, int 
   return cudaGetLastError();
 }
 
-cudaError_t launch_vp_local(int T, int Tcap, int V_s, int n_split, const Workspace& ws, float4* out,
+cudaError_t launch_vp_local(int T, int Tcap, int V_s, int n_parts, const Workspace& ws, float4* out,
                             cudaStream_t s) {
   if (T <= 0) return cudaSuccess;
-  vp_local_kernel<<<(T + 255) / 256, 256, 0, s>>>(T, Tcap, V_s, n_split, ws.pos_of_row, ws.tok_p, ws.part, ws.zx,
+  vp_local_kernel<<<(T + kTileM - 1) / kTileM, kMergeThreads, 0, s>>>(T, Tcap, V_s, n_parts, ws.pos_of_row, ws.tok_p, ws.part, ws.zx,
                                                    out);
   return cudaGetLastError();
 }

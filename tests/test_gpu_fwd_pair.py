@@ -1,0 +1,44 @@
+"""The forward on CTA pairs and the merge of its partials where they can go wrong:
+one row and one column, an empty second half of a tile (rows or vocab columns),
+remainders around 128 and 256 in both, more than one group of 16 token tiles, one
+K block, and a few rows against many vocab splits (hundreds of partials a row)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2607_21653_gb300 as molt  # noqa: E402
+from oracle import molt_oracle as O  # noqa: E402
+from workloads import random_problem  # noqa: E402
+
+from parity import LOGP_ATOL, bf, np_, t  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    molt.build()
+    molt.load()
+
+
+@pytest.mark.parametrize("T,H,V", [(1, 64, 1), (128, 128, 128), (129, 64, 129), (257, 192, 385), (300, 320, 1000),
+                                   (4353, 128, 700), (40, 256, 40001)])
+@pytest.mark.parametrize("call", ["token_logprobs", "token_logprobs_noalloc"])
+def test_forward_matches_oracle(T, H, V, call):
+    rng = np.random.default_rng(T + H + V)
+    h, W, x, m = random_problem(rng, T, H, V, mask_frac=0.3 if T > 1 else 0.0, w_std=0.05)
+    m[-1] = 1
+    x[-1] = V - 1
+    lp, ent = O.token_logprobs(O.widen_bf16(h), O.widen_bf16(W), x, m)
+    a, e = getattr(molt, call)(bf(h), bf(W), t(x), t(m))
+    torch.cuda.synchronize()
+    assert molt.device_status() == 0
+    # products of bf16 are exact in fp32, sums of H of them and of V exponentials
+    # are off by at most a few times (H + V / 256) 2^-24 of terms of order 10
+    bound = min(LOGP_ATOL, 40 * (H + V / 256 + 64) * 2.0 ** -24)
+    assert np.abs(np_(a) - lp).max() <= bound
+    assert np.abs(np_(e) - ent).max() <= bound
+    assert (np_(a)[m == 0] == 0).all() and (np_(e)[m == 0] == 0).all()
