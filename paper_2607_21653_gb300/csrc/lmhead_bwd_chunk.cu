@@ -40,15 +40,22 @@
 // tile's epilogue runs under the next tile's products.
 //
 // What bounds it, measured on T = 16384, H = 4096, V = 151936 (61.2 TFLOP in
-// three products): 38.0 ms, 1.61 PFLOP/s, at the board's power cap (1.5 GHz of
-// 2.07, 1370 W), where a cuBLAS 8192^3 product reaches 1.72 at the same clock; the
-// cluster kernel takes 54.4-57.3 ms.  A tile of 64 K blocks takes 36.0K clocks of
+// three products): 36.8 ms, 1.66 PFLOP/s, at the board's power cap (1.49 GHz of
+// 2.07, 1375 W), where a cuBLAS 8192^3 product reaches 1.72 at the same clock; the
+// cluster kernel takes 54.4-57.3 ms.  A tile of 64 K blocks takes 35.2K clocks of
 // 32.8K ideal.  Issue decides what is left of the clock: one thread that waits for
 // one stage at a time, with address arithmetic between the products, kept the
 // tensor pipe at 67 % even with all loads left out, two stages per turn with the
-// four products of each in one statement at 96 %; and one producer thread with
-// four 8 KB boxes per stage needed 830 clocks per K block of 512.
+// four products of each in one statement at 96 %; one producer thread with four
+// 8 KB boxes per stage needed 830 clocks per K block of 512; and tiles decoded by
+// the claiming warp, instead of by every role from their index, took 1 to 2K
+// clocks off each.  A tile of few K blocks (short H) is bound by its epilogue,
+// which converts without the target's and the edge's selects wherever the warp has
+// neither and signals a Z tile's stores one tile later (T = 4000, H = 320, V =
+// 50257: 0.51 ms, before these three 0.57; T = 3000, H = 1024, V = 32000: 0.355,
+// before 0.399).
 #include <atomic>
+#include <climits>
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -72,26 +79,34 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 enum TileKind : int { kTileZ = 0, kTileDH = 1, kTileDW = 2 };
 
-// What one claimed tile is.  All counts are in 256-row / 256-column tiles.
-struct Tile {
-  int kind;
+// What one claimed tile is, as the claiming warp hands it to the other roles.
+// t, v, h, t0 and v0 count 256-row / 256-column tiles.
+struct __align__(16) Tile {
+  int kind;      // TileKind, or -1 at the end of the walk
   int chunk;     // in list order
   int buf;       // chunk buffer
-  int tc, vc;    // its token and vocab chunk
+  int nk;        // K blocks
   int t, v, h;   // global tile indices (those the kind uses)
+  int order;     // dH: the vocab chunk, dW: the token chunk
   int t0, v0;    // the chunk's first token and vocab tile
-  int ct, cv;    // the chunk's tiles
+  int need;      // dH, dW: warps that store the chunk's g; Z: tiles that read the
+                 // buffer's previous chunk (0: none)
+  int pad;
 };
 
-// The tile list, walked forwards: claimed indices only grow.
+// The tile list, walked forwards by the claiming thread: claimed indices only grow.
 struct TileList {
+  int n_rows, V, H;
   int n_t, n_v, n_h, n_tc, n_vc, n_chunks, nb;
   int total;                             // tiles in the list
   int step, base;                        // list step and its first index
   int n_dh, n_z, n_dw;                   // tiles of the step
   int c_t0, c_ct, c_v0, c_cv;            // chunk step - L
   int z_t0, z_ct, z_v0, z_cv;            // chunk step
-  __device__ __forceinline__ void init(const ChunkArgs& a, int n_rows) {
+  __device__ __forceinline__ void init(const ChunkArgs& a, int rows) {
+    n_rows = rows;
+    V = a.V;
+    H = a.H;
     n_t = (n_rows + 255) / 256;
     n_v = (a.V + 255) / 256;
     n_h = (a.H + 255) / 256;
@@ -135,39 +150,44 @@ struct TileList {
       fill();
     }
     int i = j - base;
-    if (i >= n_dh && i < n_dh + n_z) {
+    const bool z = i >= n_dh && i < n_dh + n_z;
+    x.chunk = z ? step : step - (nb - 1);
+    const int tc = x.chunk / n_vc, vc = x.chunk - tc * n_vc;
+    x.buf = x.chunk % nb;
+    x.t0 = z ? z_t0 : c_t0;
+    x.v0 = z ? z_v0 : c_v0;
+    x.t = x.t0;
+    x.v = x.v0;
+    x.h = 0;
+    x.order = 0;
+    uint32_t nz, nr;
+    if (z) {
       i -= n_dh;
       x.kind = kTileZ;
-      x.chunk = step;
-      x.t0 = z_t0;
-      x.ct = z_ct;
-      x.v0 = z_v0;
-      x.cv = z_cv;
-      x.v = z_v0 + i / z_ct;
-      x.t = z_t0 + i % z_ct;
-      x.h = 0;
-    } else {
-      x.chunk = step - (nb - 1);
-      x.t0 = c_t0;
-      x.ct = c_ct;
-      x.v0 = c_v0;
-      x.cv = c_cv;
-      if (i < n_dh) {
-        x.kind = kTileDH;
-        x.h = i / c_ct;
-        x.t = c_t0 + i % c_ct;
-        x.v = c_v0;
-      } else {
-        i -= n_dh + n_z;
-        x.kind = kTileDW;
-        x.h = i / c_cv;
-        x.v = c_v0 + i % c_cv;
-        x.t = c_t0;
-      }
+      x.nk = H / kBK;
+      x.v += i / z_ct;
+      x.t += i % z_ct;
+      nr = 0;
+      if (x.chunk >= nb) chunk_counts(x.chunk - nb, nz, nr);
+      x.need = static_cast<int>(nr);
+      return;
     }
-    x.tc = x.chunk / n_vc;
-    x.vc = x.chunk - x.tc * n_vc;
-    x.buf = x.chunk % nb;
+    chunk_counts(x.chunk, nz, nr);
+    x.need = static_cast<int>(nz) * (2 * kEpiWarps);
+    if (i < n_dh) {
+      x.kind = kTileDH;
+      x.order = vc;
+      x.nk = (min(V, (c_v0 + c_cv) * 256) - c_v0 * 256 + kBK - 1) / kBK;
+      x.h = i / c_ct;
+      x.t += i % c_ct;
+    } else {
+      i -= n_dh + n_z;
+      x.kind = kTileDW;
+      x.order = tc;
+      x.nk = (min(n_rows, (c_t0 + c_ct) * 256) - c_t0 * 256 + kBK - 1) / kBK;   // 0 without rows
+      x.h = i / c_cv;
+      x.v += i % c_cv;
+    }
   }
   // tiles of chunk c that write (z) or read its buffer
   __device__ __forceinline__ void chunk_counts(int c, uint32_t& z, uint32_t& rd) const {
@@ -196,10 +216,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) uint64_t empty_bar[kStages];   // both CTAs
   __shared__ __align__(8) uint64_t accf_bar[2];          // both CTAs: accumulator full
   __shared__ __align__(8) uint64_t acce_bar[2];          // even CTA: one arrival per epilogue warp of the pair
-  __shared__ __align__(8) uint64_t jfull_bar[kSlots];    // both CTAs: tile index written
+  __shared__ __align__(8) uint64_t jfull_bar[kSlots];    // both CTAs: tile written
   __shared__ __align__(8) uint64_t jempty_bar[kSlots];   // even CTA: every reader of both CTAs has it
   __shared__ __align__(8) uint64_t done_bar;
-  __shared__ int job_sh[kSlots];
+  __shared__ Tile tile_sh[kSlots];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
 
@@ -240,29 +260,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
   const int n_rows = a.counts[3];
   const int H = a.H, V = a.V;
-  TileList list;
-  list.init(a, n_rows);
   // columns of H that tile h covers: 256, less in the last one
   auto tile_w = [&](int h) -> int { return min(256, H - h * 256); };
   // N of its products: each CTA brings one or two whole 64-column boxes, zero past H
   auto mma_n = [&](int h) -> int { return H - h * 256 > 128 ? 256 : 128; };
-  auto k_blocks = [&](const Tile& x) -> int {
-    if (x.kind == kTileZ) return H / kBK;
-    if (x.kind == kTileDH) return (min(V, (x.v0 + x.cv) * 256) - x.v0 * 256 + kBK - 1) / kBK;
-    return (min(n_rows, (x.t0 + x.ct) * 256) - x.t0 * 256 + kBK - 1) / kBK;   // 0 without rows
-  };
   uint32_t* zdone = a.ctl + kChunkCtlHead;
   uint32_t* cdone = zdone + a.max_chunks;
 
-  // the next tile index for a reader of the slot ring (called by one lane);
-  // -1 ends the walk, also after a wait that ran out
+  // the i-th tile for a reader of the slot ring; false at the end of the walk, also
+  // after a wait that ran out.  Single threads give the slot back here, a warp's
+  // lane 0 for all of them (the condition always holds: it puts the arrival after
+  // the reads).
   const uint32_t jempty_lead0 = mapa_shared(smem_u32(&jempty_bar[0]), 0);
-  auto next_job = [&](uint32_t i) -> int {
+  auto next_tile = [&](uint32_t i, Tile& x, bool whole_warp = false) -> bool {
     const uint32_t s = i % kSlots;
-    if (!mbar_wait_cluster(smem_u32(&jfull_bar[s]), (i / kSlots) & 1u, abort_flag, a.err)) return -1;
-    const int j = *reinterpret_cast<volatile int*>(&job_sh[s]);
-    if (j >= -1) mbar_arrive_cluster_relaxed(jempty_lead0 + s * 8);   // always; orders the arrival after the read
-    return j;
+    // CTA scope in both CTAs: the odd one's copy arrives as bytes of the barrier (a
+    // cluster-scope acquire here cost about 1000 clocks between two tiles)
+    if (!mbar_wait(smem_u32(&jfull_bar[s]), (i / kSlots) & 1u, abort_flag, a.err)) return false;
+    const uint32_t src = smem_u32(&tile_sh[s]);
+    int4 q[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q[k] = ld_shared_v4(src + 16 * k);
+    if (whole_warp) __syncwarp();
+    if ((!whole_warp || lane == 0) && (q[0].x & q[1].x & q[2].x) != INT_MIN)
+      mbar_arrive_cluster_relaxed(jempty_lead0 + s * 8);
+    x.kind = q[0].x;
+    x.chunk = q[0].y;
+    x.buf = q[0].z;
+    x.nk = q[0].w;
+    x.t = q[1].x;
+    x.v = q[1].y;
+    x.h = q[1].z;
+    x.order = q[1].w;
+    x.t0 = q[2].x;
+    x.v0 = q[2].y;
+    x.need = q[2].z;
+    return x.kind >= 0;
   };
 
   if (warp == 0) {
@@ -276,14 +309,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       int ready = -1;   // last chunk seen whole: both kinds of tiles that read it come in runs
       bool ok = true;
       Tile x;
-      int job = next_job(0);
-      for (uint32_t ji = 0; job >= 0; ++ji) {
-        list.seek(job, x);
-        const int nk = k_blocks(x);
+      for (uint32_t ji = 0; ok && next_tile(ji, x); ++ji) {
+        const int nk = x.nk;
         if (x.kind != kTileZ && x.chunk != ready) {
-          uint32_t nz, nr;
-          list.chunk_counts(x.chunk, nz, nr);
-          if (!turn_wait(zdone + x.chunk, nz * (2 * kEpiWarps), abort_flag, a.ctl + 1, a.err)) break;
+          if (!turn_wait(zdone + x.chunk, static_cast<uint32_t>(x.need), abort_flag, a.ctl + 1, a.err)) break;
           fence_proxy_async_global();
           ready = x.chunk;
         }
@@ -294,6 +323,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (!(ok = mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1u, abort_flag, a.err))) break;
           const uint32_t sa = smem0 + st * kStageBytes, fb = full_lead0 + st * 8;
           if (leader) mbar_arrive_expect_tx(smem_u32(&full_bar[st]), 2 * kStageBytes);
+          ++n_it;
           if (x.kind == kTileZ)
             tma_load_2d_pair(sa, &m.h128, fb, kb * kBK, trow);
           else if (x.kind == kTileDH)
@@ -305,9 +335,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             ph ^= 1u;
           }
         }
-        if (!ok) break;
-        n_it += nk;
-        job = next_job(ji + 1);
       }
       if (leader) {
         // every copy into both CTAs completes on these barriers: wait for the
@@ -327,10 +354,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       uint32_t st = 0, ph = 0;
       bool ok = true;
       Tile x;
-      int job = next_job(0);
-      for (uint32_t ji = 0; job >= 0; ++ji) {
-        list.seek(job, x);
-        const int nk = k_blocks(x);
+      for (uint32_t ji = 0; ok && next_tile(ji, x); ++ji) {
+        const int nk = x.nk;
         const bool z = x.kind == kTileZ;
         const CUtensorMap* map = x.kind == kTileDH ? &m.w64x2 : &m.h64x2;
         const int vrow = x.v * 256 + static_cast<int>(rank) * 128;
@@ -348,19 +373,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             ph ^= 1u;
           }
         }
-        if (!ok) break;
-        job = next_job(ji + 1);
       }
     }
   } else if (warp == 1) {
     if (lane == 0 && leader) {
-      uint32_t st = 0, ph = 0, ji = 0;
+      uint32_t st = 0, ph = 0;
       bool ok = true;
       Tile x;
-      int job = next_job(0);
-      for (; job >= 0; ++ji) {
-        list.seek(job, x);
-        const int nk = k_blocks(x);
+      for (uint32_t ji = 0; next_tile(ji, x); ++ji) {
+        const int nk = x.nk;
         const uint32_t buf = ji & 1u;
         if (!mbar_wait(smem_u32(&acce_bar[buf]), ((ji >> 1) & 1u) ^ 1u, abort_flag, a.err)) break;
         tc_fence_after();
@@ -400,26 +421,38 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         if (!ok) break;
         umma_commit_pair_mc(smem_u32(&accf_bar[buf]), 3);
-        job = next_job(ji + 1);
       }
       umma_commit_pair_mc(smem_u32(&done_bar), 1);
       mbar_wait_drain(smem_u32(&done_bar), 0, a.err);
     }
   } else if (warp == 2 + kEpiWarps) {
     if (lane == 0 && leader) {
-      const uint32_t job_peer0 = mapa_shared(smem_u32(&job_sh[0]), 1);
+      const uint32_t tile_peer0 = mapa_shared(smem_u32(&tile_sh[0]), 1);
       const uint32_t jfull_peer0 = mapa_shared(smem_u32(&jfull_bar[0]), 1);
-      for (uint32_t i = 0;; ++i) {
-        // claimed ahead of the slot: the counter's round trip is over when it frees
-        int j = static_cast<int>(atomicAdd(a.ctl, 1u));
-        if (j >= list.total) j = -1;
+      TileList list;
+      list.init(a, n_rows);
+      Tile x{};
+      for (uint32_t i = 0; x.kind >= 0; ++i) {
         const uint32_t s = i % kSlots;
+        // claimed when the slot frees and no earlier, so that pairs run at most
+        // kSlots tiles ahead of one another's claims
         if (!mbar_wait_cluster(smem_u32(&jempty_bar[s]), ((i / kSlots) & 1u) ^ 1u, abort_flag, a.err)) break;
-        *reinterpret_cast<volatile int*>(&job_sh[s]) = j;
+        const int j = static_cast<int>(atomicAdd(a.ctl, 1u));
+        if (j < list.total)
+          list.seek(j, x);
+        else
+          x.kind = -1;
+        const int4 q[3] = {make_int4(x.kind, x.chunk, x.buf, x.nk), make_int4(x.t, x.v, x.h, x.order),
+                           make_int4(x.t0, x.v0, x.need, 0)};
+        const uint32_t own = smem_u32(&tile_sh[s]), peer = tile_peer0 + s * static_cast<uint32_t>(sizeof(Tile));
+        const uint32_t peer_bar = jfull_peer0 + s * 8;
+        mbar_arrive_expect_tx_cluster(peer_bar, sizeof(Tile));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          st_shared_v4(own + 16 * k, q[k].x, q[k].y, q[k].z, q[k].w);
+          st_async_v4(peer + 16 * k, peer_bar, q[k]);
+        }
         mbar_arrive(smem_u32(&jfull_bar[s]));
-        st_shared_cluster_u32(job_peer0 + s * 4, static_cast<uint32_t>(j));
-        mbar_arrive_cluster(jfull_peer0 + s * 8);
-        if (j < 0) break;
       }
     }
   } else {
@@ -430,18 +463,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t acce_lead0 = mapa_shared(smem_u32(&acce_bar[0]), 0);
     const int slab = static_cast<int>(rank) * kEpiWarps + (warp - 2);
     bool ok = true;
-    // waits for this warp's box to be read out
+    // waits until this warp's box has been read out
     auto box_free = [&]() {
       if (lane == 0) bulk_wait_group_read<0>();
       __syncwarp();
     };
+    // chunk whose zdone this warp still has to raise for its last Z tile, or -1: its
+    // stores are awaited when the warp would wait anyway, and at the latest after
+    // the next tile, so nothing that waits for them is held up
+    int z_pending = -1;
+    auto raise_z = [&]() {
+      if (z_pending < 0) return;
+      if (lane == 0) {
+        bulk_wait_group<0>();
+        fence_proxy_async_global();
+        red_add_release_gpu(zdone + z_pending, 1u);
+      }
+      __syncwarp();
+      z_pending = -1;
+    };
+    // the tile's products, in order of ji
+    auto acc_full = [&](uint32_t ji) -> bool {
+      const uint32_t bar = smem_u32(&accf_bar[ji & 1u]), ph = (ji >> 1) & 1u;
+      if (z_pending >= 0 && !__all_sync(0xffffffffu, mbar_test_wait(bar, ph))) raise_z();
+      const bool full = mbar_wait(bar, ph, abort_flag, a.err);
+      tc_fence_after();
+      return full;
+    };
     Tile x;
-    for (uint32_t ji = 0; ok; ++ji) {
-      int job = -1;
-      if (lane == 0) job = next_job(ji);
-      job = __shfl_sync(0xffffffffu, job, 0);
-      if (job < 0) break;
-      list.seek(job, x);
+    for (uint32_t ji = 0; ok && next_tile(ji, x, true); ++ji) {
       const uint32_t buf = ji & 1u;
       const uint32_t taddr = tmem_base + lane_off + buf * 256 + hf * 128;
       const int r0 = static_cast<int>(rank) * 128 + q * 32;   // this warp's first row of the tile
@@ -467,18 +517,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int lx = in ? a.tok_p[row] - vbase : -1;
         const int nvalid = in ? V - vbase : 0;
         // the buffer's previous chunk must have been read
-        if (x.chunk >= list.nb) {
+        if (x.need > 0) {
+          raise_z();
           int good = 1;
           if (lane == 0) {
-            uint32_t nz, nr;
-            list.chunk_counts(x.chunk - list.nb, nz, nr);
-            good = turn_wait(cdone + x.chunk - list.nb, nr, abort_flag, a.ctl + 1, a.err) ? 1 : 0;
+            good = turn_wait(cdone + x.chunk - a.n_buf, static_cast<uint32_t>(x.need), abort_flag, a.ctl + 1, a.err) ? 1
+                                                                                                                   : 0;
             fence_proxy_async_global();
           }
           if (!(ok = __shfl_sync(0xffffffffu, good, 0) != 0)) break;
         }
-        if (!(ok = mbar_wait(smem_u32(&accf_bar[buf]), (ji >> 1) & 1u, abort_flag, a.err))) break;
-        tc_fence_after();
+        if (!(ok = acc_full(ji))) break;
         const int p0 = (x.v - x.v0) * 4 + hf * 2;
         const int gy = (x.buf * a.buf_panels + p0) * a.panel_rows + (x.t - x.t0) * 256 + r0;
 #pragma unroll 1
@@ -490,24 +539,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tmem_ld32(taddr + c * 64 + u * 32, v);
             const int lxc = lx - c * 64 - u * 32;
             const int nv = nvalid - c * 64 - u * 32;
+            auto p_of = [&](int j) -> float {   // g without the target's term
+              const float e = ex2_approx(fmaf(v[j], kLog2e, -lseL));
+              if constexpr (kEnt) return fmaf(ecoef, v[j] - mu, coef) * e;
+              return coef * e;
+            };
+            // a target or an invalid column among the warp's 32 x 32 values is rare
+            if (__any_sync(0xffffffffu, static_cast<unsigned>(lxc) < 32u || nv < 32)) {
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-              float g0, g1;
-              if constexpr (kEnt) {
-                g0 = fmaf(ecoef, v[j] - mu, coef) * ex2_approx(fmaf(v[j], kLog2e, -lseL));
-                g1 = fmaf(ecoef, v[j + 1] - mu, coef) * ex2_approx(fmaf(v[j + 1], kLog2e, -lseL));
-              } else {
-                g0 = coef * ex2_approx(fmaf(v[j], kLog2e, -lseL));
-                g1 = coef * ex2_approx(fmaf(v[j + 1], kLog2e, -lseL));
+              for (int j = 0; j < 32; j += 2) {
+                float g0 = p_of(j), g1 = p_of(j + 1);
+                if (j == lxc) g0 -= coef;
+                if (j + 1 == lxc) g1 -= coef;
+                if (j >= nv) g0 = 0.f;
+                if (j + 1 >= nv) g1 = 0.f;
+                w[u * 16 + j / 2] = pack_bf16x2(g0, g1);
               }
-              if (j == lxc) g0 -= coef;
-              if (j + 1 == lxc) g1 -= coef;
-              if (j >= nv) g0 = 0.f;
-              if (j + 1 >= nv) g1 = 0.f;
-              w[u * 16 + j / 2] = pack_bf16x2(g0, g1);
+            } else {
+#pragma unroll
+              for (int j = 0; j < 32; j += 2) w[u * 16 + j / 2] = pack_bf16x2(p_of(j), p_of(j + 1));
             }
           }
           if (c == 1) release_acc();
+          if (c == 0) raise_z();   // of the tile before, long stored
           box_free();
           const uint32_t rowp = box + lane * 128;
 #pragma unroll
@@ -521,19 +575,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             bulk_commit_group();
           }
         }
-        // stored for good: the chunk's readers may have it
-        if (lane == 0) {
-          bulk_wait_group<0>();
-          fence_proxy_async_global();
-          red_add_release_gpu(zdone + x.chunk, 1u);
-        }
-        __syncwarp();
+        z_pending = x.chunk;
         continue;
       }
       const bool dh = x.kind == kTileDH;
       const bool empty = !dh && n_rows == 0;   // dW of no rows: zeros, no products
-      if (!(ok = mbar_wait(smem_u32(&accf_bar[buf]), (ji >> 1) & 1u, abort_flag, a.err))) break;
-      tc_fence_after();
+      if (!(ok = acc_full(ji))) break;
       // the products have read the chunk buffer
       if (leader && warp == 2 && lane == 0) red_add_release_gpu(cdone + x.chunk, 1u);
       const int w = tile_w(x.h);
@@ -542,13 +589,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const CUtensorMap* map = dh ? &m.dh : &m.dw;
       uint32_t* turn = nullptr;
       if (a.det_turns) {
+        const int n_h = (H + 255) / 256;
+        raise_z();
         // reproducible sums: the contributions to a slab take turns in chunk order
-        const int64_t tile = dh ? static_cast<int64_t>(x.t) * list.n_h + x.h
-                                : static_cast<int64_t>(a.max_t + x.v) * list.n_h + x.h;
+        const int64_t tile = dh ? static_cast<int64_t>(x.t) * n_h + x.h
+                                : static_cast<int64_t>(a.max_t + x.v) * n_h + x.h;
         turn = a.det_turns + tile * (2 * kEpiWarps) + slab;
         int good = 1;
         if (lane == 0) {
-          good = turn_wait(turn, static_cast<uint32_t>(dh ? x.vc : x.tc), abort_flag, a.ctl + 1, a.err) ? 1 : 0;
+          good = turn_wait(turn, static_cast<uint32_t>(x.order), abort_flag, a.ctl + 1, a.err) ? 1 : 0;
           fence_proxy_async_global();
         }
         if (!(ok = __shfl_sync(0xffffffffu, good, 0) != 0)) break;
@@ -564,6 +613,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           for (int j = 0; j < 32; ++j) v[j] = 0.f;
         }
         if (s == 3 || col + 32 >= w) release_acc();
+        if (s == 0) raise_z();
         box_free();
         write_box32(box, lane, v);
         fence_proxy_async_smem();
@@ -573,19 +623,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tma_store_2d(map, box, x.h * 256 + col, y);
           else
             tma_reduce_add_2d(map, box, x.h * 256 + col, y);
-          bulk_commit_group();
         }
+        if (lane == 0) bulk_commit_group();
       }
       if (hf * 128 >= w) release_acc();   // no columns for this warp
+      raise_z();
       if (turn != nullptr) {
         if (lane == 0) {
           bulk_wait_group<0>();
           fence_proxy_async_global();
-          st_release_gpu(turn, static_cast<uint32_t>(dh ? x.vc : x.tc) + 1u);
+          st_release_gpu(turn, static_cast<uint32_t>(x.order) + 1u);
         }
         __syncwarp();
       }
     }
+    raise_z();
     if (lane == 0) bulk_wait_group<0>();
     __syncwarp();
   }
