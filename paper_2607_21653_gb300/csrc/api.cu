@@ -199,7 +199,7 @@ ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
 }
 
 struct Layout {
-  size_t counts, row_map, pos, tok_p, b_p, adv_p, h_p, part, zx, lse, coef, tile_flag, tile_list, red, dh32, turns, g, ctl;
+  size_t counts, row_map, pos, tok_p, b_p, adv_p, h_p, part, zx, lse, coef, tile_list, red, dh32, turns, g, ctl;
   size_t lp_p, ent_p, ecoef, mu, gate_p;
   size_t live_map, live_of, h_l, tok_l, lse_l, coef_l, ecoef_l, mu_l, total;
 };
@@ -240,13 +240,12 @@ Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = 
   L.b_p = take(Tcap * 4);
   L.adv_p = take(Tcap * 4);
   L.h_p = take(Tcap * H * 2);
-  L.part = take(static_cast<size_t>(kFwdParts) * S * Tcap * 16);
+  L.part = take(static_cast<size_t>(S) * Tcap * 16);
   L.zx = take(Tcap * 4);
   L.lse = take(Tcap * 4);
   L.coef = take(Tcap * 4);
-  L.tile_flag = take(ntile * 4);
   L.tile_list = take(ntile * 4);
-  L.red = take(ntile * kRedSlots * 8);
+  L.red = take(Tcap / kRedRows * kRedSlots * 8);
   L.dh32 = with_bwd ? take(static_cast<size_t>(Tcap) * H * 4) : o;
   const ChunkPlan cp = chunk_plan(T, H, V);
   L.turns = (with_bwd && det)
@@ -287,9 +286,8 @@ Layout vp_loss_layout(int64_t T) {
   L.row_map = take(T * 4);
   L.pos = take(T * 4);
   L.coef = take(Tcap * 4);
-  L.tile_flag = take(ntile * 4);
   L.tile_list = take(ntile * 4);
-  L.red = take(ntile * kRedSlots * 8);
+  L.red = take(Tcap / kRedRows * kRedSlots * 8);
   L.live_map = take(Tcap * 4);
   L.live_of = take(Tcap * 4);
   L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.dh32 = L.g = L.ctl = L.lp_p = L.ent_p = L.ecoef = L.mu = L.gate_p =
@@ -324,7 +322,7 @@ Layout vp_backward_layout(int64_t T, int64_t H, int64_t V) {
   const ChunkPlan cp = chunk_plan(T, H, V);
   L.g = take(cp.g_bytes());
   L.ctl = take(static_cast<size_t>(cp.ctl_words()) * 4);
-  L.row_map = L.pos = L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.coef = L.tile_flag = L.red =
+  L.row_map = L.pos = L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.coef = L.red =
       L.lp_p = L.ent_p = L.ecoef = L.mu = L.gate_p = L.ecoef_l = L.mu_l = o;
   L.turns = kNoRegion;
   L.total = o + 256;
@@ -345,7 +343,6 @@ Workspace carve(void* base, const Layout& L) {
   w.zx = reinterpret_cast<float*>(p + L.zx);
   w.lse = reinterpret_cast<float*>(p + L.lse);
   w.coef = reinterpret_cast<float*>(p + L.coef);
-  w.tile_flag = reinterpret_cast<int32_t*>(p + L.tile_flag);
   w.tile_list = reinterpret_cast<int32_t*>(p + L.tile_list);
   w.red = reinterpret_cast<double*>(p + L.red);
   w.dh32 = reinterpret_cast<float*>(p + L.dh32);
@@ -817,15 +814,15 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
   if (token_loss_out) MOLT_CUDA(cudaMemsetAsync(token_loss_out, 0, T * sizeof(float), stream), "memset token loss");
   ev_start(2, stream);
   if (opts) {
-    MOLT_LAUNCH(launch_merge_stats_ex(static_cast<int>(Tcap), static_cast<int>(V), kFwdParts * S, w, logp_out, entropy_out,
-                                    di->status, stream),
+    MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
+                           entropy_out, nullptr, w.lp_p, w.ent_p, di->status, stream),
               "merge");
     MOLT_LAUNCH(launch_seq_gate(static_cast<int>(T), static_cast<int>(Tcap), ex, w, di->status, stream), "gate");
     MOLT_LAUNCH(launch_loss_rows_ex(static_cast<int>(Tcap), denom, clip_lo, clip_hi, ex, w, token_loss_out, stream),
               "loss rows");
   } else {
-    MOLT_LAUNCH(launch_merge(true, static_cast<int>(Tcap), static_cast<int>(V), kFwdParts * S, denom, clip_lo, clip_hi, w,
-                           logp_out, entropy_out, token_loss_out, di->status, stream),
+    MOLT_LAUNCH(launch_merge(true, static_cast<int>(Tcap), static_cast<int>(V), S, denom, clip_lo, clip_hi, w,
+                           logp_out, entropy_out, token_loss_out, nullptr, nullptr, di->status, stream),
               "merge");
   }
   // rows whose gradient coefficient is 0 (masked out already; clipped, A = 0,
@@ -1055,8 +1052,8 @@ molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, c
   MOLT_CUDA(cudaMemsetAsync(logp_out, 0, T * sizeof(float), stream), "memset logp");
   if (entropy_out) MOLT_CUDA(cudaMemsetAsync(entropy_out, 0, T * sizeof(float), stream), "memset entropy");
   ev_start(2, stream);
-  MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), kFwdParts * S, 0.0, 0.f, 0.f, w, logp_out,
-                         entropy_out, nullptr, di->status, stream),
+  MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
+                         entropy_out, nullptr, nullptr, nullptr, di->status, stream),
             "merge");
   ev_stop(2, stream);
   return MOLT_OK;
@@ -1120,7 +1117,7 @@ molt_status molt_vp_partials(const uint16_t* hidden, const uint16_t* W_shard, co
   MOLT_TRY(run_forward(di, hidden, tokens, mask, nullptr, nullptr, T, H, V_shard, S, w, tm_h, tm_w, stream,
                        static_cast<int>(v_begin)));
   ev_start(2, stream);
-  MOLT_LAUNCH(launch_vp_local(static_cast<int>(T), static_cast<int>(Tcap), static_cast<int>(V_shard), kFwdParts * S, w,
+  MOLT_LAUNCH(launch_vp_local(static_cast<int>(T), static_cast<int>(Tcap), static_cast<int>(V_shard), S, w,
                               reinterpret_cast<float4*>(partials_out), stream),
               "shard statistics");
   ev_stop(2, stream);

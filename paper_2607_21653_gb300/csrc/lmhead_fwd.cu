@@ -8,9 +8,8 @@
 // in 64-element steps fed by TMA), and the epilogue warps fold it into per-row
 // running statistics:
 //   m = running max, s = sum exp(z - m), q = sum exp(z - m) (z - m)
-// and pick the target logit z[x].  The split's (m, s, q), one set for each
-// column half, go to a small workspace; a row-level merge kernel combines them
-// into
+// and pick the target logit z[x].  The split's (m, s, q) go to a small workspace;
+// a row-level merge kernel combines the splits into
 //   lse = m + log s,  logp = z[x] - lse,  entropy = log s - q / s.
 //
 // What bounds it: the tensor cores under the board's power cap, so the bytes
@@ -62,63 +61,68 @@ __device__ __forceinline__ void split_range(int s, int S, int n_vt, int& vt0, in
   vt1 = vt0 + per + (s < more ? 1 : 0);
 }
 
-// fold 32 logits (all columns valid) into the running (m, s, q2) of one row;
-// q2 is kept in log2 units: q2 = sum e * (z - m) * log2(e)
-__device__ __forceinline__ void fold_full(const float (&v)[32], float& m, float& s, float& q2) {
-  float cmax = v[0];
-#pragma unroll
-  for (int j = 1; j < 32; ++j) cmax = fmaxf(cmax, v[j]);
-  if (cmax > m) {
-    if (m != -INFINITY) {
-      const float d2 = (m - cmax) * kLog2e;
-      const float sc = ex2_approx(d2);
-      q2 = sc * fmaf(d2, s, q2);
-      s *= sc;
+// Running statistics of one row.  q2 is in log2 units: q2 = sum e (z - m) log2(e).
+// s is summed with its rounding carried along in c (Kahan), so that log s hardly
+// depends on how the columns are split.
+struct Stats {
+  float m = -INFINITY, s = 0.f, c = 0.f, q2 = 0.f;
+  __device__ __forceinline__ void raise(float cmax) {
+    if (cmax > m) {
+      if (m != -INFINITY) {
+        const float d2 = (m - cmax) * kLog2e;
+        const float sc = ex2_approx(d2);
+        q2 = sc * fmaf(d2, s, q2);
+        s *= sc;
+        c *= sc;
+      }
+      m = cmax;
     }
-    m = cmax;
   }
-  const float mL = m * kLog2e;
-  float s0 = 0.f, s1 = 0.f, q0 = 0.f, q1 = 0.f;
+  __device__ __forceinline__ void add(float ds, float dq) {
+    const float y = ds - c, t = s + y;
+    c = (t - s) - y;
+    s = t;
+    q2 += dq;
+  }
+};
+
+// fold 32 logits (all columns valid) into the row's statistics
+__device__ __forceinline__ void fold_full(const float (&v)[32], Stats& r) {
+  float cm[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-  for (int j = 0; j < 32; j += 2) {
-    const float y0 = fmaf(v[j], kLog2e, -mL);
-    const float y1 = fmaf(v[j + 1], kLog2e, -mL);
-    const float e0 = ex2_approx(y0);
-    const float e1 = ex2_approx(y1);
-    s0 += e0;
-    s1 += e1;
-    q0 = fmaf(e0, y0, q0);
-    q1 = fmaf(e1, y1, q1);
+  for (int j = 4; j < 32; ++j) cm[j & 3] = fmaxf(cm[j & 3], v[j]);
+  r.raise(fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3])));
+  const float mL = r.m * kLog2e;
+  float s[4] = {0.f, 0.f, 0.f, 0.f}, q[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int j = 0; j < 32; ++j) {
+    const float y = fmaf(v[j], kLog2e, -mL);
+    const float e = ex2_approx(y);
+    s[j & 3] += e;
+    q[j & 3] = fmaf(e, y, q[j & 3]);
   }
-  s += s0 + s1;
-  q2 += q0 + q1;
+  r.add((s[0] + s[1]) + (s[2] + s[3]), (q[0] + q[1]) + (q[2] + q[3]));
 }
 
 // same for a chunk where only the first `nv` (1..31) columns are valid
-__device__ __forceinline__ void fold_partial(const float (&v)[32], int nv, float& m, float& s, float& q2) {
+__device__ __forceinline__ void fold_partial(const float (&v)[32], int nv, Stats& r) {
   float cmax = v[0];
 #pragma unroll
   for (int j = 1; j < 32; ++j)
     if (j < nv) cmax = fmaxf(cmax, v[j]);
-  if (cmax > m) {
-    if (m != -INFINITY) {
-      const float d2 = (m - cmax) * kLog2e;
-      const float sc = ex2_approx(d2);
-      q2 = sc * fmaf(d2, s, q2);
-      s *= sc;
-    }
-    m = cmax;
-  }
-  const float mL = m * kLog2e;
+  r.raise(cmax);
+  const float mL = r.m * kLog2e;
+  float s = 0.f, q = 0.f;
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
     if (j < nv) {
       const float y = fmaf(v[j], kLog2e, -mL);
       const float e = ex2_approx(y);
       s += e;
-      q2 = fmaf(e, y, q2);
+      q = fmaf(e, y, q);
     }
   }
+  r.add(s, q);
 }
 
 // unit u of the list: 256-row token tile and vocab split
@@ -140,6 +144,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) uint64_t acce_bar[2];          // even CTA: one arrival per epilogue warp of the pair
   __shared__ __align__(8) uint64_t ufull_bar[kSlots];    // both CTAs: unit index written
   __shared__ __align__(8) uint64_t uempty_bar[kSlots];   // even CTA: every reader of both CTAs has it
+  __shared__ __align__(8) uint64_t hfull_bar[4], hempty_bar[4];   // the upper column half's (m, s, q) written / read
+  __shared__ float half_sh[4][3][32];
   __shared__ __align__(8) uint64_t done_bar;
   __shared__ int unit_sh[kSlots];
   __shared__ uint32_t tmem_base_sh;
@@ -164,6 +170,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       mbar_init(smem_u32(&ufull_bar[s]), 1);
       // readers: the MMA issuer, four producer warps, every epilogue warp
       mbar_init(smem_u32(&uempty_bar[s]), 5 + 2 * kEpiWarps);
+    }
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(smem_u32(&hfull_bar[i]), 1);
+      mbar_init(smem_u32(&hempty_bar[i]), 1);
     }
     mbar_init(smem_u32(&done_bar), 1);
     abort_sh = 0;
@@ -318,7 +328,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const int row = mt * 256 + r_in_tile;
       const bool valid = row < n_rows;
       const int x = valid ? a.tok_p[row] : -1;
-      float m = -INFINITY, ssum = 0.f, q2 = 0.f, zxv = 0.f;
+      Stats st;
+      float zxv = 0.f;
       bool found = false;
       for (int vt = vt0; vt < vt1; ++vt) {
         const uint32_t buf = acc_it & 1u;
@@ -341,9 +352,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             found = true;
           }
           if (c0 + 32 <= ncols)
-            fold_full(v, m, ssum, q2);
+            fold_full(v, st);
           else
-            fold_partial(v, ncols - c0, m, ssum, q2);
+            fold_partial(v, ncols - c0, st);
         }
         // every lane's TMEM reads are complete: one arrival per warp hands it back
         tc_fence_before();
@@ -352,9 +363,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         ++acc_it;
       }
       if (!ok) break;
-      if (valid) {
-        a.part[static_cast<int64_t>(2 * s + hf) * a.rows_cap + row] = make_float4(m, ssum, q2 * kLn2, 0.f);
-        if (found) a.zx[row] = zxv;
+      if (valid && found) a.zx[row] = zxv;
+      // the two warps of a lane quarter put their column halves together
+      if (hf == 1) {
+        if (!(ok = mbar_wait(smem_u32(&hempty_bar[q]), (ui & 1u) ^ 1u, abort_flag, a.err))) break;
+        half_sh[q][0][lane] = st.m;
+        half_sh[q][1][lane] = st.s;
+        half_sh[q][2][lane] = st.q2;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&hfull_bar[q]));
+      } else {
+        if (!(ok = mbar_wait(smem_u32(&hfull_bar[q]), ui & 1u, abort_flag, a.err))) break;
+        const float mo = half_sh[q][0][lane], so = half_sh[q][1][lane], qo = half_sh[q][2][lane];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&hempty_bar[q]));
+        const float M = fmaxf(st.m, mo);
+        float S2 = 0.f, Q2 = 0.f;
+        auto add = [&](float mi, float si, float qi) {
+          if (si > 0.f) {
+            const float d = (mi - M) * kLog2e;
+            const float f = ex2_approx(d);
+            S2 = fmaf(f, si, S2);
+            Q2 = fmaf(f, fmaf(d, si, qi), Q2);
+          }
+        };
+        add(st.m, st.s, st.q2);
+        add(mo, so, qo);
+        if (valid) a.part[static_cast<int64_t>(s) * a.rows_cap + row] = make_float4(M, S2, Q2 * kLn2, 0.f);
       }
     }
   }

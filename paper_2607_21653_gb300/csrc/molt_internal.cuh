@@ -12,7 +12,6 @@ namespace molt {
 
 constexpr int kTileM = 128;   // token rows per tile (TMEM lanes)
 constexpr int kFwdBN = 256;   // vocab columns per forward MMA tile
-constexpr int kFwdParts = 2;  // partial statistics per row and vocab split (one per column half)
 constexpr int kBwdBV = 256;   // vocab columns per backward unit
 constexpr int kBK = 64;       // K elements per 128-byte swizzled row
 
@@ -26,13 +25,12 @@ struct Workspace {
   float* b_p;           // [Tcap] packed behaviour log-probs
   float* adv_p;         // [Tcap] packed advantages
   uint16_t* h_p;        // [Tcap, H] packed hidden rows (bf16 bits), rows >= n zeroed
-  float4* part;         // [kFwdParts S, Tcap] per-split (max, sum exp, sum exp*(z-max), -)
+  float4* part;         // [S, Tcap] per-split (max, sum exp, sum exp*(z-max), -)
   float* zx;            // [Tcap] target logit
   float* lse;           // [Tcap]
   float* coef;          // [Tcap] m c / D
-  int32_t* tile_flag;   // [Tcap/128]
   int32_t* tile_list;   // [Tcap/128]
-  double* red;          // [n_tiles * kRedSlots] per-tile partial sums
+  double* red;          // [Tcap/kRedRows, kRedSlots] partial sums of kRedRows packed rows
   float* dh32;          // [Tcap, H] fp32 dhidden accumulator, by backward row (loss call only)
   // rows with a nonzero gradient coefficient, packed again (loss call only)
   int32_t* live_map;    // [Tcap] backward row -> packed row
@@ -54,7 +52,7 @@ struct Workspace {
   float* mu;            // [Tcap] sum_v p_v z_v = lse - entropy
   uint8_t* gate_p;      // [Tcap] sequence-gate weight per packed row
 };
-constexpr int kRedSlots = 8;
+constexpr int kRedRows = 32, kRedSlots = 8;
 
 // advantage estimators (values of molt_adv_estimator)
 constexpr int kAdvGrpo = 0, kAdvGroupMean = 1, kAdvDrGrpo = 2, kAdvRloo = 3, kAdvReinforcePP = 4;
@@ -67,7 +65,7 @@ struct FwdArgs {
   int n_split;
   int n_vtiles;
   int32_t* next_unit;   // zeroed
-  float4* part;         // [kFwdParts n_split, rows_cap]
+  float4* part;         // [n_split, rows_cap]
   float* zx;
   unsigned* err;
 };
@@ -157,16 +155,15 @@ cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, cuda
 // tok_shift is subtracted from every token (a vocabulary shard's first column)
 cudaError_t launch_gather(const uint16_t* hidden, const int32_t* tokens, const float* b, const float* adv, int T,
                           int Tcap, int H, const Workspace& ws, int n_sm, cudaStream_t s, int tok_shift = 0);
+// lp_p, ent_p: packed log-probs and entropies for the extended objective, or nullptr
 cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
-                         const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, unsigned* err,
-                         cudaStream_t s);
+                         const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, float* lp_p,
+                         float* ent_p, unsigned* err, cudaStream_t s);
 cudaError_t launch_finalize(int Tcap, double denom, bool with_ecoef, const Workspace& ws, float* loss_out,
                             void* stats_out, void* stats_ex_out, unsigned* err, cudaStream_t s);
 // the rows with a gradient (finalize's list) packed into whole tiles for the backward
 cudaError_t launch_live_gather(int H, bool with_ecoef, const Workspace& ws, int n_sm, cudaStream_t s);
 // extended objective: packed stats -> sequence gate -> loss rows
-cudaError_t launch_merge_stats_ex(int Tcap, int V, int n_parts, const Workspace& ws, float* logp_out, float* ent_out,
-                                  unsigned* err, cudaStream_t s);
 cudaError_t launch_seq_gate(int T, int Tcap, const LossEx& ex, const Workspace& ws, unsigned* err, cudaStream_t s);
 cudaError_t launch_loss_rows_ex(int Tcap, double denom, float clip_lo, float clip_hi, const LossEx& ex,
                                 const Workspace& ws, float* tokloss_out, cudaStream_t s);

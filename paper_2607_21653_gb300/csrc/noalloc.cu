@@ -67,15 +67,16 @@ __global__ void noalloc_init_kernel(int T, int32_t* counts, float* zx) {
 
 // merge the per-split partials of each row into logp and entropy; masked rows
 // are written as 0, active rows with an out-of-range token raise the status flag
-__global__ void __launch_bounds__(kMergeThreads)
+template <int kGroups>
+__global__ void __launch_bounds__(kRedRows * kGroups)
     noalloc_merge_kernel(int T, int V, int n_parts, int rows_cap, const int32_t* __restrict__ tokens,
                          const uint8_t* __restrict__ mask, const float4* __restrict__ part,
                          const float* __restrict__ zx, float* __restrict__ logp_out, float* __restrict__ ent_out,
                          unsigned* err) {
-  const int t = blockIdx.x * kTileM + threadIdx.x % kTileM;
+  const int t = blockIdx.x * kRedRows + threadIdx.x % kRedRows;
   const bool act = t < T && (mask == nullptr || mask[t] != 0);
-  const RowStats st = merge_row_parts(part, rows_cap, n_parts, t, act);
-  if (threadIdx.x >= kTileM || t >= T) return;
+  const RowStats st = merge_row_parts<kGroups>(part, rows_cap, n_parts, t, act);
+  if (threadIdx.x >= kRedRows || t >= T) return;
   if (!act) {
     logp_out[t] = 0.f;
     if (ent_out) ent_out[t] = 0.f;
@@ -149,7 +150,7 @@ extern "C" molt_status molt_token_logprobs_fwd_noalloc(const uint16_t* hidden, c
   // as far as the partials fit
   const int64_t S = std::max<int64_t>(
       1, std::min<int64_t>(forward_splits(Tcap, H, V, n_sm),
-                           static_cast<int64_t>(kNoAllocParts) * kNoAllocMaxRows / (kFwdParts * Tcap)));
+                           static_cast<int64_t>(kNoAllocParts) * kNoAllocMaxRows / Tcap));
 
   int32_t* counts = reinterpret_cast<int32_t*>(scratch);
   float4* part = reinterpret_cast<float4*>(scratch + kCountsBytes);
@@ -180,8 +181,11 @@ extern "C" molt_status molt_token_logprobs_fwd_noalloc(const uint16_t* hidden, c
   note_launches(1);
   timing_event(1, true, stream);
   timing_event(2, false, stream);
-  noalloc_merge_kernel<<<static_cast<int>((T + kTileM - 1) / kTileM), kMergeThreads, 0, stream>>>(
-      static_cast<int>(T), static_cast<int>(V), static_cast<int>(kFwdParts * S), static_cast<int>(Tcap), tokens, mask, part, zx, logp_out,
+  const int groups = merge_groups(static_cast<int>(S));
+  auto* merge = groups == kMergeGroupsMany ? &noalloc_merge_kernel<kMergeGroupsMany>
+                                           : &noalloc_merge_kernel<kMergeGroupsFew>;
+  merge<<<static_cast<int>((T + kRedRows - 1) / kRedRows), kRedRows * groups, 0, stream>>>(
+      static_cast<int>(T), static_cast<int>(V), static_cast<int>(S), static_cast<int>(Tcap), tokens, mask, part, zx, logp_out,
       entropy_out, status_word);
   if ((e = cudaGetLastError()) != cudaSuccess) return noalloc_fail(MOLT_ERR_CUDA, cudaGetErrorString(e));
   note_launches(1);

@@ -144,53 +144,47 @@ __global__ void mask_count_kernel(const uint8_t* __restrict__ mask, int64_t T,
   }
 }
 
-// block-wide exclusive scan of one int per thread (blockDim.x = 1024)
-__device__ int block_exclusive_scan(int v, int* total) {
+// Order-preserving compaction of rows [0, n) by one block of 1024 threads: every
+// row k gets emit(k, live, its index among the live ones).  Each warp takes a
+// contiguous stretch, 32 neighbouring rows at a time (a ballot counts them), so
+// loads and stores are whole lines; pred is evaluated twice.  Returns the count.
+template <class Pred, class Emit>
+__device__ __forceinline__ int compact_rows(int n, Pred pred, Emit emit) {
   __shared__ int wsum[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
+  const int per = ((n + 31) / 32 + 31) / 32 * 32;
+  const int k0 = w * per, k1 = min(n, k0 + per);
+  int c = 0;
+#pragma unroll 4
+  for (int k = k0 + lane; k - lane < k1; k += 32) c += __popc(__ballot_sync(0xffffffffu, k < k1 && pred(k)));
+  if (lane == 0) wsum[w] = c;
+  __syncthreads();
+  int before = 0, total = 0;
+  {
+    const int x = wsum[lane];
+    before = __reduce_add_sync(0xffffffffu, lane < w ? x : 0);
+    total = __reduce_add_sync(0xffffffffu, x);
   }
-  if (lane == 31) wsum[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int s = (lane < (int)(blockDim.x >> 5)) ? wsum[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += y;
-    }
-    wsum[lane] = s;
+#pragma unroll 4
+  for (int k = k0 + lane; k - lane < k1; k += 32) {
+    const bool live = k < k1 && pred(k);
+    const unsigned m = __ballot_sync(0xffffffffu, live);
+    if (k < k1) emit(k, live, before + __popc(m & ((1u << lane) - 1u)));
+    before += __popc(m);
   }
-  __syncthreads();
-  const int before = (w > 0 ? wsum[w - 1] : 0) + x - v;
-  if (total) *total = wsum[(blockDim.x >> 5) - 1];
-  __syncthreads();
-  return before;
+  return total;
 }
 
-// order-preserving list of active rows (mask != 0): one block, each thread a
-// contiguous chunk
+// order-preserving list of active rows (mask != 0)
 __global__ void __launch_bounds__(1024) compact_kernel(const uint8_t* __restrict__ mask, int T,
                                                        int32_t* __restrict__ row_map, int32_t* __restrict__ pos,
                                                        int32_t* __restrict__ counts) {
-  const int per = (T + blockDim.x - 1) / blockDim.x;
-  const int b = threadIdx.x * per, e = min(T, b + per);
-  int c = 0;
-  for (int t = b; t < e; ++t) c += (mask == nullptr || mask[t]) ? 1 : 0;
-  int total;
-  int k = block_exclusive_scan(c, &total);
-  for (int t = b; t < e; ++t) {
-    if (mask == nullptr || mask[t]) {
-      row_map[k] = t;
-      pos[t] = k++;
-    } else {
-      pos[t] = -1;
-    }
-  }
+  const int total = compact_rows(
+      T, [&](int t) { return mask == nullptr || mask[t] != 0; },
+      [&](int t, bool live, int k) {
+        if (live) row_map[k] = t;
+        pos[t] = live ? k : -1;
+      });
   if (threadIdx.x == 0) {
     counts[0] = total;
     counts[1] = 0;
@@ -231,28 +225,17 @@ __global__ void gather_kernel(const uint16_t* __restrict__ hidden, const int32_t
   }
 }
 
-// barrier of a block's first 128 threads
-__device__ __forceinline__ void sync128() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
-// deterministic sum over a block's first 128 threads (fixed tree)
+// sums over a warp in a fixed tree
 template <typename T>
-__device__ T block128_sum(T v, T* sh) {
+__device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  sync128();
-  T r = (sh[0] + sh[1]) + (sh[2] + sh[3]);
-  sync128();
-  return r;
+  return v;
 }
-__device__ double block128_max(double v, double* sh) {
+__device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  sync128();
-  double r = fmax(fmax(sh[0], sh[1]), fmax(sh[2], sh[3]));
-  sync128();
-  return r;
+  return v;
 }
 
 // Eq. 2 terms of one active row (Sec. 4.5: ratio against the behaviour
@@ -278,53 +261,49 @@ __device__ __forceinline__ RowLoss surrogate_row(float logp, float b, float A, f
   return r;
 }
 
-// the tile's fixed-tree partial sums (loss, ratio, entropy, max |log ratio|,
-// clip counts) and its activity flag; a block's first 128 threads call it
-__device__ void tile_partials(bool act, const RowLoss& rl, float ent, double* __restrict__ red,
-                              int32_t* __restrict__ tile_flag) {
-  __shared__ double shd[4];
-  __shared__ long long shl[4];
-  const long long any = block128_sum<long long>(act && rl.coef != 0.f ? 1 : 0, shl);
-  double* r = red + (int64_t)blockIdx.x * kRedSlots;
-  const double s_loss = block128_sum<double>(act ? (double)rl.tl : 0.0, shd);
-  const double s_ratio = block128_sum<double>(act ? (double)rl.ratio : 0.0, shd);
-  const double s_ent = block128_sum<double>(act ? (double)ent : 0.0, shd);
-  const double m_alr = block128_max(act ? rl.alr : 0.0, shd);
-  const long long c_lo = block128_sum<long long>(act ? rl.clip_lo_hit : 0, shl);
-  const long long c_hi = block128_sum<long long>(act ? rl.clip_hi_hit : 0, shl);
-  if (threadIdx.x == 0) {
-    tile_flag[blockIdx.x] = any ? 1 : 0;
+// partial sums of a warp's 32 packed rows (loss, ratio, entropy, max |log ratio|,
+// clip counts, KL, rejections): red[8 * row tile ..]
+__device__ void warp_partials(bool act, const RowLoss& rl, float ent, float kl, int rejected,
+                              double* __restrict__ r) {
+  const double s_loss = warp_sum<double>(act ? (double)rl.tl : 0.0);
+  const double s_ratio = warp_sum<double>(act ? (double)rl.ratio : 0.0);
+  const double s_ent = warp_sum<double>(act ? (double)ent : 0.0);
+  const double m_alr = warp_max(act ? rl.alr : 0.0);
+  const int c_lo = __reduce_add_sync(0xffffffffu, act ? rl.clip_lo_hit : 0);
+  const int c_hi = __reduce_add_sync(0xffffffffu, act ? rl.clip_hi_hit : 0);
+  const double s_kl = warp_sum<double>(act ? (double)kl : 0.0);
+  const int c_rej = __reduce_add_sync(0xffffffffu, rejected);
+  if ((threadIdx.x & 31) == 0) {
     r[0] = s_loss;
     r[1] = s_ratio;
     r[2] = s_ent;
     r[3] = m_alr;
     r[4] = static_cast<double>(c_lo);
     r[5] = static_cast<double>(c_hi);
-    r[6] = 0.0;
-    r[7] = 0.0;
+    r[6] = s_kl;
+    r[7] = static_cast<double>(c_rej);
   }
 }
 
-// One block per packed tile of 128 rows (merge_row_parts' threads): merge the
-// per-split online softmax partials of each row into lse, logp and entropy; in
-// loss mode the first 128 threads also form
+// One block per kRedRows packed rows (merge_row_parts' threads): merge the per-split
+// online softmax partials of each row into lse, logp and entropy; in loss mode also
 // the ratio, the clipped surrogate (Sec. 4.5, PPO form), the Eq. 2 coefficient
-// m c / D, per-tile partial sums and the tile's activity flag.
-__global__ void __launch_bounds__(kMergeThreads) merge_kernel(
+// m c / D and the rows' partial sums.
+template <int kGroups>
+__global__ void __launch_bounds__(kRedRows * kGroups) merge_kernel(
     int loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
     const int32_t* __restrict__ counts, const int32_t* __restrict__ row_map, const int32_t* __restrict__ tok_p,
     const float* __restrict__ b_p, const float* __restrict__ adv_p, const float4* __restrict__ part,
     const float* __restrict__ zx, float* __restrict__ lse_o, float* __restrict__ coef_o,
-    int32_t* __restrict__ tile_flag, double* __restrict__ red, float* __restrict__ logp_out,
-    float* __restrict__ ent_out, float* __restrict__ tokloss_out, float* __restrict__ lp_p,
+    double* __restrict__ red, float* __restrict__ logp_out, float* __restrict__ ent_out,
+    float* __restrict__ tokloss_out, float* __restrict__ lp_p,
     float* __restrict__ ent_p, unsigned* err) {
   const int n = counts[0];
-  const int n_tiles = (n + kTileM - 1) / kTileM;
-  if ((int)blockIdx.x >= n_tiles) return;
-  const int k = blockIdx.x * kTileM + threadIdx.x % kTileM;
+  if ((int)blockIdx.x * kRedRows >= n) return;
+  const int k = blockIdx.x * kRedRows + threadIdx.x % kRedRows;
   const bool act = k < n;
-  const RowStats st = merge_row_parts(part, Tcap, n_parts, k, act);
-  if (threadIdx.x >= kTileM) return;
+  const RowStats st = merge_row_parts<kGroups>(part, Tcap, n_parts, k, act);
+  if (threadIdx.x >= kRedRows) return;
   const double D = denom > 0.0 ? denom : static_cast<double>(n);
   float logp = 0.f, ent = 0.f;
   RowLoss rl{0.f, 0.f, 0.f, 0, 0, 0.0};
@@ -345,8 +324,8 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(
     if (ent_p) ent_p[k] = ent;
   }
   if (!loss_mode) return;
-  if (k < Tcap) coef_o[k] = rl.coef;
-  tile_partials(act, rl, ent, red, tile_flag);
+  if (act) coef_o[k] = rl.coef;
+  warp_partials(act, rl, ent, 0.f, 0, red + (int64_t)blockIdx.x * kRedSlots);
 }
 
 // ---------------------------------------------------------------------------
@@ -361,13 +340,14 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(
 // sum exp(z - M), Q = sum exp(z - M) (z - M), z_x the target logit if the
 // target lies in the shard (tok_p holds the shard-local token) and -inf
 // otherwise.  Masked rows get the empty statistics (-inf, 0, 0, -inf).
-__global__ void __launch_bounds__(kMergeThreads) vp_local_kernel(
+template <int kGroups>
+__global__ void __launch_bounds__(kRedRows * kGroups) vp_local_kernel(
     int T, int Tcap, int V_s, int n_parts, const int32_t* __restrict__ pos, const int32_t* __restrict__ tok_p,
     const float4* __restrict__ part, const float* __restrict__ zx, float4* __restrict__ out) {
-  const int t = blockIdx.x * kTileM + threadIdx.x % kTileM;
+  const int t = blockIdx.x * kRedRows + threadIdx.x % kRedRows;
   const int k = t < T ? pos[t] : -1;
-  const RowStats st = merge_row_parts(part, Tcap, n_parts, k, k >= 0);
-  if (threadIdx.x >= kTileM || t >= T) return;
+  const RowStats st = merge_row_parts<kGroups>(part, Tcap, n_parts, k, k >= 0);
+  if (threadIdx.x >= kRedRows || t >= T) return;
   if (k < 0) {
     out[t] = make_float4(-INFINITY, 0.f, 0.f, -INFINITY);
     return;
@@ -384,8 +364,7 @@ __global__ void __launch_bounds__(kMergeThreads) vp_local_kernel(
 __global__ void __launch_bounds__(128) vp_merge_kernel(
     int T, int n_shards, double denom, float clip_lo, float clip_hi, const int32_t* __restrict__ counts,
     const int32_t* __restrict__ row_map, const float4* __restrict__ parts, const float* __restrict__ b,
-    const float* __restrict__ adv, float* __restrict__ coef_p, int32_t* __restrict__ tile_flag,
-    double* __restrict__ red, float* __restrict__ lse_out, float* __restrict__ coef_out,
+    const float* __restrict__ adv, float* __restrict__ coef_p, double* __restrict__ red, float* __restrict__ lse_out, float* __restrict__ coef_out,
     float* __restrict__ logp_out, float* __restrict__ ent_out, float* __restrict__ tokloss_out, unsigned* err) {
   const int n = counts[0];
   const int n_tiles = (n + kTileM - 1) / kTileM;
@@ -425,8 +404,8 @@ __global__ void __launch_bounds__(128) vp_merge_kernel(
     if (ent_out) ent_out[t] = ent;
     if (tokloss_out) tokloss_out[t] = rl.tl;
   }
-  if (k < ((n + kTileM - 1) / kTileM) * kTileM) coef_p[k] = rl.coef;
-  tile_partials(act, rl, ent, red, tile_flag);
+  if (act) coef_p[k] = rl.coef;
+  if (k / kRedRows * kRedRows < n) warp_partials(act, rl, ent, 0.f, 0, red + (int64_t)(k / kRedRows) * kRedSlots);
 }
 
 // The rows of one shard's backward: those with a gradient coefficient (coef
@@ -436,20 +415,12 @@ __global__ void __launch_bounds__(1024) vp_live_kernel(int T, const float* __res
                                                        int32_t* __restrict__ counts, int32_t* __restrict__ tile_list,
                                                        int32_t* __restrict__ live_map,
                                                        int32_t* __restrict__ live_of) {
-  const int per = (T + blockDim.x - 1) / blockDim.x;
-  const int t0 = threadIdx.x * per, t1 = min(T, t0 + per);
-  int c = 0;
-  for (int t = t0; t < t1; ++t) c += coef[t] != 0.f ? 1 : 0;
-  int total;
-  int j = block_exclusive_scan(c, &total);
-  for (int t = t0; t < t1; ++t) {
-    if (coef[t] != 0.f) {
-      live_map[j] = t;
-      live_of[t] = j++;
-    } else {
-      live_of[t] = -1;
-    }
-  }
+  const int total = compact_rows(
+      T, [&](int t) { return coef[t] != 0.f; },
+      [&](int t, bool live, int j) {
+        if (live) live_map[j] = t;
+        live_of[t] = live ? j : -1;
+      });
   const int n_lt = (total + kTileM - 1) / kTileM;
   for (int b = threadIdx.x; b < n_lt; b += blockDim.x) tile_list[b] = b;
   if (threadIdx.x == 0) {
@@ -535,23 +506,21 @@ __global__ void __launch_bounds__(128) loss_rows_ex_kernel(
     const int32_t* __restrict__ row_map, const float* __restrict__ b_p, const float* __restrict__ adv_p,
     const float* __restrict__ lp_p, const float* __restrict__ ent_p, const float* __restrict__ lse,
     const uint8_t* __restrict__ gate_p, float* __restrict__ coef_o, float* __restrict__ ecoef_o,
-    float* __restrict__ mu_o, int32_t* __restrict__ tile_flag, double* __restrict__ red,
-    float* __restrict__ tokloss_out) {
-  __shared__ double shd[4];
-  __shared__ long long shl[4];
+    float* __restrict__ mu_o, double* __restrict__ red, float* __restrict__ tokloss_out) {
   const int n = counts[0];
   const int n_tiles = (n + kTileM - 1) / kTileM;
   if ((int)blockIdx.x >= n_tiles) return;
   const int k = blockIdx.x * kTileM + threadIdx.x;
   const bool act = k < n;
   const double D = denom > 0.0 ? denom : static_cast<double>(n);
-  float coef = 0.f, ecoef = 0.f, mu = 0.f, tl = 0.f, ratio = 0.f, ent = 0.f, kl = 0.f;
-  int clip_lo_hit = 0, clip_hi_hit = 0, rejected = 0;
-  double alr = 0.0;
+  float ecoef = 0.f, mu = 0.f, ent = 0.f, kl = 0.f;
+  int rejected = 0;
+  RowLoss rl{0.f, 0.f, 0.f, 0, 0, 0.0};
   if (act) {
     const float logp = lp_p[k], b = b_p[k], A = adv_p[k];
     ent = ent_p[k];
-    ratio = expf(logp - b);
+    const float ratio = expf(logp - b);
+    rl.ratio = ratio;
     const float lo = 1.0f - clip_lo, hi = 1.0f + clip_hi;
     const bool clipped = (A > 0.f && ratio > hi) || (A < 0.f && ratio < lo);
     const float rc = fminf(fmaxf(ratio, lo), hi);
@@ -566,45 +535,25 @@ __global__ void __launch_bounds__(128) loss_rows_ex_kernel(
     }
     const bool keep = gate_p == nullptr || gate_p[k] != 0;
     if (keep) {
-      tl = l_pg + ex.kl_coef * kl - ex.entropy_coef * ent;
-      coef = (D > 0.0) ? static_cast<float>(static_cast<double>(c + c_kl) / D) : 0.f;
+      rl.tl = l_pg + ex.kl_coef * kl - ex.entropy_coef * ent;
+      rl.coef = (D > 0.0) ? static_cast<float>(static_cast<double>(c + c_kl) / D) : 0.f;
       ecoef = (D > 0.0) ? static_cast<float>(static_cast<double>(ex.entropy_coef) / D) : 0.f;
-      clip_lo_hit = (clipped && A < 0.f) ? 1 : 0;
-      clip_hi_hit = (clipped && A > 0.f) ? 1 : 0;
+      rl.clip_lo_hit = (clipped && A < 0.f) ? 1 : 0;
+      rl.clip_hi_hit = (clipped && A > 0.f) ? 1 : 0;
     } else {
       kl = 0.f;
       rejected = 1;
     }
     mu = lse[k] - ent;
-    alr = fabs(static_cast<double>(logp) - static_cast<double>(b));
-    if (tokloss_out) tokloss_out[row_map[k]] = tl;
+    rl.alr = fabs(static_cast<double>(logp) - static_cast<double>(b));
+    if (tokloss_out) tokloss_out[row_map[k]] = rl.tl;
   }
   if (k < Tcap) {
-    coef_o[k] = coef;
+    coef_o[k] = rl.coef;
     ecoef_o[k] = ecoef;
     mu_o[k] = mu;
   }
-  const long long any = block128_sum<long long>(coef != 0.f || ecoef != 0.f ? 1 : 0, shl);
-  double* rr = red + (int64_t)blockIdx.x * kRedSlots;
-  const double s_loss = block128_sum<double>(act ? (double)tl : 0.0, shd);
-  const double s_ratio = block128_sum<double>(act ? (double)ratio : 0.0, shd);
-  const double s_ent = block128_sum<double>(act ? (double)ent : 0.0, shd);
-  const double m_alr = block128_max(alr, shd);
-  const long long c_lo = block128_sum<long long>(clip_lo_hit, shl);
-  const long long c_hi = block128_sum<long long>(clip_hi_hit, shl);
-  const double s_kl = block128_sum<double>(act ? (double)kl : 0.0, shd);
-  const long long c_rej = block128_sum<long long>(rejected, shl);
-  if (threadIdx.x == 0) {
-    tile_flag[blockIdx.x] = any ? 1 : 0;
-    rr[0] = s_loss;
-    rr[1] = s_ratio;
-    rr[2] = s_ent;
-    rr[3] = m_alr;
-    rr[4] = static_cast<double>(c_lo);
-    rr[5] = static_cast<double>(c_hi);
-    rr[6] = s_kl;
-    rr[7] = static_cast<double>(c_rej);
-  }
+  if (k / kRedRows * kRedRows < n) warp_partials(act, rl, ent, kl, rejected, red + (int64_t)(k / kRedRows) * kRedSlots);
 }
 
 struct StatsDev {
@@ -630,88 +579,64 @@ __global__ void __launch_bounds__(1024) finalize_kernel(double denom, int32_t* _
                                                         const float* __restrict__ ecoef,
                                                         int32_t* __restrict__ live_map,
                                                         int32_t* __restrict__ live_of, unsigned* err) {
-  __shared__ double sh[kFinSlots][32];
+  __shared__ double sh[kFinSlots][4];
   const int n = counts[0];
-  const int n_tiles = (n + kTileM - 1) / kTileM;
-  double a[kFinSlots] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int b = threadIdx.x; b < n_tiles; b += blockDim.x) {
-    const double* r = red + (int64_t)b * kRedSlots;
-#pragma unroll
-    for (int q = 0; q < kFinSlots; ++q) a[q] = (q == 3) ? fmax(a[q], r[q]) : a[q] + r[q];
-  }
-  // fixed shuffle tree inside each warp, then warp 0 over the 32 warp results
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int q = 0; q < kFinSlots; ++q) {
-      const double y = __shfl_xor_sync(0xffffffffu, a[q], o);
-      a[q] = (q == 3) ? fmax(a[q], y) : a[q] + y;
+  const int n_rt = (n + kRedRows - 1) / kRedRows;
+  // four warps to a slot, then thread 0 over their results: a fixed order
+  {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = w >> 2;
+    double a = 0.0;
+#pragma unroll 4
+    for (int b = (w & 3) * 32 + lane; b < n_rt; b += 128) {
+      const double x = red[(int64_t)b * kRedSlots + q];
+      a = (q == 3) ? fmax(a, x) : a + x;
     }
-  }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0)
-    for (int q = 0; q < kFinSlots; ++q) sh[q][w] = a[q];
-  __syncthreads();
-  if (w == 0) {
-    for (int q = 0; q < kFinSlots; ++q) a[q] = sh[q][lane];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-      for (int q = 0; q < kFinSlots; ++q) {
-        const double y = __shfl_xor_sync(0xffffffffu, a[q], o);
-        a[q] = (q == 3) ? fmax(a[q], y) : a[q] + y;
-      }
-    }
-    if (lane == 0)
-      for (int q = 0; q < kFinSlots; ++q) sh[q][0] = a[q];
+    a = (q == 3) ? warp_max(a) : warp_sum(a);
+    if (lane == 0) sh[q][w & 3] = a;
   }
   __syncthreads();
   const double D = denom > 0.0 ? denom : static_cast<double>(n);
   if (threadIdx.x == 0) {
+    double tot[kFinSlots];
+#pragma unroll
+    for (int q = 0; q < kFinSlots; ++q)
+      tot[q] = (q == 3) ? fmax(fmax(sh[q][0], sh[q][1]), fmax(sh[q][2], sh[q][3]))
+                        : (sh[q][0] + sh[q][1]) + (sh[q][2] + sh[q][3]);
     if (!(D > 0.0)) atomicOr(err, kDevErrZeroDenom);
-    const double loss = D > 0.0 ? sh[0][0] / D : 0.0;
+    const double loss = D > 0.0 ? tot[0] / D : 0.0;
     if (loss_out) *loss_out = static_cast<float>(loss);
     if (stats) {
       stats->denom = D;
       stats->loss = loss;
-      stats->sum_ratio = sh[1][0];
-      stats->sum_entropy = sh[2][0];
-      stats->max_abs_log_ratio = sh[3][0];
+      stats->sum_ratio = tot[1];
+      stats->sum_entropy = tot[2];
+      stats->max_abs_log_ratio = tot[3];
       stats->n_active = n;
-      stats->n_clip_low = static_cast<long long>(sh[4][0]);
-      stats->n_clip_high = static_cast<long long>(sh[5][0]);
+      stats->n_clip_low = static_cast<long long>(tot[4]);
+      stats->n_clip_high = static_cast<long long>(tot[5]);
     }
     if (stats_ex) {
       StatsDev& b = stats_ex->base;
       b.denom = D;
       b.loss = loss;
-      b.sum_ratio = sh[1][0];
-      b.sum_entropy = sh[2][0];
-      b.max_abs_log_ratio = sh[3][0];
+      b.sum_ratio = tot[1];
+      b.sum_entropy = tot[2];
+      b.max_abs_log_ratio = tot[3];
       b.n_active = n;
-      b.n_clip_low = static_cast<long long>(sh[4][0]);
-      b.n_clip_high = static_cast<long long>(sh[5][0]);
-      stats_ex->sum_kl = sh[6][0];
-      stats_ex->n_tokens_rejected = static_cast<long long>(sh[7][0]);
+      b.n_clip_low = static_cast<long long>(tot[4]);
+      b.n_clip_high = static_cast<long long>(tot[5]);
+      stats_ex->sum_kl = tot[6];
+      stats_ex->n_tokens_rejected = static_cast<long long>(tot[7]);
       stats_ex->n_seq_rejected = counts[2];
     }
   }
   // compact the rows with a gradient (order preserving)
-  auto live = [&](int k) { return coef[k] != 0.f || (ecoef != nullptr && ecoef[k] != 0.f); };
-  const int per = (n + blockDim.x - 1) / blockDim.x;
-  const int k0 = threadIdx.x * per, k1 = min(n, k0 + per);
-  int c = 0;
-  for (int k = k0; k < k1; ++k) c += live(k) ? 1 : 0;
-  int total;
-  int j = block_exclusive_scan(c, &total);
-  for (int k = k0; k < k1; ++k) {
-    if (live(k)) {
-      live_map[j] = k;
-      live_of[k] = j++;
-    } else {
-      live_of[k] = -1;
-    }
-  }
+  const int total = compact_rows(
+      n, [&](int k) { return coef[k] != 0.f || (ecoef != nullptr && ecoef[k] != 0.f); },
+      [&](int k, bool live, int j) {
+        if (live) live_map[j] = k;
+        live_of[k] = live ? j : -1;
+      });
   const int n_lt = (total + kTileM - 1) / kTileM;
   for (int b = threadIdx.x; b < n_lt; b += blockDim.x) tile_list[b] = b;
   if (threadIdx.x == 0) {
@@ -858,23 +783,15 @@ cudaError_t launch_gather(const uint16_t* hidden, const int32_t* tokens, const f
 }
 
 cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
-                         const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, unsigned* err,
-                         cudaStream_t s) {
-  const int blocks = Tcap / kTileM;
-  merge_kernel<<<blocks, kMergeThreads, 0, s>>>(loss_mode ? 1 : 0, Tcap, V, n_parts, denom, clip_lo, clip_hi, ws.counts,
-                                          ws.row_map, ws.tok_p, ws.b_p, ws.adv_p, ws.part, ws.zx, ws.lse, ws.coef,
-                                          ws.tile_flag, ws.red, logp_out, ent_out, tokloss_out, nullptr, nullptr,
-                                          err);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_merge_stats_ex(int Tcap, int V, int n_parts, const Workspace& ws, float* logp_out, float* ent_out,
-                                  unsigned* err, cudaStream_t s) {
-  const int blocks = Tcap / kTileM;
+                         const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, float* lp_p,
+                         float* ent_p, unsigned* err, cudaStream_t s) {
+  const int blocks = Tcap / kRedRows;
   if (blocks == 0) return cudaSuccess;
-  merge_kernel<<<blocks, kMergeThreads, 0, s>>>(0, Tcap, V, n_parts, 0.0, 0.f, 0.f, ws.counts, ws.row_map, ws.tok_p, ws.b_p,
-                                          ws.adv_p, ws.part, ws.zx, ws.lse, ws.coef, ws.tile_flag, ws.red, logp_out,
-                                          ent_out, nullptr, ws.lp_p, ws.ent_p, err);
+  const int groups = merge_groups(n_parts);
+  auto* k = groups == kMergeGroupsMany ? &merge_kernel<kMergeGroupsMany> : &merge_kernel<kMergeGroupsFew>;
+  k<<<blocks, kRedRows * groups, 0, s>>>(loss_mode ? 1 : 0, Tcap, V, n_parts, denom, clip_lo, clip_hi, ws.counts,
+                                         ws.row_map, ws.tok_p, ws.b_p, ws.adv_p, ws.part, ws.zx, ws.lse, ws.coef,
+                                         ws.red, logp_out, ent_out, tokloss_out, lp_p, ent_p, err);
   return cudaGetLastError();
 }
 
@@ -893,7 +810,7 @@ cudaError_t launch_loss_rows_ex(int Tcap, double denom, float clip_lo, float cli
   loss_rows_ex_kernel<<<blocks, kTileM, 0, s>>>(Tcap, denom, clip_lo, clip_hi, ex, ws.counts, ws.row_map, ws.b_p,
                                                  ws.adv_p, ws.lp_p, ws.ent_p, ws.lse,
                                                  ex.seq ? ws.gate_p : nullptr, ws.coef, ws.ecoef, ws.mu,
-                                                 ws.tile_flag, ws.red, tokloss_out);
+                                                 ws.red, tokloss_out);
   return cudaGetLastError();
 }
 
@@ -917,8 +834,10 @@ cudaError_t launch_live_gather(int H, bool with_ecoef, const Workspace& ws, int 
 cudaError_t launch_vp_local(int T, int Tcap, int V_s, int n_parts, const Workspace& ws, float4* out,
                             cudaStream_t s) {
   if (T <= 0) return cudaSuccess;
-  vp_local_kernel<<<(T + kTileM - 1) / kTileM, kMergeThreads, 0, s>>>(T, Tcap, V_s, n_parts, ws.pos_of_row, ws.tok_p, ws.part, ws.zx,
-                                                   out);
+  const int groups = merge_groups(n_parts);
+  auto* k = groups == kMergeGroupsMany ? &vp_local_kernel<kMergeGroupsMany> : &vp_local_kernel<kMergeGroupsFew>;
+  k<<<(T + kRedRows - 1) / kRedRows, kRedRows * groups, 0, s>>>(T, Tcap, V_s, n_parts, ws.pos_of_row, ws.tok_p, ws.part,
+                                                                ws.zx, out);
   return cudaGetLastError();
 }
 
@@ -929,7 +848,7 @@ cudaError_t launch_vp_merge(int T, int Tcap, int n_shards, double denom, float c
   const int blocks = Tcap / kTileM;
   if (blocks == 0) return cudaSuccess;
   vp_merge_kernel<<<blocks, kTileM, 0, s>>>(T, n_shards, denom, clip_lo, clip_hi, ws.counts, ws.row_map, parts, b,
-                                            adv, ws.coef, ws.tile_flag, ws.red, lse_out, coef_out, logp_out,
+                                            adv, ws.coef, ws.red, lse_out, coef_out, logp_out,
                                             ent_out, tokloss_out, err);
   return cudaGetLastError();
 }
