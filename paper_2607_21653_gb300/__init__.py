@@ -406,7 +406,7 @@ def policy_loss_fwd_bwd(hidden, weight, tokens, behavior_logp, adv, mask=None, c
     if dW is None:
         dW = torch.empty(V, H, dtype=torch.float32, device=dev)
         accumulate_dW = False
-    stats = torch.zeros(9, dtype=torch.float64, device=dev)
+    stats = torch.empty(9, dtype=torch.float64, device=dev)
     logp = ent = tl = None
     if want_token_outputs:
         logp = torch.empty(T, dtype=torch.float32, device=dev)
@@ -467,7 +467,7 @@ def policy_loss_fwd_bwd_ex(hidden, weight, tokens, behavior_logp, adv, mask=None
     if dW is None:
         dW = torch.empty(V, H, dtype=torch.float32, device=dev)
         accumulate_dW = False
-    stats = torch.zeros(12, dtype=torch.float64, device=dev)
+    stats = torch.empty(12, dtype=torch.float64, device=dev)
     logp = ent = tl = None
     if want_token_outputs:
         logp = torch.empty(T, dtype=torch.float32, device=dev)
@@ -526,7 +526,7 @@ def vp_loss(partials, behavior_logp, adv, mask=None, clip_lo=0.2, clip_hi=0.2, d
     out = {"loss": torch.empty(1, dtype=torch.float32, device=dev)}
     for k in ("lse", "coef", "logp", "entropy", "token_loss"):
         out[k] = torch.empty(T, dtype=torch.float32, device=dev)
-    out["stats"] = torch.zeros(9, dtype=torch.float64, device=dev)
+    out["stats"] = torch.empty(9, dtype=torch.float64, device=dev)
     nbytes = int(load().molt_vp_loss_workspace_bytes(T))
     ws = _workspace(nbytes, dev, "vp_loss", stream)
     _check(load().molt_vp_loss(

@@ -144,10 +144,9 @@ struct ChunkPlan {
   int64_t n_t = 0, n_v = 0, n_h = 0, chunk_t = 0, chunk_v = 0, max_chunks = 0;
   int64_t panel_rows = 0, buf_panels = 0;   // of one chunk buffer: token rows of a panel, 64-column panels
   int n_buf = 0;
-  bool one_token_chunk = false;
   int64_t g_rows() const { return n_buf * buf_panels * panel_rows; }
   size_t g_bytes() const { return use ? static_cast<size_t>(g_rows()) * kBK * 2 : 0; }
-  int64_t ctl_words() const { return use ? kChunkCtlHead + 2 * max_chunks : 0; }
+  int64_t ctl_words() const { return use ? kChunkCtlHead + 4 * max_chunks : 0; }
   int64_t turn_words() const { return use ? (n_t + n_v) * n_h * 16 : 0; }
 };
 // T is the call's row count; the rows with a gradient, at most as many, are
@@ -194,7 +193,6 @@ ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
   p.buf_panels = cv * 4;
   // all buffers together stay at 64 MB, half of L2
   p.n_buf = static_cast<int>(std::min<int64_t>(8, std::max<int64_t>(2, 512 / (ct * cv))));
-  p.one_token_chunk = n_tc == 1;
   return p;
 }
 
@@ -531,10 +529,10 @@ struct ZeroJoin {
 molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int32_t* tokens, const uint8_t* mask,
                         const float* b, const float* adv, int64_t T, int64_t H, int64_t V, int S,
                         const Workspace& w, const CUtensorMap& tm_h, const CUtensorMap& tm_w, cudaStream_t s,
-                        int tok_shift = 0) {
+                        const ZeroRows& zero, int64_t ctl_words = 0, int tok_shift = 0) {
   const int64_t Tcap = round_tiles(T);
   ev_start(0, s);
-  MOLT_LAUNCH(launch_compact(mask, static_cast<int>(T), w, s), "compact");
+  MOLT_LAUNCH(launch_compact(mask, static_cast<int>(T), w, zero, ctl_words, s), "compact");
   MOLT_LAUNCH(launch_gather(hidden, tokens, b, adv, static_cast<int>(T), static_cast<int>(Tcap), static_cast<int>(H),
                           w, di->n_sm, s, tok_shift),
             "gather");
@@ -557,21 +555,21 @@ molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int3
   return MOLT_OK;
 }
 
-// Zero what the backward adds to on stream s: the dhidden accumulator, the
-// chunk counters, the deterministic schedule's turn counters and, unless the
-// call accumulates into it or stores it whole, dW.
+// Zero on stream s what the backward adds to: the deterministic schedule's turn
+// counters and, for the kernels that only add, the dhidden accumulator and, unless
+// the call accumulates into it, dW (the backward over chunks stores the first
+// contributions; its counters are zeroed with the compaction).
 molt_status zero_backward_targets(const Workspace& w, int64_t T, int64_t H, int64_t V, bool det, float* dW_out,
                                   int accumulate_dW, cudaStream_t s) {
   const int64_t Tcap = round_tiles(T);
   const ChunkPlan cp = chunk_plan(T, H, V);
-  MOLT_CUDA(cudaMemsetAsync(w.dh32, 0, static_cast<size_t>(Tcap) * H * sizeof(float), s), "memset dh32");
-  if (cp.use) MOLT_CUDA(cudaMemsetAsync(w.ctl, 0, static_cast<size_t>(cp.ctl_words()) * 4, s), "memset counters");
   if (det) {
     const int64_t words = cp.use ? cp.turn_words() : turn_layout(Tcap, H, V).words;
     MOLT_CUDA(cudaMemsetAsync(w.turns, 0, static_cast<size_t>(words) * 4, s), "memset turns");
   }
-  if (!accumulate_dW && !(cp.use && cp.one_token_chunk))
-    MOLT_CUDA(cudaMemsetAsync(dW_out, 0, static_cast<size_t>(V) * H * sizeof(float), s), "memset dW");
+  if (cp.use) return MOLT_OK;
+  MOLT_CUDA(cudaMemsetAsync(w.dh32, 0, static_cast<size_t>(Tcap) * H * sizeof(float), s), "memset dh32");
+  if (!accumulate_dW) MOLT_CUDA(cudaMemsetAsync(dW_out, 0, static_cast<size_t>(V) * H * sizeof(float), s), "memset dW");
   return MOLT_OK;
 }
 
@@ -609,7 +607,7 @@ molt_status run_backward_chunk(const DeviceInfo* di, const ChunkPlan& cp, const 
   a.chunk_v = static_cast<int>(cp.chunk_v);
   a.buf_panels = static_cast<int>(cp.buf_panels);
   a.panel_rows = static_cast<int>(cp.panel_rows);
-  a.store_dw = cp.one_token_chunk && !accumulate_dW;
+  a.add_dw = accumulate_dW ? 1 : 0;
   a.max_t = static_cast<int>(cp.n_t);
   a.max_chunks = static_cast<int>(cp.max_chunks);
   a.ctl = w.ctl;
@@ -793,7 +791,8 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
   // the caller's stream waits for them before the backward, or on any early
   // return before the workspace is released
   ZeroJoin zj;
-  if (const SideLane* zl = side_lane(stream)) {
+  const ChunkPlan cp = chunk_plan(T, H, V);
+  if (const SideLane* zl = cp.use ? nullptr : side_lane(stream)) {
     MOLT_CUDA(cudaEventRecord(zl->fork, stream), "zero fork");
     MOLT_CUDA(cudaStreamWaitEvent(zl->side, zl->fork, 0), "zero fork");
     const molt_status zs = zero_backward_targets(w, T, H, V, det, dW_out, accumulate_dW, zl->side);
@@ -808,10 +807,8 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
     zj.pending = true;
     if (zs != MOLT_OK) return zs;
   }
-  MOLT_TRY(run_forward(di, hidden, tokens, mask, behavior_logp, adv, T, H, V, S, w, tm_h, tm_w, stream));
-  if (logp_out) MOLT_CUDA(cudaMemsetAsync(logp_out, 0, T * sizeof(float), stream), "memset logp");
-  if (entropy_out) MOLT_CUDA(cudaMemsetAsync(entropy_out, 0, T * sizeof(float), stream), "memset entropy");
-  if (token_loss_out) MOLT_CUDA(cudaMemsetAsync(token_loss_out, 0, T * sizeof(float), stream), "memset token loss");
+  MOLT_TRY(run_forward(di, hidden, tokens, mask, behavior_logp, adv, T, H, V, S, w, tm_h, tm_w, stream,
+                       ZeroRows{{logp_out, entropy_out, token_loss_out}}, cp.ctl_words()));
   ev_start(2, stream);
   if (opts) {
     MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
@@ -1048,9 +1045,8 @@ molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, c
   CUtensorMap tm_h, tm_w;
   MOLT_TRY(make_tmap(&tm_h, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w.h_p, Tcap, H, kBK, kTileM));
   MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W, V, H, kBK, 128));
-  MOLT_TRY(run_forward(di, hidden, tokens, mask, nullptr, nullptr, T, H, V, S, w, tm_h, tm_w, stream));
-  MOLT_CUDA(cudaMemsetAsync(logp_out, 0, T * sizeof(float), stream), "memset logp");
-  if (entropy_out) MOLT_CUDA(cudaMemsetAsync(entropy_out, 0, T * sizeof(float), stream), "memset entropy");
+  MOLT_TRY(run_forward(di, hidden, tokens, mask, nullptr, nullptr, T, H, V, S, w, tm_h, tm_w, stream,
+                       ZeroRows{{logp_out, entropy_out}}));
   ev_start(2, stream);
   MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
                          entropy_out, nullptr, nullptr, nullptr, di->status, stream),
@@ -1115,7 +1111,7 @@ molt_status molt_vp_partials(const uint16_t* hidden, const uint16_t* W_shard, co
   MOLT_TRY(make_tmap(&tm_h, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w.h_p, Tcap, H, kBK, kTileM));
   MOLT_TRY(make_tmap(&tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, W_shard, V_shard, H, kBK, 128));
   MOLT_TRY(run_forward(di, hidden, tokens, mask, nullptr, nullptr, T, H, V_shard, S, w, tm_h, tm_w, stream,
-                       static_cast<int>(v_begin)));
+                       ZeroRows{}, 0, static_cast<int>(v_begin)));
   ev_start(2, stream);
   MOLT_LAUNCH(launch_vp_local(static_cast<int>(T), static_cast<int>(Tcap), static_cast<int>(V_shard), S, w,
                               reinterpret_cast<float4*>(partials_out), stream),
@@ -1155,13 +1151,10 @@ molt_status molt_vp_loss(const float* partials, int n_shards, const float* behav
   Scratch sc;
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
-  MOLT_CUDA(cudaMemsetAsync(lse_out, 0, T * sizeof(float), stream), "memset lse");
-  MOLT_CUDA(cudaMemsetAsync(coef_out, 0, T * sizeof(float), stream), "memset coef");
-  if (logp_out) MOLT_CUDA(cudaMemsetAsync(logp_out, 0, T * sizeof(float), stream), "memset logp");
-  if (entropy_out) MOLT_CUDA(cudaMemsetAsync(entropy_out, 0, T * sizeof(float), stream), "memset entropy");
-  if (token_loss_out) MOLT_CUDA(cudaMemsetAsync(token_loss_out, 0, T * sizeof(float), stream), "memset token loss");
   ev_start(0, stream);
-  MOLT_LAUNCH(launch_compact(mask, static_cast<int>(T), w, stream), "compact");
+  MOLT_LAUNCH(launch_compact(mask, static_cast<int>(T), w,
+                             ZeroRows{{lse_out, coef_out, logp_out, entropy_out, token_loss_out}}, 0, stream),
+              "compact");
   ev_stop(0, stream);
   ev_start(2, stream);
   MOLT_LAUNCH(launch_vp_merge(static_cast<int>(T), static_cast<int>(Tcap), n_shards, denom, clip_lo, clip_hi,
@@ -1205,7 +1198,7 @@ molt_status molt_vp_backward(const uint16_t* hidden, const uint16_t* W_shard, co
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
   ev_start(2, stream);
-  MOLT_LAUNCH(launch_vp_live(static_cast<int>(T), coef, w, stream), "shard rows");
+  MOLT_LAUNCH(launch_vp_live(static_cast<int>(T), coef, w, chunk_plan(T, H, V_shard).ctl_words(), stream), "shard rows");
   MOLT_LAUNCH(launch_vp_gather(hidden, tokens, lse, coef, static_cast<int>(v_begin), static_cast<int>(H), w,
                                di->n_sm, stream),
               "shard gather");

@@ -12,10 +12,10 @@
 // products are then plain 256 x 256 tiles on CTA pairs (tcgen05 cta_group::2):
 //   Z    z = h W^T, M = 256 tokens, N = 256 vocab, K = H; the epilogue turns z
 //        into g and stores it to the chunk buffer
-//   dH   M = 256 tokens, N = 256 of H, K = the chunk's vocab; reduce-added into
-//        the fp32 dhidden accumulator
-//   dW   M = 256 vocab, N = 256 of H, K = the chunk's tokens; reduce-added into
-//        dW, or stored when the call has one token chunk
+//   dH   M = 256 tokens, N = 256 of H, K = the chunk's vocab; stored to the fp32
+//        dhidden accumulator by the first vocab chunk, reduce-added by the others
+//   dW   M = 256 vocab, N = 256 of H, K = the chunk's tokens; stored to dW by the
+//        first token chunk (unless the call adds to it), reduce-added by the others
 //
 // Why chunks.  Every unit that holds g in one cluster's memory (512 x 512 at
 // most) drains 4 H (Tu + Vu) bytes of fp32 partial sums for 6 Tu Vu H flops
@@ -91,12 +91,15 @@ struct __align__(16) Tile {
   int t0, v0;    // the chunk's first token and vocab tile
   int need;      // dH, dW: warps that store the chunk's g; Z: tiles that read the
                  // buffer's previous chunk (0: none)
-  int pad;
+  int first;     // dH, dW: warps that store the first contribution to this sum, which
+                 // the tile's own is added to (0: it is the first, or dW is added to
+                 // what the caller has there)
 };
 
 // The tile list, walked forwards by the claiming thread: claimed indices only grow.
 struct TileList {
   int n_rows, V, H;
+  bool add_dw;
   int n_t, n_v, n_h, n_tc, n_vc, n_chunks, nb;
   int total;                             // tiles in the list
   int step, base;                        // list step and its first index
@@ -111,9 +114,9 @@ struct TileList {
     n_v = (a.V + 255) / 256;
     n_h = (a.H + 255) / 256;
     n_tc = (n_t + a.chunk_t - 1) / a.chunk_t;
-    // no rows: with dW stored rather than added to, one chunk of no tokens whose
-    // dW tiles store zeros
-    if (n_t == 0 && a.store_dw) n_tc = 1;
+    // no rows: unless dW is added to, one chunk of no tokens whose dW tiles store zeros
+    add_dw = a.add_dw != 0;
+    if (n_t == 0 && !add_dw) n_tc = 1;
     n_vc = (n_v + a.chunk_v - 1) / a.chunk_v;
     n_chunks = n_tc * n_vc;
     total = n_t * n_v + (n_t * n_vc + n_v * n_tc) * n_h;   // Z + dH + dW tiles of all chunks
@@ -160,6 +163,7 @@ struct TileList {
     x.v = x.v0;
     x.h = 0;
     x.order = 0;
+    x.first = 0;
     uint32_t nz, nr;
     if (z) {
       i -= n_dh;
@@ -180,6 +184,7 @@ struct TileList {
       x.nk = (min(V, (c_v0 + c_cv) * 256) - c_v0 * 256 + kBK - 1) / kBK;
       x.h = i / c_ct;
       x.t += i % c_ct;
+      if (vc > 0) x.first = c_ct * n_h * (2 * kEpiWarps);
     } else {
       i -= n_dh + n_z;
       x.kind = kTileDW;
@@ -187,6 +192,7 @@ struct TileList {
       x.nk = (min(n_rows, (c_t0 + c_ct) * 256) - c_t0 * 256 + kBK - 1) / kBK;   // 0 without rows
       x.h = i / c_cv;
       x.v += i % c_cv;
+      if (tc > 0 && !add_dw) x.first = c_cv * n_h * (2 * kEpiWarps);
     }
   }
   // tiles of chunk c that write (z) or read its buffer
@@ -266,6 +272,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   auto mma_n = [&](int h) -> int { return H - h * 256 > 128 ? 256 : 128; };
   uint32_t* zdone = a.ctl + kChunkCtlHead;
   uint32_t* cdone = zdone + a.max_chunks;
+  // per token chunk (vocab chunk), at its first chunk: warps that have stored the
+  // first contributions to its dhidden (dW) rows
+  uint32_t* dh_first = cdone + a.max_chunks;
+  uint32_t* dw_first = dh_first + a.max_chunks;
+  const int n_vc = ((V + 255) / 256 + a.chunk_v - 1) / a.chunk_v;
 
   // the i-th tile for a reader of the slot ring; false at the end of the walk, also
   // after a wait that ran out.  Single threads give the slot back here, a warp's
@@ -295,6 +306,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     x.t0 = q[2].x;
     x.v0 = q[2].y;
     x.need = q[2].z;
+    x.first = q[2].w;
     return x.kind >= 0;
   };
 
@@ -443,7 +455,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         else
           x.kind = -1;
         const int4 q[3] = {make_int4(x.kind, x.chunk, x.buf, x.nk), make_int4(x.t, x.v, x.h, x.order),
-                           make_int4(x.t0, x.v0, x.need, 0)};
+                           make_int4(x.t0, x.v0, x.need, x.first)};
         const uint32_t own = smem_u32(&tile_sh[s]), peer = tile_peer0 + s * static_cast<uint32_t>(sizeof(Tile));
         const uint32_t peer_bar = jfull_peer0 + s * 8;
         mbar_arrive_expect_tx_cluster(peer_bar, sizeof(Tile));
@@ -468,24 +480,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (lane == 0) bulk_wait_group_read<0>();
       __syncwarp();
     };
-    // chunk whose zdone this warp still has to raise for its last Z tile, or -1: its
-    // stores are awaited when the warp would wait anyway, and at the latest after
-    // the next tile, so nothing that waits for them is held up
-    int z_pending = -1;
-    auto raise_z = [&]() {
-      if (z_pending < 0) return;
+    // counter that this warp still has to raise for its last tile's stores, or
+    // nullptr: they are awaited when the warp would wait anyway, and at the latest
+    // in the next tile, so nothing that waits for them is held up
+    uint32_t* pending = nullptr;
+    auto raise = [&]() {
+      if (pending == nullptr) return;
       if (lane == 0) {
         bulk_wait_group<0>();
         fence_proxy_async_global();
-        red_add_release_gpu(zdone + z_pending, 1u);
+        red_add_release_gpu(pending, 1u);
       }
       __syncwarp();
-      z_pending = -1;
+      pending = nullptr;
     };
+    // waits (bounded) until a counter that earlier tiles raise reaches `count`
+    auto wait_count = [&](const uint32_t* counter, int count) -> bool {
+      raise();
+      int good = 1;
+      if (lane == 0) {
+        good = turn_wait(counter, static_cast<uint32_t>(count), abort_flag, a.ctl + 1, a.err) ? 1 : 0;
+        fence_proxy_async_global();
+      }
+      return __shfl_sync(0xffffffffu, good, 0) != 0;
+    };
+    int seen_dh = -1, seen_dw = -1;   // last first chunks seen stored
     // the tile's products, in order of ji
     auto acc_full = [&](uint32_t ji) -> bool {
       const uint32_t bar = smem_u32(&accf_bar[ji & 1u]), ph = (ji >> 1) & 1u;
-      if (z_pending >= 0 && !__all_sync(0xffffffffu, mbar_test_wait(bar, ph))) raise_z();
+      if (pending != nullptr && !__all_sync(0xffffffffu, mbar_test_wait(bar, ph))) raise();
       const bool full = mbar_wait(bar, ph, abort_flag, a.err);
       tc_fence_after();
       return full;
@@ -517,16 +540,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int lx = in ? a.tok_p[row] - vbase : -1;
         const int nvalid = in ? V - vbase : 0;
         // the buffer's previous chunk must have been read
-        if (x.need > 0) {
-          raise_z();
-          int good = 1;
-          if (lane == 0) {
-            good = turn_wait(cdone + x.chunk - a.n_buf, static_cast<uint32_t>(x.need), abort_flag, a.ctl + 1, a.err) ? 1
-                                                                                                                   : 0;
-            fence_proxy_async_global();
-          }
-          if (!(ok = __shfl_sync(0xffffffffu, good, 0) != 0)) break;
-        }
+        if (x.need > 0 && !(ok = wait_count(cdone + x.chunk - a.n_buf, x.need))) break;
         if (!(ok = acc_full(ji))) break;
         const int p0 = (x.v - x.v0) * 4 + hf * 2;
         const int gy = (x.buf * a.buf_panels + p0) * a.panel_rows + (x.t - x.t0) * 256 + r0;
@@ -561,7 +575,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
           }
           if (c == 1) release_acc();
-          if (c == 0) raise_z();   // of the tile before, long stored
+          if (c == 0) raise();   // of the tile before, long stored
           box_free();
           const uint32_t rowp = box + lane * 128;
 #pragma unroll
@@ -575,7 +589,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             bulk_commit_group();
           }
         }
-        z_pending = x.chunk;
+        pending = zdone + x.chunk;
         continue;
       }
       const bool dh = x.kind == kTileDH;
@@ -587,20 +601,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const int y = (dh ? x.t : x.v) * 256 + r0;
       const bool rows_in = y < (dh ? n_rows : V);
       const CUtensorMap* map = dh ? &m.dh : &m.dw;
+      // the first contribution to a sum is stored, so nothing has to be zeroed
+      // before; the others are added once it is there: it was a tile of an earlier
+      // step, so the wait is a formality
+      const bool first = x.order == 0 && (dh || !a.add_dw);
       uint32_t* turn = nullptr;
       if (a.det_turns) {
-        const int n_h = (H + 255) / 256;
-        raise_z();
         // reproducible sums: the contributions to a slab take turns in chunk order
-        const int64_t tile = dh ? static_cast<int64_t>(x.t) * n_h + x.h
-                                : static_cast<int64_t>(a.max_t + x.v) * n_h + x.h;
+        const int n_h = (H + 255) / 256;
+        const int64_t tile = static_cast<int64_t>(dh ? x.t : a.max_t + x.v) * n_h + x.h;
         turn = a.det_turns + tile * (2 * kEpiWarps) + slab;
-        int good = 1;
-        if (lane == 0) {
-          good = turn_wait(turn, static_cast<uint32_t>(x.order), abort_flag, a.ctl + 1, a.err) ? 1 : 0;
-          fence_proxy_async_global();
+        if (!(ok = wait_count(turn, x.order))) break;
+      } else if (x.first > 0) {
+        const int c0 = dh ? x.chunk - x.order : x.chunk - x.order * n_vc;
+        int& seen = dh ? seen_dh : seen_dw;
+        if (seen != c0) {
+          if (!(ok = wait_count((dh ? dh_first : dw_first) + c0, x.first))) break;
+          seen = c0;
         }
-        if (!(ok = __shfl_sync(0xffffffffu, good, 0) != 0)) break;
       }
 #pragma unroll 1
       for (int s = 0; s < 4; ++s) {
@@ -613,13 +631,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           for (int j = 0; j < 32; ++j) v[j] = 0.f;
         }
         if (s == 3 || col + 32 >= w) release_acc();
-        if (s == 0) raise_z();
+        if (s == 0) raise();
         box_free();
         write_box32(box, lane, v);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0 && rows_in) {
-          if (!dh && a.store_dw)
+          if (first)
             tma_store_2d(map, box, x.h * 256 + col, y);
           else
             tma_reduce_add_2d(map, box, x.h * 256 + col, y);
@@ -627,7 +645,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (lane == 0) bulk_commit_group();
       }
       if (hf * 128 >= w) release_acc();   // no columns for this warp
-      raise_z();
+      raise();
+      if (turn == nullptr && first) pending = dh ? dh_first + x.chunk : dw_first + x.chunk;
       if (turn != nullptr) {
         if (lane == 0) {
           bulk_wait_group<0>();
@@ -637,7 +656,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         __syncwarp();
       }
     }
-    raise_z();
+    raise();
     if (lane == 0) bulk_wait_group<0>();
     __syncwarp();
   }

@@ -113,10 +113,10 @@ struct ChunkArgs {
   int n_buf;                 // chunk buffers (>= 2)
   int buf_panels;            // 64-column panels of one buffer
   int panel_rows;            // token rows of one panel (128 bytes each)
-  int store_dw;              // dW is stored, not added to (one token chunk)
+  int add_dw;                // the call adds to dW
   int max_t;                 // token tiles of the call's capacity
   int max_chunks;
-  uint32_t* ctl;             // zeroed: kChunkCtlHead words, then tiles stored and tiles read per chunk
+  uint32_t* ctl;             // zeroed: kChunkCtlHead words, then four counters per chunk
   uint32_t* det_turns;       // reproducible sums: zeroed [token tiles + vocab tiles, H tiles, 16] counters, or nullptr
   unsigned* err;
 };
@@ -151,7 +151,14 @@ cudaError_t launch_advantages(const float* rewards, const int32_t* gids, int n, 
                               float* out, unsigned* err, cudaStream_t s);
 cudaError_t launch_broadcast(const float* adv, const int32_t* rot, int n_resp, int T, float* out, cudaStream_t s);
 cudaError_t launch_mask_count(const uint8_t* mask, int64_t T, int64_t* out, cudaStream_t s);
-cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, cudaStream_t s);
+// fp32 outputs [T] that are 0 on masked rows (nullptr: none)
+struct ZeroRows {
+  static constexpr int kMax = 5;
+  float* out[kMax];
+};
+// the active rows; also zeroes z on the masked ones and the first ctl_words of ws.ctl
+cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, const ZeroRows& z, int64_t ctl_words,
+                           cudaStream_t s);
 // tok_shift is subtracted from every token (a vocabulary shard's first column)
 cudaError_t launch_gather(const uint16_t* hidden, const int32_t* tokens, const float* b, const float* adv, int T,
                           int Tcap, int H, const Workspace& ws, int n_sm, cudaStream_t s, int tok_shift = 0);
@@ -178,7 +185,7 @@ cudaError_t launch_vp_merge(int T, int Tcap, int n_shards, double denom, float c
                             const float4* parts, const float* b, const float* adv, const Workspace& ws,
                             float* lse_out, float* coef_out, float* logp_out, float* ent_out, float* tokloss_out,
                             unsigned* err, cudaStream_t s);
-cudaError_t launch_vp_live(int T, const float* coef, const Workspace& ws, cudaStream_t s);
+cudaError_t launch_vp_live(int T, const float* coef, const Workspace& ws, int64_t ctl_words, cudaStream_t s);
 cudaError_t launch_vp_gather(const uint16_t* hidden, const int32_t* tokens, const float* lse, const float* coef,
                              int tok_shift, int H, const Workspace& ws, int n_sm, cudaStream_t s);
 cudaError_t launch_vp_dh_out(const Workspace& ws, int T, int H, float* out, int n_sm, cudaStream_t s);

@@ -176,14 +176,23 @@ __device__ __forceinline__ int compact_rows(int n, Pred pred, Emit emit) {
 }
 
 // order-preserving list of active rows (mask != 0)
+// and, of the same block, the call's zeroing: the outputs of masked rows and the
+// backward's counters, which separate memsets cost a launch each
 __global__ void __launch_bounds__(1024) compact_kernel(const uint8_t* __restrict__ mask, int T,
                                                        int32_t* __restrict__ row_map, int32_t* __restrict__ pos,
-                                                       int32_t* __restrict__ counts) {
+                                                       int32_t* __restrict__ counts, ZeroRows z,
+                                                       uint32_t* __restrict__ ctl, int ctl_words) {
+  for (int i = threadIdx.x; i < ctl_words; i += blockDim.x) ctl[i] = 0u;
   const int total = compact_rows(
       T, [&](int t) { return mask == nullptr || mask[t] != 0; },
       [&](int t, bool live, int k) {
         if (live) row_map[k] = t;
         pos[t] = live ? k : -1;
+        if (!live) {
+#pragma unroll
+          for (int i = 0; i < ZeroRows::kMax; ++i)
+            if (z.out[i]) z.out[i][t] = 0.f;
+        }
       });
   if (threadIdx.x == 0) {
     counts[0] = total;
@@ -414,7 +423,9 @@ __global__ void __launch_bounds__(128) vp_merge_kernel(
 __global__ void __launch_bounds__(1024) vp_live_kernel(int T, const float* __restrict__ coef,
                                                        int32_t* __restrict__ counts, int32_t* __restrict__ tile_list,
                                                        int32_t* __restrict__ live_map,
-                                                       int32_t* __restrict__ live_of) {
+                                                       int32_t* __restrict__ live_of, uint32_t* __restrict__ ctl,
+                                                       int ctl_words) {
+  for (int i = threadIdx.x; i < ctl_words; i += blockDim.x) ctl[i] = 0u;
   const int total = compact_rows(
       T, [&](int t) { return coef[t] != 0.f; },
       [&](int t, bool live, int j) {
@@ -769,8 +780,10 @@ cudaError_t launch_mask_count(const uint8_t* mask, int64_t T, int64_t* out, cuda
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, cudaStream_t s) {
-  compact_kernel<<<1, 1024, 0, s>>>(mask, T, ws.row_map, ws.pos_of_row, ws.counts);
+cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, const ZeroRows& z, int64_t ctl_words,
+                           cudaStream_t s) {
+  compact_kernel<<<1, 1024, 0, s>>>(mask, T, ws.row_map, ws.pos_of_row, ws.counts, z, ws.ctl,
+                                    static_cast<int>(ctl_words));
   return cudaGetLastError();
 }
 
@@ -853,8 +866,9 @@ cudaError_t launch_vp_merge(int T, int Tcap, int n_shards, double denom, float c
   return cudaGetLastError();
 }
 
-cudaError_t launch_vp_live(int T, const float* coef, const Workspace& ws, cudaStream_t s) {
-  vp_live_kernel<<<1, 1024, 0, s>>>(T, coef, ws.counts, ws.tile_list, ws.live_map, ws.live_of);
+cudaError_t launch_vp_live(int T, const float* coef, const Workspace& ws, int64_t ctl_words, cudaStream_t s) {
+  vp_live_kernel<<<1, 1024, 0, s>>>(T, coef, ws.counts, ws.tile_list, ws.live_map, ws.live_of, ws.ctl,
+                                    static_cast<int>(ctl_words));
   return cudaGetLastError();
 }
 
