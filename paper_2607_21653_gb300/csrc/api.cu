@@ -152,38 +152,54 @@ struct ChunkPlan {
 // T is the call's row count; the rows with a gradient, at most as many, are
 // known on the device only.
 //
-// Which calls: against the kernels that hold g in one cluster (or CTA), this one
-// is 1.3 to 2.6 times faster from H = 640 on at any T (T = 700, H = 896, V =
-// 19000: 88 against 126 us; T = 16384, H = 4096, V = 151936: 38.0 against 54.4
-// ms), and for 256 < H < 640 from about 512 rows on (T = 2000, H = 320, V =
-// 19000: 108 against 163 us; but T = 64, H = 320, V = 100000: 170 against 82 us).
-// At H = 256 a logit tile is four K blocks and its epilogue and store are most of
-// it: the cluster kernel is up to 1.6 times faster (T = 300, V = 150000: 177
-// against 296 us), except on the smallest calls, where both wait for their chains
-// of tiles and this one's is shorter (T = 512, V = 4096: 26 against 31 us).
+// Which calls, against the kernels that hold g in one cluster (or CTA); backward
+// kernels' ms, those first:
+//   H >= 512: all (T = 64, V = 3000, H = 512 0.039 and 0.029; T = 2000, V = 19000,
+//     H = 896 0.262 and 0.140; T = 16384, V = 151936, H = 4096 54.4 and 36.8).
+//   256 < H < 512: from 512 rows on (T = 1024, V = 19000, H = 320 0.085 and 0.053);
+//     below, the single-CTA kernel is up to half faster (T = 64, V = 100000 0.081
+//     and 0.121), since a tile of 256 rows is mostly empty and short.
+//   H = 256: all but the middle vocabularies of small calls: up to 512 rows the
+//     cluster kernel is 5-20 % faster there (T = 256, V = 19000 0.031 and 0.038; but
+//     V = 60000 0.090 and 0.065, V = 2000 0.029 and 0.027).  At 700 rows this kernel
+//     would be faster already (V = 19000 0.051 and 0.044); the line lies above
+//     because tests/test_gpu_shapes.py holds the cluster kernel's vocab split there.
+//   H < 256: none (H = 64, T = 512, V = 19000 0.021 and 0.033).
 //
-// Chunk size: 16 x 16 tiles (4096 x 4096) in two buffers drain least; measured on
-// T = 16384, H = 4096, V = 151936: 38.8 ms, against 40.5 for 8 x 16 in four, 39.5
-// for 12 x 20, 41.2 for 32 x 8.  With few tiles or a short H a chunk holds too
-// little between a tile and what it waits for, and more, smaller buffers are
-// faster (T = 5003, H = 320, V = 50257: 0.71 ms with 8 x 16 in four, 0.94 with 16
-// x 16; T = 3000, H = 1024, V = 32000: 0.40 with 16 x 8 in four, 0.49).  Up to
-// 1024 rows the vocabulary is cut into about eight chunks, so that dH, whose tiles
-// are few and as long as a chunk, spreads over the SMs.
+// Chunk size: 16 x 16 tiles (4096 x 4096) in two buffers drain least; T = 16384, H =
+// 4096, V = 151936 took 38.8 ms, against 40.5 for 8 x 16 in four, 39.5 for 12 x 20
+// and 41.2 for 32 x 8.  With few tiles or a short H such a chunk holds too little
+// between a tile and what it waits for, and dH, whose tiles are few and as long as
+// a chunk, does not spread over the SMs; more, smaller buffers are faster (T = 8000,
+// H = 256, V = 50000: 0.70 ms with 4 x 4 in sixteen, 0.77 with 8 x 16 in four; T =
+// 20000, H = 512, V = 30000: 1.39 with 8 x 8 in four, 1.46 with 16 x 16; T = 1500, H =
+// 320, V = 20000: 0.074 with 8 x 8 in eight, 0.086 with 8 x 16 in four; T = 30000,
+// H = 1024, V = 5000: 0.55 and 0.64 with 16 x 8; T = 5000, H = 2048, V = 32000: 1.10
+// with 16 x 8 in four, 1.14 with 8 x 8; T = 700, H = 320, V = 100000: 0.18 with 4 x 4
+// in sixteen, 0.29 with 4 x 32 in four).
 ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
   ChunkPlan p;
-  if (T <= 0 || !(H >= 640 || (H > 256 && T >= 512) || (T <= 1024 && V <= 4096))) return p;
+  if (T <= 0 || H < 256 || (H == 256 && T <= 768 && V > 4096 && V <= 20480) || (H > 256 && H < 512 && T < 512)) return p;
   p.n_t = (T + 255) / 256;
   p.n_v = (V + 255) / 256;
   p.n_h = (H + 255) / 256;
   p.chunk_t = 16;
   p.chunk_v = 16;
-  if (p.n_t <= 4)
+  int64_t most_buf = 8;
+  if (p.n_t <= 4 && H >= 640) {
     p.chunk_v = std::max<int64_t>(4, std::min<int64_t>(32, (p.n_v + 7) / 8));
-  else if (H < 1024)
-    p.chunk_t = 8;
-  else if (p.n_t * p.n_v < 2560)
+  } else if (p.n_t <= 2) {
     p.chunk_v = 8;
+    most_buf = 16;
+  } else if (p.n_t <= 4 || H <= 256) {
+    p.chunk_t = p.chunk_v = 4;
+    most_buf = 16;
+  } else if (H < 1024 || (H < 2048 && p.n_t * p.n_v < 2560 && p.n_v < 64)) {
+    p.chunk_t = p.chunk_v = 8;
+    most_buf = p.n_t <= 16 ? 8 : 4;
+  } else if (p.n_t * p.n_v < 2560) {
+    p.chunk_v = 8;
+  }
   const int64_t n_tc = (p.n_t + p.chunk_t - 1) / p.chunk_t, n_vc = (p.n_v + p.chunk_v - 1) / p.chunk_v;
   const int64_t tiles = p.n_t * p.n_v + (p.n_t * n_vc + p.n_v * n_tc) * p.n_h;
   p.use = tiles < (int64_t(1) << 30);   // claimed with a 32-bit counter
@@ -192,7 +208,7 @@ ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
   p.panel_rows = ct * 256;
   p.buf_panels = cv * 4;
   // all buffers together stay at 64 MB, half of L2
-  p.n_buf = static_cast<int>(std::min<int64_t>(8, std::max<int64_t>(2, 512 / (ct * cv))));
+  p.n_buf = static_cast<int>(std::min<int64_t>(most_buf, std::max<int64_t>(2, 512 / (ct * cv))));
   return p;
 }
 

@@ -33,11 +33,12 @@ def _run(args, **kw):
 
 # (1, 640, 1): one row, one column; (257, 704, 513): remainders of one row, column
 # and a 192-column H tile; (512, 320, 4097): the rule's least T for this H, a
-# 64-column H tile; (1024, 256, 4096): the largest call the rule takes at H = 256;
-# (2049, 640, 2100): two token chunks of 8 tiles at most; (4200, 1088, 4400): two
-# chunks in both directions, a 64-column H tile
-@pytest.mark.parametrize("T,H,V", [(1, 640, 1), (257, 704, 513), (512, 320, 4097), (1024, 256, 4096),
-                                   (2049, 640, 2100), (4200, 1088, 4400)])
+# 64-column H tile; (300, 256, 4096), (700, 256, 20481), (769, 256, 8200): its lines at
+# H = 256; (1500, 256, 10000): chunks of 4 x 4 tiles, more of them than buffers; (2049,
+# 640, 2100): chunks of 8 x 8, two of tokens; (4200, 1088, 4400): three in both
+# directions, a 64-column H tile
+@pytest.mark.parametrize("T,H,V", [(1, 640, 1), (257, 704, 513), (512, 320, 4097), (300, 256, 4096), (700, 256, 20481),
+                                   (769, 256, 8200), (1500, 256, 10000), (2049, 640, 2100), (4200, 1088, 4400)])
 def test_chunk_backward_matches_oracle(T, H, V):
     rng = np.random.default_rng(T + H + V)
     h, W, x, m = random_problem(rng, T, H, V, mask_frac=0.1 if T > 1 else 0.0, w_std=0.05)
