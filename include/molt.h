@@ -21,11 +21,11 @@
  *     makes the call allocate and free it stream-ordered (cudaMallocAsync).
  *   - The library keeps no state between calls except cached device
  *     properties, the per-device status word, the kernel-launch counter, the
- *     no-allocation forward's fixed scratch array, and, for the loss call's
- *     vocabulary split and the zeroing of its backward targets, one side stream
- *     with fork, join and zeroed events per (device, caller stream), created on
- *     first use (at most 64, never while the
- *     caller's stream is being captured) and kept for the life of the process.
+ *     no-allocation forward's fixed scratch array, and, for loss calls that take
+ *     the cluster backward (short hidden sizes), one side stream with fork, join
+ *     and zeroed events per (device, caller stream), created on first use (at
+ *     most 64, never while the caller's stream is being captured) and kept for
+ *     the life of the process.
  *     It is safe to call from several threads on different streams with
  *     different workspaces; calls sharing a stream must come from one thread at
  *     a time (their launches would interleave on it).
@@ -186,14 +186,15 @@ molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, c
  * Outputs: loss_out (device fp32 scalar), dhidden_out, dW_out; optional
  * (may be NULL): logp_out [T], entropy_out [T], token_loss_out [T] (= m_t l_t),
  * stats_out (device molt_stats).
- * The [T,V] logits and gradients never reach global memory: each vocab tile is
- * recomputed on chip in the backward pass and fed to the dhidden / dW tensor-
- * core products from shared memory.
- * Streams: all work is ordered on `stream`.  Part of the backward, and the
- * zeroing of dW and of the fp32 dhidden accumulator (during the forward), may
- * run on an internal lowest-priority stream of the library (one per device and
- * caller stream, created on the first such call), forked from `stream` and
- * joined back to it with events before the call's later work, so nothing needs
+ * The [T,V] logits never reach global memory, and their gradient never exists as a
+ * whole: the backward recomputes it in chunks of at most 4096 x 4096, which pass
+ * from one tensor-core product to the next through a ring in the workspace that
+ * is at most 64 MB, half of L2 (short hidden sizes: through shared memory).
+ * Streams: all work is ordered on `stream`.  For short hidden sizes part of the
+ * backward, and the zeroing of dW and of the fp32 dhidden accumulator (during the
+ * forward), may run on an internal lowest-priority stream of the library (one per
+ * device and caller stream, created on the first such call), forked from `stream`
+ * and joined back to it with events before the call's later work, so nothing needs
  * to be synchronised by the caller.  The call can be captured into a CUDA graph;
  * the side stream is only used under capture if an earlier uncaptured call on
  * the same stream created it.
@@ -231,25 +232,25 @@ molt_status molt_policy_loss_fwd_bwd(const uint16_t* hidden, const uint16_t* W, 
  *                 0 <= gate_lo <= gate_hi (gate_hi may be +inf)
  *   deterministic 1: dW and dhidden are bitwise reproducible for the same inputs
  *                 (no paper counterpart).  The backward then fixes the order of
- *                 every partial-sum reduction: the partial products of a
- *                 512-token quad x 512-column vocabulary block are reduce-added
- *                 into dW in token-quad order and into dhidden in vocabulary
- *                 block order, each [32 x 128] slab waiting its turn on a
- *                 counter in the workspace.  The order does not depend on the
- *                 number C of clusters of four CTAs the backward runs (see
- *                 det_clusters).  The C clusters wait on one another, so they
- *                 must be resident together: if other work keeps SMs busy for
- *                 seconds, a wait gives up after about 4 s, the call's backward
- *                 returns early with dW and dhidden incomplete, and
- *                 molt_device_status reports MOLT_ERR_DEVICE_TIMEOUT
- *                 (MOLT_DEV_TIMEOUT bit); nothing hangs.  Needs H % 128 == 0
+ *                 every partial-sum reduction: the contributions to dW are added
+ *                 in token order and those to dhidden in vocabulary order, chunk by
+ *                 chunk (of up to 4096 x 4096; 512 x 512 blocks for short hidden
+ *                 sizes), each [32 x 128] slab waiting its turn on a counter in
+ *                 the workspace.  The order does not depend on the number of SMs
+ *                 the backward runs on (see det_clusters).  For short hidden sizes
+ *                 its clusters wait on one another and must be resident together.
+ *                 If other work keeps SMs busy for seconds, a wait gives up after
+ *                 about 4 s, the call's backward returns early with dW and dhidden
+ *                 incomplete, and molt_device_status reports
+ *                 MOLT_ERR_DEVICE_TIMEOUT (MOLT_DEV_TIMEOUT bit); nothing hangs.
+ *                 Needs H % 128 == 0
  *                 (MOLT_ERR_UNSUPPORTED_SHAPE otherwise) and the workspace of
  *                 molt_policy_loss_workspace_bytes_ex (the raster's plus the
  *                 counters).  0: reduce-adds in arrival order (results agree
  *                 to fp32 rounding).
  *   det_clusters  deterministic mode only: the number C of clusters to run, a
  *                 multiple of 4 from 4 up to the number that fit on the device
- *                 at once (36 on a GB300); 0 takes that maximum.  A caller that
+ *                 at once (36 on a GB300); 0 runs on all the SMs.  A caller that
  *                 shares the GPU with other work can leave SMs to it with a
  *                 smaller C.  The results are the same bits for every C.  Other
  *                 values return MOLT_ERR_INVALID_ARG.

@@ -444,9 +444,9 @@ molt_status get_scratch(Scratch& sc, void* ws, size_t ws_bytes, size_t need, cud
   return MOLT_OK;
 }
 
-// Side lanes of the loss call.  Clusters of four leave the SMs that cannot
-// hold a whole cluster idle (8 of 152 on a GB300); the single-CTA backward runs
-// there concurrently on a slice of the vocabulary.  The backward's reduce-add
+// Side lanes of the calls that take the cluster kernel.  Clusters of four leave the
+// SMs that cannot hold a whole cluster idle (8 of 152 on a GB300); the single-CTA
+// backward runs there concurrently on a slice of the vocabulary.  The reduce-add
 // targets are zeroed on the same lane while the forward runs (the memset
 // kernels fit beside the forward's one CTA per SM).  One low-priority side
 // stream and fork / join / zeroed events per (device, caller stream), created
@@ -847,6 +847,9 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
   MOLT_LAUNCH(launch_live_gather(static_cast<int>(H), with_ecoef, w, di->n_sm, stream), "live gather");
   ev_stop(2, stream);
   MOLT_CUDA(zj.join(), "zero join");
+  // the backward over chunks waits only for tiles claimed earlier, so unless the
+  // caller asked for a count it takes every pair of SMs (0), not whole clusters of four
+  if (cp.use && det && opts->det_clusters == 0) n_det = 0;
   MOLT_TRY(run_backward(di, W, T, H, V, w, det, n_det, with_ecoef, dW_out, accumulate_dW, zj.lane != nullptr, stream));
   ev_start(4, stream);
   MOLT_LAUNCH(launch_cast_dh(w, static_cast<int>(T), static_cast<int>(H), dhidden_out, di->n_sm, stream), "cast dh");

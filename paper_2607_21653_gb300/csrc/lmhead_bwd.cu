@@ -4,6 +4,9 @@
 //          (+ ecoef_t softmax(z_t)_v (z_tv - mu_t) with an entropy bonus)
 //   dH_t = sum_v g_tv W_v          dW_v = sum_t g_tv h_t
 //
+// Used for H = 64 and 192, for 256 < H < 512 with H % 128 == 64 below 512 rows (see
+// chunk_plan in api.cu), and beside the cluster kernel on the SMs no cluster can use.
+//
 // Neither the logits nor g touch global memory.  A work unit is one 128-row
 // tile of active tokens times one 256-column vocab chunk j (chunks counted from
 // vc_begin, so the kernel can take a slice of the vocabulary while the cluster

@@ -1,5 +1,9 @@
 // Backward pass of the fused LM-head + policy loss on clusters of four CTAs
-// (two tcgen05 CTA pairs), used when H is a multiple of 128.
+// (two tcgen05 CTA pairs), used for short hidden sizes that are multiples of 128
+// where the backward over chunks (lmhead_bwd_chunk.cu) is slower: H = 128, the middle
+// vocabularies of small calls at H = 256, and H = 384 below 512 rows (chunk_plan in
+// api.cu has the rule and the times).  g never leaves the cluster here, so a small
+// call needs no round trip through L2 between its products.
 //
 //   g_tv = coef_t (softmax(z_t)_v - [v == x_t]),  coef_t = m_t c_t / D   (Eq. 2)
 //          (+ ecoef_t softmax(z_t)_v (z_tv - mu_t) with an entropy bonus)
@@ -49,19 +53,13 @@
 // unit's Z_a stages fill the MMA issuer's wait for that hand-back.
 //
 // Operands stream through a ring of four 16 KB stages.  Every stage is a round
-// trip (the MMA frees it, the producer refills it from L2), and the ring's
-// bytes in flight over that latency set the rate at which operands arrive, so
-// the ring is cut fine: a logit stage holds K = 32 of h and W in the 64-byte
-// swizzle, a dH stage 64 vocab rows x 128 columns of W, a dW stage 64 token
-// rows x 128 columns of h.  The MMA issuer waits for operand stages about a
-// quarter of the time, yet no unit on the way is saturated: each SM's
-// interface to the crossbar is the busiest (about two thirds, mostly the
-// reduce-add payload at one cycle per 32-byte sector, the load requests at one
-// cycle each), which caps the kernel near 70 % of the tensor roofline, and the
-// rest is the latency of the unit's chain of dependencies.  More stages (a
-// fifth one paid for with smaller drain boxes, six with the drains issued from
-// registers) and multicasting the operands both pairs load did not make it
-// faster.
+// trip (the MMA frees it, the producer refills it from L2), so the ring is cut
+// fine: a logit stage holds K = 32 of h and W in the 64-byte swizzle, a dH stage 64
+// vocab rows x 128 columns of W, a dW stage 64 token rows x 128 columns of h.  On
+// long calls the fp32 drains of the 512 x 512 units bound the kernel: they share
+// each SM's path to L2 with the operand loads (1.1 PFLOP/s executed at H = 4096,
+// against 1.7 over chunks).  More stages, finer or coarser ones and multicasting the
+// operands both pairs load did not make it faster.
 //
 // Roles per CTA (320 threads): warp 0 TMA producer (each CTA loads its half of
 // every operand; bytes complete on the pair leader's barrier), warp 1 MMA issuer
