@@ -215,7 +215,7 @@ ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
 struct Layout {
   size_t counts, row_map, pos, tok_p, b_p, adv_p, h_p, part, zx, lse, coef, tile_list, red, dh32, turns, g, ctl;
   size_t lp_p, ent_p, ecoef, mu, gate_p;
-  size_t live_map, live_of, h_l, tok_l, lse_l, coef_l, ecoef_l, mu_l, total;
+  size_t live_of, h_l, tok_l, lse_l, coef_l, ecoef_l, mu_l, total;
 };
 
 constexpr size_t kNoRegion = ~size_t(0);   // a Layout region that is not allocated
@@ -272,7 +272,6 @@ Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = 
   L.ecoef = with_bwd ? take(Tcap * 4) : o;
   L.mu = with_bwd ? take(Tcap * 4) : o;
   L.gate_p = with_bwd ? take(Tcap) : o;
-  L.live_map = with_bwd ? take(Tcap * 4) : o;
   L.live_of = with_bwd ? take(Tcap * 4) : o;
   L.h_l = with_bwd ? take(Tcap * H * 2) : o;
   L.tok_l = with_bwd ? take(Tcap * 4) : o;
@@ -302,7 +301,6 @@ Layout vp_loss_layout(int64_t T) {
   L.coef = take(Tcap * 4);
   L.tile_list = take(ntile * 4);
   L.red = take(Tcap / kRedRows * kRedSlots * 8);
-  L.live_map = take(Tcap * 4);
   L.live_of = take(Tcap * 4);
   L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.dh32 = L.g = L.ctl = L.lp_p = L.ent_p = L.ecoef = L.mu = L.gate_p =
       L.h_l = L.tok_l = L.lse_l = L.coef_l = L.ecoef_l = L.mu_l = o;
@@ -326,7 +324,6 @@ Layout vp_backward_layout(int64_t T, int64_t H, int64_t V) {
   };
   L.counts = take(64);
   L.tile_list = take(ntile * 4);
-  L.live_map = take(Tcap * 4);
   L.live_of = take(Tcap * 4);
   L.h_l = take(Tcap * H * 2);
   L.tok_l = take(Tcap * 4);
@@ -368,7 +365,6 @@ Workspace carve(void* base, const Layout& L) {
   w.ecoef = reinterpret_cast<float*>(p + L.ecoef);
   w.mu = reinterpret_cast<float*>(p + L.mu);
   w.gate_p = p + L.gate_p;
-  w.live_map = reinterpret_cast<int32_t*>(p + L.live_map);
   w.live_of = reinterpret_cast<int32_t*>(p + L.live_of);
   w.h_l = reinterpret_cast<uint16_t*>(p + L.h_l);
   w.tok_l = reinterpret_cast<int32_t*>(p + L.tok_l);
@@ -548,10 +544,9 @@ molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int3
                         const ZeroRows& zero, int64_t ctl_words = 0, int tok_shift = 0) {
   const int64_t Tcap = round_tiles(T);
   ev_start(0, s);
-  MOLT_LAUNCH(launch_compact(mask, static_cast<int>(T), w, zero, ctl_words, s), "compact");
-  MOLT_LAUNCH(launch_gather(hidden, tokens, b, adv, static_cast<int>(T), static_cast<int>(Tcap), static_cast<int>(H),
-                          w, di->n_sm, s, tok_shift),
-            "gather");
+  MOLT_LAUNCH(launch_pack(mask, static_cast<int>(T), static_cast<int>(H), hidden, tokens, b, adv, tok_shift, w, zero,
+                          ctl_words, di->n_sm, s),
+              "pack");
   ev_stop(0, s);
   FwdArgs fa{};
   fa.tok_p = w.tok_p;
@@ -841,10 +836,9 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
   // rows whose gradient coefficient is 0 (masked out already; clipped, A = 0,
   // rejected) are left out of the backward
   const bool with_ecoef = opts && ex.entropy_coef != 0.f;
-  MOLT_LAUNCH(launch_finalize(static_cast<int>(Tcap), denom, with_ecoef, w, loss_out, stats_out, stats_ex_out,
-                              di->status, stream),
-              "finalize");
-  MOLT_LAUNCH(launch_live_gather(static_cast<int>(H), with_ecoef, w, di->n_sm, stream), "live gather");
+  MOLT_LAUNCH(launch_finish(static_cast<int>(H), cp.use ? kBK : kTileM, with_ecoef, denom, w, loss_out, stats_out, stats_ex_out, di->status,
+                            di->n_sm, stream),
+              "finish");
   ev_stop(2, stream);
   MOLT_CUDA(zj.join(), "zero join");
   // the backward over chunks waits only for tiles claimed earlier, so unless the
@@ -1171,18 +1165,16 @@ molt_status molt_vp_loss(const float* partials, int n_shards, const float* behav
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
   ev_start(0, stream);
-  MOLT_LAUNCH(launch_compact(mask, static_cast<int>(T), w,
-                             ZeroRows{{lse_out, coef_out, logp_out, entropy_out, token_loss_out}}, 0, stream),
-              "compact");
+  MOLT_LAUNCH(launch_pack(mask, static_cast<int>(T), 8, nullptr, nullptr, nullptr, nullptr, 0, w,
+                          ZeroRows{{lse_out, coef_out, logp_out, entropy_out, token_loss_out}}, 0, di->n_sm, stream),
+              "pack");
   ev_stop(0, stream);
   ev_start(2, stream);
   MOLT_LAUNCH(launch_vp_merge(static_cast<int>(T), static_cast<int>(Tcap), n_shards, denom, clip_lo, clip_hi,
                               reinterpret_cast<const float4*>(partials), behavior_logp, adv, w, lse_out, coef_out,
                               logp_out, entropy_out, token_loss_out, di->status, stream),
               "shard merge");
-  MOLT_LAUNCH(launch_finalize(static_cast<int>(Tcap), denom, false, w, loss_out, stats_out, nullptr, di->status,
-                              stream),
-              "finalize");
+  MOLT_LAUNCH(launch_finish(8, 0, false, denom, w, loss_out, stats_out, nullptr, di->status, di->n_sm, stream), "finish");
   ev_stop(2, stream);
   return MOLT_OK;
 }
@@ -1217,10 +1209,10 @@ molt_status molt_vp_backward(const uint16_t* hidden, const uint16_t* W_shard, co
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
   ev_start(2, stream);
-  MOLT_LAUNCH(launch_vp_live(static_cast<int>(T), coef, w, chunk_plan(T, H, V_shard).ctl_words(), stream), "shard rows");
-  MOLT_LAUNCH(launch_vp_gather(hidden, tokens, lse, coef, static_cast<int>(v_begin), static_cast<int>(H), w,
-                               di->n_sm, stream),
-              "shard gather");
+  const ChunkPlan cp = chunk_plan(T, H, V_shard);
+  MOLT_LAUNCH(launch_vp_pack(static_cast<int>(T), static_cast<int>(H), cp.use ? kBK : kTileM, hidden, tokens, lse, coef,
+                             static_cast<int>(v_begin), w, cp.ctl_words(), di->n_sm, stream),
+              "shard rows");
   ev_stop(2, stream);
   MOLT_TRY(
       run_backward(di, W_shard, T, H, V_shard, w, false, 0, false, dW_shard_out, accumulate_dW, false, stream));

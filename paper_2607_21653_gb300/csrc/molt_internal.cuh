@@ -24,7 +24,7 @@ struct Workspace {
   int32_t* tok_p;       // [Tcap] packed tokens
   float* b_p;           // [Tcap] packed behaviour log-probs
   float* adv_p;         // [Tcap] packed advantages
-  uint16_t* h_p;        // [Tcap, H] packed hidden rows (bf16 bits), rows >= n zeroed
+  uint16_t* h_p;        // [Tcap, H] packed hidden rows (bf16 bits)
   float4* part;         // [S, Tcap] per-split (max, sum exp, sum exp*(z-max), -)
   float* zx;            // [Tcap] target logit
   float* lse;           // [Tcap]
@@ -33,9 +33,8 @@ struct Workspace {
   double* red;          // [Tcap/kRedRows, kRedSlots] partial sums of kRedRows packed rows
   float* dh32;          // [Tcap, H] fp32 dhidden accumulator, by backward row (loss call only)
   // rows with a nonzero gradient coefficient, packed again (loss call only)
-  int32_t* live_map;    // [Tcap] backward row -> packed row
   int32_t* live_of;     // [Tcap] packed row -> backward row or -1
-  uint16_t* h_l;        // [Tcap, H] their hidden rows (bf16 bits), rows >= n_live zeroed
+  uint16_t* h_l;        // [Tcap, H] their hidden rows (bf16 bits), zero rows up to a multiple of the pad
   int32_t* tok_l;       // [Tcap] their tokens
   float* lse_l;         // [Tcap]
   float* coef_l;        // [Tcap] m c / D
@@ -156,20 +155,20 @@ struct ZeroRows {
   static constexpr int kMax = 5;
   float* out[kMax];
 };
-// the active rows; also zeroes z on the masked ones and the first ctl_words of ws.ctl
-cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, const ZeroRows& z, int64_t ctl_words,
-                           cudaStream_t s);
-// tok_shift is subtracted from every token (a vocabulary shard's first column)
-cudaError_t launch_gather(const uint16_t* hidden, const int32_t* tokens, const float* b, const float* adv, int T,
-                          int Tcap, int H, const Workspace& ws, int n_sm, cudaStream_t s, int tok_shift = 0);
+// the active rows packed, with hidden (or nullptr: the maps only) also their hidden
+// rows, tokens (minus tok_shift, a vocabulary shard's first column), b and adv; zeroes
+// z on the masked rows and the first ctl_words of ws.ctl
+cudaError_t launch_pack(const uint8_t* mask, int T, int H, const uint16_t* hidden, const int32_t* tokens, const float* b,
+                        const float* adv, int tok_shift, const Workspace& ws, const ZeroRows& z, int64_t ctl_words,
+                        int n_sm, cudaStream_t s);
 // lp_p, ent_p: packed log-probs and entropies for the extended objective, or nullptr
 cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
                          const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, float* lp_p,
                          float* ent_p, unsigned* err, cudaStream_t s);
-cudaError_t launch_finalize(int Tcap, double denom, bool with_ecoef, const Workspace& ws, float* loss_out,
-                            void* stats_out, void* stats_ex_out, unsigned* err, cudaStream_t s);
-// the rows with a gradient (finalize's list) packed into whole tiles for the backward
-cudaError_t launch_live_gather(int H, bool with_ecoef, const Workspace& ws, int n_sm, cudaStream_t s);
+// the loss and stats, and the list of the rows with a gradient, with pad > 0 packed
+// for the backward and padded with zero rows to a multiple of it
+cudaError_t launch_finish(int H, int pad, bool with_ecoef, double denom, const Workspace& ws, float* loss_out,
+                          void* stats_out, void* stats_ex_out, unsigned* err, int n_sm, cudaStream_t s);
 // extended objective: packed stats -> sequence gate -> loss rows
 cudaError_t launch_seq_gate(int T, int Tcap, const LossEx& ex, const Workspace& ws, unsigned* err, cudaStream_t s);
 cudaError_t launch_loss_rows_ex(int Tcap, double denom, float clip_lo, float clip_hi, const LossEx& ex,
@@ -185,9 +184,9 @@ cudaError_t launch_vp_merge(int T, int Tcap, int n_shards, double denom, float c
                             const float4* parts, const float* b, const float* adv, const Workspace& ws,
                             float* lse_out, float* coef_out, float* logp_out, float* ent_out, float* tokloss_out,
                             unsigned* err, cudaStream_t s);
-cudaError_t launch_vp_live(int T, const float* coef, const Workspace& ws, int64_t ctl_words, cudaStream_t s);
-cudaError_t launch_vp_gather(const uint16_t* hidden, const int32_t* tokens, const float* lse, const float* coef,
-                             int tok_shift, int H, const Workspace& ws, int n_sm, cudaStream_t s);
+cudaError_t launch_vp_pack(int T, int H, int pad, const uint16_t* hidden, const int32_t* tokens, const float* lse,
+                           const float* coef, int tok_shift, const Workspace& ws, int64_t ctl_words, int n_sm,
+                           cudaStream_t s);
 cudaError_t launch_vp_dh_out(const Workspace& ws, int T, int H, float* out, int n_sm, cudaStream_t s);
 
 // lmhead_fwd.cu

@@ -144,93 +144,122 @@ __global__ void mask_count_kernel(const uint8_t* __restrict__ mask, int64_t T,
   }
 }
 
-// Order-preserving compaction of rows [0, n) by one block of 1024 threads: every
-// row k gets emit(k, live, its index among the live ones).  Each warp takes a
-// contiguous stretch, 32 neighbouring rows at a time (a ballot counts them), so
-// loads and stores are whole lines; pred is evaluated twice.  Returns the count.
-template <class Pred, class Emit>
-__device__ __forceinline__ int compact_rows(int n, Pred pred, Emit emit) {
-  __shared__ int wsum[32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int per = ((n + 31) / 32 + 31) / 32 * 32;
-  const int k0 = w * per, k1 = min(n, k0 + per);
-  int c = 0;
-#pragma unroll 4
-  for (int k = k0 + lane; k - lane < k1; k += 32) c += __popc(__ballot_sync(0xffffffffu, k < k1 && pred(k)));
-  if (lane == 0) wsum[w] = c;
+// ---------------------------------------------------------------------------
+// Order-preserving packing.  A grid of kPackThreads-thread blocks splits the rows
+// evenly; each block counts the live rows before its own (a vectorised scan of the
+// flags up to there, a few us at most: they sit in L2), so the count, the maps and
+// the copies are one launch.  Before, one block compacted and a second kernel
+// copied: 4 us more on the smallest call, 13 of 46 at T = 32768.
+// ---------------------------------------------------------------------------
+constexpr int kPackThreads = 256;
+
+__device__ __forceinline__ int block_sum(int v) {
+  __shared__ int ws[kPackThreads / 32];
+  v = __reduce_add_sync(0xffffffffu, v);
   __syncthreads();
-  int before = 0, total = 0;
-  {
-    const int x = wsum[lane];
-    before = __reduce_add_sync(0xffffffffu, lane < w ? x : 0);
-    total = __reduce_add_sync(0xffffffffu, x);
-  }
-#pragma unroll 4
-  for (int k = k0 + lane; k - lane < k1; k += 32) {
-    const bool live = k < k1 && pred(k);
-    const unsigned m = __ballot_sync(0xffffffffu, live);
-    if (k < k1) emit(k, live, before + __popc(m & ((1u << lane) - 1u)));
-    before += __popc(m);
-  }
-  return total;
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int t = 0;
+#pragma unroll
+  for (int i = 0; i < kPackThreads / 32; ++i) t += ws[i];
+  return t;
 }
 
-// order-preserving list of active rows (mask != 0)
-// and, of the same block, the call's zeroing: the outputs of masked rows and the
-// backward's counters, which separate memsets cost a launch each
-__global__ void __launch_bounds__(1024) compact_kernel(const uint8_t* __restrict__ mask, int T,
-                                                       int32_t* __restrict__ row_map, int32_t* __restrict__ pos,
-                                                       int32_t* __restrict__ counts, ZeroRows z,
-                                                       uint32_t* __restrict__ ctl, int ctl_words) {
-  for (int i = threadIdx.x; i < ctl_words; i += blockDim.x) ctl[i] = 0u;
-  const int total = compact_rows(
-      T, [&](int t) { return mask == nullptr || mask[t] != 0; },
+// nonzero bytes of m[0, n), by the whole block
+__device__ __forceinline__ int count_bytes(const uint8_t* __restrict__ m, int n) {
+  const int head = min(n, static_cast<int>((16 - (reinterpret_cast<uintptr_t>(m) & 15)) & 15));
+  const int nvec = (n - head) / 16;
+  const uint4* v = reinterpret_cast<const uint4*>(m + head);
+  auto word = [](uint32_t w) { return __popc((((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w) & 0x80808080u); };
+  int c = 0;
+  for (int i = threadIdx.x; i < head; i += kPackThreads) c += m[i] ? 1 : 0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < nvec; i += kPackThreads) {
+    const uint4 x = v[i];
+    c += word(x.x) + word(x.y) + word(x.z) + word(x.w);
+  }
+  for (int i = head + 16 * nvec + threadIdx.x; i < n; i += kPackThreads) c += m[i] ? 1 : 0;
+  return block_sum(c);
+}
+
+// The block's share of rows [0, n), 256 at a time: row(k, live, j) for every row k
+// (j its index among the live ones, `before` of which precede the share), then the
+// live rows' hidden rows copied from src row k to dst row j (src nullptr: none).
+// Returns the number of live rows up to the end of the share.
+template <class Live, class Row>
+__device__ __forceinline__ int pack_rows(int k0, int k1, int before, int H, const uint16_t* __restrict__ src,
+                                         uint16_t* __restrict__ dst, Live live_of_row, Row row) {
+  __shared__ int wsum[kPackThreads / 32];
+  __shared__ int list[kPackThreads];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int vpr = H / 8;   // 16-byte vectors per row
+  for (int base = k0; base < k1; base += kPackThreads) {
+    const int k = base + threadIdx.x;
+    const bool live = k < k1 && live_of_row(k);
+    const unsigned m = __ballot_sync(0xffffffffu, live);
+    __syncthreads();
+    if (lane == 0) wsum[w] = __popc(m);
+    __syncthreads();
+    int pre = 0, cnt = 0;
+#pragma unroll
+    for (int i = 0; i < kPackThreads / 32; ++i) {
+      pre += i < w ? wsum[i] : 0;
+      cnt += wsum[i];
+    }
+    const int j = pre + __popc(m & ((1u << lane) - 1u));
+    if (live) list[j] = k;
+    if (k < k1) row(k, live, before + j);
+    __syncthreads();
+    if (src != nullptr) {
+#pragma unroll 4
+      for (int i = threadIdx.x; i < cnt * vpr; i += kPackThreads) {
+        const int q = i / vpr, v = i - q * vpr;
+        reinterpret_cast<uint4*>(dst + static_cast<int64_t>(before + q) * H)[v] =
+            reinterpret_cast<const uint4*>(src + static_cast<int64_t>(list[q]) * H)[v];
+      }
+    }
+    before += cnt;
+  }
+  return before;
+}
+
+// The active rows (mask != 0) packed: maps, and with `hidden` their hidden rows,
+// tokens, behaviour log-probs and advantages.  (Rows past the last one stay as they
+// are: the forward's products are independent by row.)  Also the call's zeroing:
+// the outputs of masked rows and the backward's counters, which separate memsets
+// cost a launch each.
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(
+    const uint8_t* __restrict__ mask, int T, int H, const uint16_t* __restrict__ hidden,
+    const int32_t* __restrict__ tokens, const float* __restrict__ b, const float* __restrict__ adv, int tok_shift,
+    int32_t* __restrict__ row_map, int32_t* __restrict__ pos, int32_t* __restrict__ counts,
+    uint16_t* __restrict__ h_p, int32_t* __restrict__ tok_p, float* __restrict__ b_p, float* __restrict__ adv_p,
+    ZeroRows z, uint32_t* __restrict__ ctl, int ctl_words) {
+  for (int i = blockIdx.x * kPackThreads + threadIdx.x; i < ctl_words; i += gridDim.x * kPackThreads) ctl[i] = 0u;
+  const int share = (T + gridDim.x - 1) / gridDim.x;
+  const int64_t first = static_cast<int64_t>(blockIdx.x) * share;
+  if (first >= T) return;
+  const int t0 = static_cast<int>(first), t1 = min(T, t0 + share);
+  const int before = mask == nullptr ? t0 : count_bytes(mask, t0);
+  const int total = pack_rows(
+      t0, t1, before, H, hidden, h_p, [&](int t) { return mask == nullptr || mask[t] != 0; },
       [&](int t, bool live, int k) {
-        if (live) row_map[k] = t;
         pos[t] = live ? k : -1;
-        if (!live) {
+        if (live) {
+          row_map[k] = t;
+          if (tokens) tok_p[k] = tokens[t] - tok_shift;
+          if (b) b_p[k] = b[t];
+          if (adv) adv_p[k] = adv[t];
+        } else {
 #pragma unroll
           for (int i = 0; i < ZeroRows::kMax; ++i)
             if (z.out[i]) z.out[i][t] = 0.f;
         }
       });
-  if (threadIdx.x == 0) {
+  if (t1 == T && threadIdx.x == 0) {
     counts[0] = total;
     counts[1] = 0;
     counts[2] = 0;
     counts[4] = 0;
-  }
-}
-
-// packed copies of the active rows; rows in [n, round_up(n,128)) are zeroed so
-// that the last tile holds finite values
-__global__ void gather_kernel(const uint16_t* __restrict__ hidden, const int32_t* __restrict__ tokens,
-                              const float* __restrict__ b, const float* __restrict__ adv, int tok_shift, int Tcap,
-                              int H,
-                              const int32_t* __restrict__ row_map, const int32_t* __restrict__ counts,
-                              uint16_t* __restrict__ h_p, int32_t* __restrict__ tok_p, float* __restrict__ b_p,
-                              float* __restrict__ adv_p) {
-  const int n = counts[0];
-  const int nz = min(Tcap, ((n + kTileM - 1) / kTileM) * kTileM);
-  const int vpr = H / 8;   // 16-byte vectors per row
-  const int64_t total = (int64_t)nz * vpr;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int k = (int)(i / vpr), v = (int)(i - (int64_t)k * vpr);
-    uint4 val = make_uint4(0, 0, 0, 0);
-    if (k < n) {
-      const int t = row_map[k];
-      val = reinterpret_cast<const uint4*>(hidden + (int64_t)t * H)[v];
-      if (v == 0) {
-        tok_p[k] = tokens[t] - tok_shift;
-        if (b_p) b_p[k] = b[t];
-        if (adv_p) adv_p[k] = adv[t];
-      }
-    } else if (v == 0) {
-      tok_p[k] = 0;
-      if (b_p) b_p[k] = 0.f;
-      if (adv_p) adv_p[k] = 0.f;
-    }
-    reinterpret_cast<uint4*>(h_p + (int64_t)k * H)[v] = val;
   }
 }
 
@@ -417,31 +446,6 @@ __global__ void __launch_bounds__(128) vp_merge_kernel(
   if (k / kRedRows * kRedRows < n) warp_partials(act, rl, ent, 0.f, 0, red + (int64_t)(k / kRedRows) * kRedSlots);
 }
 
-// The rows of one shard's backward: those with a gradient coefficient (coef
-// from vp_merge_kernel, original order; masked and clipped rows have 0), in
-// order.  One block; as finalize_kernel's list.
-__global__ void __launch_bounds__(1024) vp_live_kernel(int T, const float* __restrict__ coef,
-                                                       int32_t* __restrict__ counts, int32_t* __restrict__ tile_list,
-                                                       int32_t* __restrict__ live_map,
-                                                       int32_t* __restrict__ live_of, uint32_t* __restrict__ ctl,
-                                                       int ctl_words) {
-  for (int i = threadIdx.x; i < ctl_words; i += blockDim.x) ctl[i] = 0u;
-  const int total = compact_rows(
-      T, [&](int t) { return coef[t] != 0.f; },
-      [&](int t, bool live, int j) {
-        if (live) live_map[j] = t;
-        live_of[t] = live ? j : -1;
-      });
-  const int n_lt = (total + kTileM - 1) / kTileM;
-  for (int b = threadIdx.x; b < n_lt; b += blockDim.x) tile_list[b] = b;
-  if (threadIdx.x == 0) {
-    counts[0] = total;
-    counts[1] = n_lt;
-    counts[2] = 0;
-    counts[3] = total;
-  }
-}
-
 // one shard's dhidden contribution in the original row order, fp32: the
 // accumulator row of t's backward row, 0 for rows without a gradient
 __global__ void vp_dh_out_kernel(const float* __restrict__ dh32, const int32_t* __restrict__ live_of, int T, int H,
@@ -578,128 +582,112 @@ struct StatsExDev {
 };
 constexpr int kFinSlots = 8;
 
-// fixed-order reduction of the per-tile partials, the loss scalar and the
-// stats; then the order-preserving list of the packed rows whose gradient
-// coefficient is nonzero (coef, or ecoef with an entropy bonus): the rows the
-// backward processes, packed again by live_gather_kernel into whole tiles
-__global__ void __launch_bounds__(1024) finalize_kernel(double denom, int32_t* __restrict__ counts,
-                                                        int32_t* __restrict__ tile_list,
-                                                        const double* __restrict__ red, float* __restrict__ loss_out,
-                                                        StatsDev* __restrict__ stats, StatsExDev* __restrict__ stats_ex,
-                                                        const float* __restrict__ coef,
-                                                        const float* __restrict__ ecoef,
-                                                        int32_t* __restrict__ live_map,
-                                                        int32_t* __restrict__ live_of, unsigned* err) {
-  __shared__ double sh[kFinSlots][4];
-  const int n = counts[0];
+// fixed-order reduction of the rows' partial sums, the loss scalar and the stats;
+// by one block of kPackThreads threads, a warp to each slot
+__device__ __forceinline__ void reduce_loss(int n, double denom, const int32_t* __restrict__ counts,
+                                            const double* __restrict__ red, float* __restrict__ loss_out,
+                                            StatsDev* __restrict__ stats, StatsExDev* __restrict__ stats_ex,
+                                            unsigned* err) {
+  static_assert(kFinSlots == kPackThreads / 32, "a warp to each slot");
+  __shared__ double tot[kFinSlots];
   const int n_rt = (n + kRedRows - 1) / kRedRows;
-  // four warps to a slot, then thread 0 over their results: a fixed order
-  {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = w >> 2;
-    double a = 0.0;
-#pragma unroll 4
-    for (int b = (w & 3) * 32 + lane; b < n_rt; b += 128) {
-      const double x = red[(int64_t)b * kRedSlots + q];
-      a = (q == 3) ? fmax(a, x) : a + x;
-    }
-    a = (q == 3) ? warp_max(a) : warp_sum(a);
-    if (lane == 0) sh[q][w & 3] = a;
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  double a = 0.0;
+#pragma unroll 8
+  for (int b = lane; b < n_rt; b += 32) {
+    const double x = red[(int64_t)b * kRedSlots + q];
+    a = (q == 3) ? fmax(a, x) : a + x;
   }
+  a = (q == 3) ? warp_max(a) : warp_sum(a);
+  if (lane == 0) tot[q] = a;
   __syncthreads();
+  if (threadIdx.x != 0) return;
   const double D = denom > 0.0 ? denom : static_cast<double>(n);
-  if (threadIdx.x == 0) {
-    double tot[kFinSlots];
+  if (!(D > 0.0)) atomicOr(err, kDevErrZeroDenom);
+  const double loss = D > 0.0 ? tot[0] / D : 0.0;
+  if (loss_out) *loss_out = static_cast<float>(loss);
+  StatsDev* st[2] = {stats, stats_ex ? &stats_ex->base : nullptr};
 #pragma unroll
-    for (int q = 0; q < kFinSlots; ++q)
-      tot[q] = (q == 3) ? fmax(fmax(sh[q][0], sh[q][1]), fmax(sh[q][2], sh[q][3]))
-                        : (sh[q][0] + sh[q][1]) + (sh[q][2] + sh[q][3]);
-    if (!(D > 0.0)) atomicOr(err, kDevErrZeroDenom);
-    const double loss = D > 0.0 ? tot[0] / D : 0.0;
-    if (loss_out) *loss_out = static_cast<float>(loss);
-    if (stats) {
-      stats->denom = D;
-      stats->loss = loss;
-      stats->sum_ratio = tot[1];
-      stats->sum_entropy = tot[2];
-      stats->max_abs_log_ratio = tot[3];
-      stats->n_active = n;
-      stats->n_clip_low = static_cast<long long>(tot[4]);
-      stats->n_clip_high = static_cast<long long>(tot[5]);
-    }
-    if (stats_ex) {
-      StatsDev& b = stats_ex->base;
-      b.denom = D;
-      b.loss = loss;
-      b.sum_ratio = tot[1];
-      b.sum_entropy = tot[2];
-      b.max_abs_log_ratio = tot[3];
-      b.n_active = n;
-      b.n_clip_low = static_cast<long long>(tot[4]);
-      b.n_clip_high = static_cast<long long>(tot[5]);
-      stats_ex->sum_kl = tot[6];
-      stats_ex->n_tokens_rejected = static_cast<long long>(tot[7]);
-      stats_ex->n_seq_rejected = counts[2];
-    }
+  for (int i = 0; i < 2; ++i) {
+    if (!st[i]) continue;
+    st[i]->denom = D;
+    st[i]->loss = loss;
+    st[i]->sum_ratio = tot[1];
+    st[i]->sum_entropy = tot[2];
+    st[i]->max_abs_log_ratio = tot[3];
+    st[i]->n_active = n;
+    st[i]->n_clip_low = static_cast<long long>(tot[4]);
+    st[i]->n_clip_high = static_cast<long long>(tot[5]);
   }
-  // compact the rows with a gradient (order preserving)
-  const int total = compact_rows(
-      n, [&](int k) { return coef[k] != 0.f || (ecoef != nullptr && ecoef[k] != 0.f); },
-      [&](int k, bool live, int j) {
-        if (live) live_map[j] = k;
-        live_of[k] = live ? j : -1;
-      });
+  if (stats_ex) {
+    stats_ex->sum_kl = tot[6];
+    stats_ex->n_tokens_rejected = static_cast<long long>(tot[7]);
+    stats_ex->n_seq_rejected = counts[2];
+  }
+}
+
+// Packs the rows whose gradient coefficient is nonzero (coef, or ecoef with an
+// entropy bonus), the rows the backward processes, into whole tiles of 128: with
+// `src` their hidden rows, tokens, lse, m c / D and, with an entropy bonus, its
+// coefficient and mu; rows in [n_live, round_up(n_live, pad)) are zeroed, which the
+// backward's products read with them (64 over chunks, 128 else; the last block does
+// it alone: 127 rows of H = 5120 took 10 us).  n_rows < 0: rows are the packed
+// active ones and the first block also reduces the loss.  Writes counts[1] (tiles)
+// and counts[3] (rows), and for a shard's backward zeroes the chunk counters.
+__global__ void __launch_bounds__(kPackThreads) finish_kernel(
+    int n_rows, int pad, double denom, int32_t* __restrict__ counts, int32_t* __restrict__ tile_list,
+    const double* __restrict__ red, float* __restrict__ loss_out, StatsDev* __restrict__ stats,
+    StatsExDev* __restrict__ stats_ex, int H, int tok_shift, const uint16_t* __restrict__ src,
+    const int32_t* __restrict__ tok, const float* __restrict__ lse, const float* __restrict__ coef,
+    const float* __restrict__ ecoef, const float* __restrict__ mu, int32_t* __restrict__ live_of,
+    uint16_t* __restrict__ h_l, int32_t* __restrict__ tok_l, float* __restrict__ lse_l, float* __restrict__ coef_l,
+    float* __restrict__ ecoef_l, float* __restrict__ mu_l, uint32_t* __restrict__ ctl, int ctl_words, unsigned* err) {
+  for (int i = blockIdx.x * kPackThreads + threadIdx.x; i < ctl_words; i += gridDim.x * kPackThreads) ctl[i] = 0u;
+  const int n = n_rows < 0 ? counts[0] : n_rows;
+  if (n_rows < 0 && blockIdx.x == 0) reduce_loss(n, denom, counts, red, loss_out, stats, stats_ex, err);
+  const int share = (n + gridDim.x - 1) / gridDim.x;
+  const int64_t first = static_cast<int64_t>(blockIdx.x) * share;
+  if (first >= n && !(n == 0 && blockIdx.x == 0)) return;
+  const int k0 = static_cast<int>(first), k1 = min(n, k0 + share);
+  auto live = [&](int k) { return coef[k] != 0.f || (ecoef != nullptr && ecoef[k] != 0.f); };
+  int c = 0;
+#pragma unroll 8
+  for (int k = threadIdx.x; k < k0; k += kPackThreads) c += live(k) ? 1 : 0;
+  const int total = pack_rows(k0, k1, block_sum(c), H, src, h_l, live, [&](int k, bool is_live, int j) {
+    live_of[k] = is_live ? j : -1;
+    if (is_live && src != nullptr) {
+      tok_l[j] = tok[k] - tok_shift;
+      lse_l[j] = lse[k];
+      coef_l[j] = coef[k];
+      if (ecoef) {
+        ecoef_l[j] = ecoef[k];
+        mu_l[j] = mu[k];
+      }
+    }
+  });
+  if (k1 != n) return;
   const int n_lt = (total + kTileM - 1) / kTileM;
-  for (int b = threadIdx.x; b < n_lt; b += blockDim.x) tile_list[b] = b;
+  for (int b = threadIdx.x; b < n_lt; b += kPackThreads) tile_list[b] = b;
   if (threadIdx.x == 0) {
     counts[1] = n_lt;
     counts[3] = total;
     if (stats) stats->n_grad_rows = total;
     if (stats_ex) stats_ex->base.n_grad_rows = total;
   }
-}
-
-// packed copies of the rows with a gradient (live_map from finalize_kernel):
-// hidden row, token, lse, m c / D and, with an entropy bonus, its coefficient
-// and mu; rows in [n_live, round_up(n_live, 128)) are zeroed so that the last
-// tile holds finite values and no gradient
-__global__ void live_gather_kernel(int H, int tok_shift, const int32_t* __restrict__ counts,
-                                   const int32_t* __restrict__ live_map,
-                                   const uint16_t* __restrict__ h_p, const int32_t* __restrict__ tok_p,
-                                   const float* __restrict__ lse, const float* __restrict__ coef,
-                                   const float* __restrict__ ecoef, const float* __restrict__ mu,
-                                   uint16_t* __restrict__ h_l, int32_t* __restrict__ tok_l,
-                                   float* __restrict__ lse_l, float* __restrict__ coef_l,
-                                   float* __restrict__ ecoef_l, float* __restrict__ mu_l) {
-  const int n = counts[3];
-  const int nz = ((n + kTileM - 1) / kTileM) * kTileM;
-  const int vpr = H / 8;   // 16-byte vectors per row
-  const int64_t total = (int64_t)nz * vpr;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int j = (int)(i / vpr), v = (int)(i - (int64_t)j * vpr);
-    uint4 val = make_uint4(0, 0, 0, 0);
-    if (j < n) {
-      const int k = live_map[j];
-      val = reinterpret_cast<const uint4*>(h_p + (int64_t)k * H)[v];
-      if (v == 0) {
-        tok_l[j] = tok_p[k] - tok_shift;
-        lse_l[j] = lse[k];
-        coef_l[j] = coef[k];
-        if (ecoef) {
-          ecoef_l[j] = ecoef[k];
-          mu_l[j] = mu[k];
-        }
-      }
-    } else if (v == 0) {
-      tok_l[j] = 0;
-      lse_l[j] = 0.f;
-      coef_l[j] = 0.f;
-      if (ecoef) {
-        ecoef_l[j] = 0.f;
-        mu_l[j] = 0.f;
-      }
+  if (src == nullptr) return;
+  const int n_pad = (total + pad - 1) / pad * pad;
+  for (int j = total + threadIdx.x; j < n_pad; j += kPackThreads) {
+    tok_l[j] = 0;
+    lse_l[j] = 0.f;
+    coef_l[j] = 0.f;
+    if (ecoef) {
+      ecoef_l[j] = 0.f;
+      mu_l[j] = 0.f;
     }
-    reinterpret_cast<uint4*>(h_l + (int64_t)j * H)[v] = val;
   }
+  const int64_t v0 = static_cast<int64_t>(total) * (H / 8), v1 = static_cast<int64_t>(n_pad) * (H / 8);
+#pragma unroll 4
+  for (int64_t v = v0 + threadIdx.x; v < v1; v += kPackThreads) reinterpret_cast<uint4*>(h_l)[v] = make_uint4(0, 0, 0, 0);
 }
 
 // dhidden_out[t] = bf16(dh32[live_of[pos[t]]]) for rows with a gradient, 0 for
@@ -780,18 +768,12 @@ cudaError_t launch_mask_count(const uint8_t* mask, int64_t T, int64_t* out, cuda
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact(const uint8_t* mask, int T, const Workspace& ws, const ZeroRows& z, int64_t ctl_words,
-                           cudaStream_t s) {
-  compact_kernel<<<1, 1024, 0, s>>>(mask, T, ws.row_map, ws.pos_of_row, ws.counts, z, ws.ctl,
-                                    static_cast<int>(ctl_words));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gather(const uint16_t* hidden, const int32_t* tokens, const float* b, const float* adv, int T,
-                          int Tcap, int H, const Workspace& ws, int n_sm, cudaStream_t s, int tok_shift) {
-  (void)T;
-  gather_kernel<<<n_sm * 8, 256, 0, s>>>(hidden, tokens, b, adv, tok_shift, Tcap, H, ws.row_map, ws.counts, ws.h_p,
-                                         ws.tok_p, b ? ws.b_p : nullptr, adv ? ws.adv_p : nullptr);
+cudaError_t launch_pack(const uint8_t* mask, int T, int H, const uint16_t* hidden, const int32_t* tokens, const float* b,
+                        const float* adv, int tok_shift, const Workspace& ws, const ZeroRows& z, int64_t ctl_words,
+                        int n_sm, cudaStream_t s) {
+  pack_kernel<<<n_sm * 8, kPackThreads, 0, s>>>(mask, T, H, hidden, tokens, b, adv, tok_shift, ws.row_map, ws.pos_of_row,
+                                                ws.counts, ws.h_p, ws.tok_p, ws.b_p, ws.adv_p, z, ws.ctl,
+                                                static_cast<int>(ctl_words));
   return cudaGetLastError();
 }
 
@@ -827,20 +809,23 @@ cudaError_t launch_loss_rows_ex(int Tcap, double denom, float clip_lo, float cli
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(int Tcap, double denom, bool with_ecoef, const Workspace& ws, float* loss_out,
-                            void* stats_out, void* stats_ex_out, unsigned* err, cudaStream_t s) {
-  (void)Tcap;
-  finalize_kernel<<<1, 1024, 0, s>>>(denom, ws.counts, ws.tile_list, ws.red, loss_out,
-                                     reinterpret_cast<StatsDev*>(stats_out),
-                                     reinterpret_cast<StatsExDev*>(stats_ex_out), ws.coef,
-                                     with_ecoef ? ws.ecoef : nullptr, ws.live_map, ws.live_of, err);
+cudaError_t launch_finish(int H, int pad, bool with_ecoef, double denom, const Workspace& ws, float* loss_out,
+                          void* stats_out, void* stats_ex_out, unsigned* err, int n_sm, cudaStream_t s) {
+  finish_kernel<<<n_sm * 8, kPackThreads, 0, s>>>(
+      -1, pad, denom, ws.counts, ws.tile_list, ws.red, loss_out, reinterpret_cast<StatsDev*>(stats_out),
+      reinterpret_cast<StatsExDev*>(stats_ex_out), H, 0, pad > 0 ? ws.h_p : nullptr, ws.tok_p, ws.lse, ws.coef,
+      with_ecoef ? ws.ecoef : nullptr, ws.mu, ws.live_of, ws.h_l, ws.tok_l, ws.lse_l, ws.coef_l, ws.ecoef_l, ws.mu_l,
+      nullptr, 0, err);
   return cudaGetLastError();
 }
 
-cudaError_t launch_live_gather(int H, bool with_ecoef, const Workspace& ws, int n_sm, cudaStream_t s) {
-  live_gather_kernel<<<n_sm * 8, 256, 0, s>>>(H, 0, ws.counts, ws.live_map, ws.h_p, ws.tok_p, ws.lse, ws.coef,
-                                              with_ecoef ? ws.ecoef : nullptr, ws.mu, ws.h_l, ws.tok_l, ws.lse_l,
-                                              ws.coef_l, ws.ecoef_l, ws.mu_l);
+cudaError_t launch_vp_pack(int T, int H, int pad, const uint16_t* hidden, const int32_t* tokens, const float* lse,
+                           const float* coef, int tok_shift, const Workspace& ws, int64_t ctl_words, int n_sm,
+                           cudaStream_t s) {
+  finish_kernel<<<n_sm * 8, kPackThreads, 0, s>>>(T, pad, 0.0, ws.counts, ws.tile_list, nullptr, nullptr, nullptr, nullptr, H,
+                                                  tok_shift, hidden, tokens, lse, coef, nullptr, nullptr, ws.live_of,
+                                                  ws.h_l, ws.tok_l, ws.lse_l, ws.coef_l, ws.ecoef_l, ws.mu_l, ws.ctl,
+                                                  static_cast<int>(ctl_words), nullptr);
   return cudaGetLastError();
 }
 
@@ -863,20 +848,6 @@ cudaError_t launch_vp_merge(int T, int Tcap, int n_shards, double denom, float c
   vp_merge_kernel<<<blocks, kTileM, 0, s>>>(T, n_shards, denom, clip_lo, clip_hi, ws.counts, ws.row_map, parts, b,
                                             adv, ws.coef, ws.red, lse_out, coef_out, logp_out,
                                             ent_out, tokloss_out, err);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_vp_live(int T, const float* coef, const Workspace& ws, int64_t ctl_words, cudaStream_t s) {
-  vp_live_kernel<<<1, 1024, 0, s>>>(T, coef, ws.counts, ws.tile_list, ws.live_map, ws.live_of, ws.ctl,
-                                    static_cast<int>(ctl_words));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_vp_gather(const uint16_t* hidden, const int32_t* tokens, const float* lse, const float* coef,
-                             int tok_shift, int H, const Workspace& ws, int n_sm, cudaStream_t s) {
-  live_gather_kernel<<<n_sm * 8, 256, 0, s>>>(H, tok_shift, ws.counts, ws.live_map, hidden, tokens, lse, coef,
-                                              nullptr, nullptr, ws.h_l, ws.tok_l, ws.lse_l, ws.coef_l, ws.ecoef_l,
-                                              ws.mu_l);
   return cudaGetLastError();
 }
 
