@@ -380,7 +380,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const float M = fmaxf(st.m, mo);
         float S2 = 0.f, Q2 = 0.f;
         auto add = [&](float mi, float si, float qi) {
-          if (si > 0.f) {
+          if (si != 0.f) {   // 0: no columns.  A NaN passes, so that the row shows it
             const float d = (mi - M) * kLog2e;
             const float f = ex2_approx(d);
             S2 = fmaf(f, si, S2);

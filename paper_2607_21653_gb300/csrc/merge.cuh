@@ -46,7 +46,7 @@ __device__ __forceinline__ RowStats merge_row_parts(const float4* __restrict__ p
 #pragma unroll 4
     for (int s = g; s < n_parts; s += kGroups) {
       const float4 p = p0[s * stride];
-      if (p.y > 0.f) {
+      if (p.y != 0.f) {   // 0: no columns.  A NaN passes
         const float d = p.x - M;
         const float f = ex2_approx(d * kLog2e);
         S += f * p.y;

@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(128) vp_merge_kernel(
     float S = 0.f, Q = 0.f;
     for (int s = 0; s < n_shards; ++s) {
       const float4 p = parts[(int64_t)s * T + t];
-      if (p.y > 0.f) {
+      if (p.y != 0.f) {   // 0: no columns.  A NaN passes
         const float d = p.x - M;
         const float f = ex2_approx(d * kLog2e);
         S += f * p.y;
