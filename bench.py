@@ -91,21 +91,15 @@ def code_hash(path):
     return hashlib.sha256(src.encode()).hexdigest()[:16]
 
 
-def quads_of(rows):
-    """512-row token quads (units of the cluster backward along the tokens)."""
-    return -(-(-(-rows // 128)) // 4)
-
-
 def recorded_traffic(kernel, workload, schedule, rows):
     """DRAM bytes per launch of `kernel` on `workload` under `schedule`
-    ("raster" or "deterministic") from the ncu summaries under profiles/, or
+    ("default" or "deterministic") from the ncu summaries under profiles/, or
     None if no summary matches them and the current source of the kernel.
     A summary captured on fewer token rows (the same H and V) is scaled to
-    `rows` by the units the launch processes, which for the same H and V is
-    the number of 512-row token quads: each quad is one more pass over the
-    vocabulary, and each raster group of four quads one more sweep of the
-    fp32 reduce targets.  Returns (bytes, note)."""
+    `rows` by 256-row token tiles: each is formed, read and added to the same
+    number of times whatever their number.  Returns (bytes, note)."""
     import glob
+    tiles = lambda r: -(-r // 256)
     for path in sorted(glob.glob(os.path.join(ROOT, "profiles", "*.md"))):
         with open(path) as f:
             for line in f:
@@ -121,9 +115,8 @@ def recorded_traffic(kernel, workload, schedule, rows):
                 b = float(kv["dram_bytes_per_launch"])
                 r = int(kv.get("rows", "0"))
                 if r > 0 and r != rows:
-                    q_cap, q_run = quads_of(r), quads_of(rows)
-                    return b * q_run / q_cap, (f"ncu capture on {r} backward rows ({q_cap} token quads), "
-                                               f"scaled to {q_run} quads")
+                    return b * tiles(rows) / tiles(r), (f"ncu capture on {r} backward rows ({tiles(r)} token tiles), "
+                                                        f"scaled to {tiles(rows)} tiles")
                 return b, "ncu capture of this launch"
     return None, None
 
@@ -571,24 +564,17 @@ def run_ours(args):
     step_s = ms / 1e3 / args.steps
     step_flops = (2.0 * n_active + 4.0 * tp) * H * V_work
     step_frac = step_flops / step_s / 1e12 / peak
-    bwd_kernel = "lmhead_bwd_quad_kernel" if H % 128 == 0 else "lmhead_bwd_kernel"
-    traffic, traffic_note = recorded_traffic(bwd_kernel, w.name, "deterministic" if args.deterministic else "raster",
+    bwd_kernel = "lmhead_bwd_chunk_kernel"
+    traffic, traffic_note = recorded_traffic(bwd_kernel, w.name, "deterministic" if args.deterministic else "default",
                                              tp)
     roofline = {
         "kernel": bwd_kernel, "bound": "tensor", "achieved": achieved_bwd, "peak": peak, "unit": "TFLOP/s",
         "frac": achieved_bwd / peak,
         "traffic": traffic,
         "traffic_source": traffic_note,
-        "limiter": ("fp32 reduce-add payload of the 512 x 512 units: operand loads queue behind it on each "
-                    "GPC's way into the crossbar (read coalescer held back ~46% of cycles); no unit saturated, "
-                    "the SM-to-crossbar interface 68% busy caps the kernel near 70% of the tensor roofline"
-                    if H % 128 == 0 else
-                    "per-SM reduce-add egress of the fp32 partial products of 128 x 256 units"),
+        "limiter": ("tensor cores under the board's power cap: the tensor pipe is busy about 90% of the cycles on "
+                    "three products (6 T_p H V executed, 4 T_p H V counted), and the clock settles near cuBLAS's"),
         "peak_source": f"{peaks['source']} bf16 sustained (kernel timed inside a long step)",
-        "concurrent": ("when the call splits the vocabulary (raster schedule; the library picks the split "
-                       "that evens out the two kernels), lmhead_bwd_kernel runs on the SMs no cluster of four "
-                       "can use over the last few percent of it; achieved and the event time cover both"
-                       if H % 128 == 0 and not args.deterministic else None),
         "kernels_per_step": launches / args.steps,
         "algorithmic_flops_per_launch": 4.0 * tp * H * V_work / max(1, len(mine)),
         "backward_rows": tp,
@@ -651,7 +637,7 @@ def l2_note(T, H, V):
     """Why no L2 flush runs between steps: what one step reads and writes."""
     w_gb, h_gb = V * H * 2 / 1e9, T * H * 2 / 1e9
     total = w_gb + h_gb + (V * H * 4 + T * H * 4) / 1e9
-    return (f"no flush: each step reads W ({w_gb:.2f} GB) and hidden ({h_gb:.2f} GB) and reduce-adds into "
+    return (f"no flush: each step reads W ({w_gb:.2f} GB) and hidden ({h_gb:.2f} GB) and writes "
             f"fp32 dW and dhidden, {total:.2f} GB in all, against 129 MB of L2")
 
 

@@ -379,7 +379,7 @@ molt_status molt_vp_backward(const uint16_t* hidden, const uint16_t* W_shard, co
  *     Make the first call on a device before any stream capture on it.
  *   - The timing hook (molt_set_timing_events) records kernel groups 1 (the
  *     forward kernel) and 2 (the merge) of this call.
- * Masked rows are computed and then written as 0 (there is no compaction),
+ * Masked rows are computed and then written as 0 (no row is packed away),
  * so prefer molt_token_logprobs_fwd when allocation is allowed.
  */
 #define MOLT_NOALLOC_MAX_TOKENS 32768
@@ -391,7 +391,7 @@ molt_status molt_token_logprobs_fwd_noalloc(const uint16_t* hidden, const uint16
  * Per-kernel timing hook for benchmarks.  While set, every LM-head call made
  * from the calling thread records starts[k] / stops[k] (caller-created CUDA
  * events) on its stream around kernel group k:
- *   k = 0  active-row compaction and packed gather
+ *   k = 0  the packing of the active rows
  *   k = 1  LM-head forward kernel (online log-softmax)
  *   k = 2  split merge, surrogate loss, the fixed-order reductions and the
  *          packing of the rows with a gradient for the backward

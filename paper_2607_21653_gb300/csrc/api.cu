@@ -283,8 +283,8 @@ Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = 
   return L;
 }
 
-// Workspace of the shard merge (molt_vp_loss): the active-row compaction,
-// per-row m c / D, the tile partial sums and finalize's row list.
+// Workspace of the shard merge (molt_vp_loss): the active rows' maps,
+// per-row m c / D, the rows' partial sums and the list of the rows with a gradient.
 Layout vp_loss_layout(int64_t T) {
   const int64_t Tcap = round_tiles(T);
   const int64_t ntile = Tcap / kTileM;
@@ -535,7 +535,7 @@ struct ZeroJoin {
     if (s_ != MOLT_OK) return s_;        \
   } while (0)
 
-// Shared front half of both LM-head calls: compaction, packed gather and the
+// Shared front half of the LM-head calls: the active rows packed and the
 // forward kernel (tensor maps already encoded by the caller).
 // tok_shift is subtracted from the tokens (a vocabulary shard's first column).
 molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int32_t* tokens, const uint8_t* mask,
@@ -569,7 +569,7 @@ molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int3
 // Zero on stream s what the backward adds to: the deterministic schedule's turn
 // counters and, for the kernels that only add, the dhidden accumulator and, unless
 // the call accumulates into it, dW (the backward over chunks stores the first
-// contributions; its counters are zeroed with the compaction).
+// contributions; its counters are zeroed where the rows are packed).
 molt_status zero_backward_targets(const Workspace& w, int64_t T, int64_t H, int64_t V, bool det, float* dW_out,
                                   int accumulate_dW, cudaStream_t s) {
   const int64_t Tcap = round_tiles(T);

@@ -9,7 +9,7 @@
 // GPU loading the library holds until the process exits.  The caller still owns
 // and passes every input and output; the call allocates nothing.
 //
-// Differences from molt_token_logprobs_fwd: no active-row compaction (masked
+// Differences from molt_token_logprobs_fwd: no packing of the active rows (masked
 // rows are computed and then written as 0), as many vocab splits as the array's
 // kNoAllocParts partial statistics per row of the largest batch leave room for,
 // and T <= kNoAllocMaxRows.  The same forward kernel does the work.

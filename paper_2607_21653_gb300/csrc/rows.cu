@@ -1,7 +1,7 @@
 // Row-level kernels of the policy-update path: GRPO advantages, advantage
-// broadcast, mask count, active-row compaction, packed gathers, the split-vocab
-// merge with the clipped surrogate, the fixed-order loss reduction and the
-// dhidden cast.  None of these is a contraction; they are launch- or HBM-bound.
+// broadcast, mask count, the packing of the active rows and of the rows with a
+// gradient, the split-vocab merge with the clipped surrogate, the fixed-order loss
+// reduction and the dhidden cast.  None of these is a contraction; they are launch- or HBM-bound.
 #include <cstdint>
 #include <cuda_runtime.h>
 
