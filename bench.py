@@ -565,8 +565,8 @@ def run_ours(args):
     step_flops = (2.0 * n_active + 4.0 * tp) * H * V_work
     step_frac = step_flops / step_s / 1e12 / peak
     bwd_kernel = "lmhead_bwd_chunk_kernel"
-    traffic, traffic_note = recorded_traffic(bwd_kernel, w.name, "deterministic" if args.deterministic else "default",
-                                             tp)
+    traffic, traffic_note = (None, None) if vshard > 1 else recorded_traffic(
+        bwd_kernel, w.name, "deterministic" if args.deterministic else "default", tp)
     roofline = {
         "kernel": bwd_kernel, "bound": "tensor", "achieved": achieved_bwd, "peak": peak, "unit": "TFLOP/s",
         "frac": achieved_bwd / peak,
