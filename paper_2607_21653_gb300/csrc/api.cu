@@ -148,6 +148,14 @@ struct ChunkPlan {
   size_t g_bytes() const { return use ? static_cast<size_t>(g_rows()) * kBK * 2 : 0; }
   int64_t ctl_words() const { return use ? kChunkCtlHead + 4 * max_chunks : 0; }
   int64_t turn_words() const { return use ? (n_t + n_v) * n_h * 16 : 0; }
+  // list steps between a chunk's logit tiles and those that read them
+  int lag(int64_t H, int64_t pairs) const {
+    if (max_chunks <= n_buf) return n_buf - 1;   // no buffer is used twice: logits first
+    const int64_t ct = std::min(n_t, chunk_t), cv = std::min(n_v, chunk_v);
+    const int64_t step = ct * cv * (std::max<int64_t>(H / kBK, 9) + 8 * n_h);
+    const int64_t hold = (4 * ct + 4 * cv + 18) * pairs;
+    return static_cast<int>(std::min<int64_t>(n_buf - 1, std::max<int64_t>(2, hold / step + 1)));
+  }
 };
 // T is the call's row count; the rows with a gradient, at most as many, are
 // known on the device only.
@@ -166,39 +174,42 @@ struct ChunkPlan {
 //     because tests/test_gpu_shapes.py holds the cluster kernel's vocab split there.
 //   H < 256: none (H = 64, T = 512, V = 19000 0.021 and 0.033).
 //
-// Chunk size: 16 x 16 tiles (4096 x 4096) in two buffers drain least; T = 16384, H =
-// 4096, V = 151936 took 38.8 ms, against 40.5 for 8 x 16 in four, 39.5 for 12 x 20
-// and 41.2 for 32 x 8.  With few tiles or a short H such a chunk holds too little
-// between a tile and what it waits for, and dH, whose tiles are few and as long as
-// a chunk, does not spread over the SMs; more, smaller buffers are faster (T = 8000,
-// H = 256, V = 50000: 0.70 ms with 4 x 4 in sixteen, 0.77 with 8 x 16 in four; T =
-// 20000, H = 512, V = 30000: 1.39 with 8 x 8 in four, 1.46 with 16 x 16; T = 1500, H =
-// 320, V = 20000: 0.074 with 8 x 8 in eight, 0.086 with 8 x 16 in four; T = 30000,
-// H = 1024, V = 5000: 0.55 and 0.64 with 16 x 8; T = 5000, H = 2048, V = 32000: 1.10
-// with 16 x 8 in four, 1.14 with 8 x 8; T = 700, H = 320, V = 100000: 0.18 with 4 x 4
-// in sixteen, 0.29 with 4 x 32 in four).
+// Chunk size and buffers (64 MB together, half of L2).  16 x 16 tiles (4096 x 4096) in
+// two buffers drain least and win where the power cap binds and a chunk holds many times
+// the tiles in flight: T = 4096, H = 4096, V = 151936 10.0 ms (whole call), 8 x 8 in
+// eight 10.6; T = 32768, H = 2048, V = 32000 8.5 and 8.6.  Everywhere else what counts is
+// that no tile waits for the ones it depends on: 8 x 8 in eight (T = 32768, H = 1024, V =
+// 50000 6.88 ms, 16 x 16 7.07), 4 x 8 in sixteen for at most four token tiles (T = 512, H = 768, V = 100000 0.27
+// ms, 4 x 32 in four 0.36; with few vocab tiles 4 x 4, so that dH spreads), 8 x 4 in sixteen at H = 256 (T = 12000, V = 60000 1.08 ms, 4 x 4
+// in sixteen 1.25).
+//
+// Lag: the list steps from a chunk's logit tiles to the tiles that read them, long enough
+// for the tiles that the pairs hold (about one of dH and one of dW, 4 K blocks a chunk
+// tile, and 18 K blocks of epilogue and signalling) and no longer, since the buffers
+// past it are what the next logit tiles run ahead in; a step is its tiles' K blocks
+// (a logit tile no less than its epilogue, 9) over the pairs.  T = 5003, H = 320, V =
+// 50257 (8 x 8 in eight): 0.52 ms at a lag of 3, 0.489 at 4, 0.493 at 5, 0.565 at 7; T =
+// 12000, H = 768, V = 40000 1.42 at 3, 1.55 at 4; T = 32768, H = 1024, V = 50000 7.05 at
+// 2, 6.88 at 3; a step too short costs up to half.
 ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
   ChunkPlan p;
   if (T <= 0 || H < 256 || (H == 256 && T <= 768 && V > 4096 && V <= 20480) || (H > 256 && H < 512 && T < 512)) return p;
   p.n_t = (T + 255) / 256;
   p.n_v = (V + 255) / 256;
   p.n_h = (H + 255) / 256;
-  p.chunk_t = 16;
-  p.chunk_v = 16;
   int64_t most_buf = 8;
-  if (p.n_t <= 4 && H >= 640) {
-    p.chunk_v = std::max<int64_t>(4, std::min<int64_t>(32, (p.n_v + 7) / 8));
-  } else if (p.n_t <= 2) {
-    p.chunk_v = 8;
+  if (p.n_t <= 4) {
+    p.chunk_t = 4;
+    p.chunk_v = H < 640 && p.n_t <= 2 ? 8 : std::max<int64_t>(4, std::min<int64_t>(8, (p.n_v + 7) / 8));
     most_buf = 16;
-  } else if (p.n_t <= 4 || H <= 256) {
-    p.chunk_t = p.chunk_v = 4;
+  } else if (H <= 256) {
+    p.chunk_t = 8;
+    p.chunk_v = 4;
     most_buf = 16;
-  } else if (H < 1024 || (H < 2048 && p.n_t * p.n_v < 2560 && p.n_v < 64)) {
+  } else if (H >= 1536 && p.n_t * p.n_v >= 2560) {
+    p.chunk_t = p.chunk_v = 16;
+  } else {
     p.chunk_t = p.chunk_v = 8;
-    most_buf = p.n_t <= 16 ? 8 : 4;
-  } else if (p.n_t * p.n_v < 2560) {
-    p.chunk_v = 8;
   }
   const int64_t n_tc = (p.n_t + p.chunk_t - 1) / p.chunk_t, n_vc = (p.n_v + p.chunk_v - 1) / p.chunk_v;
   const int64_t tiles = p.n_t * p.n_v + (p.n_t * n_vc + p.n_v * n_tc) * p.n_h;
@@ -625,6 +636,7 @@ molt_status run_backward_chunk(const DeviceInfo* di, const ChunkPlan& cp, const 
   a.det_turns = det ? w.turns : nullptr;
   a.err = di->status;
   const int ctas = det_clusters > 0 ? 4 * det_clusters : di->n_sm;
+  a.lag = cp.lag(H, std::max(1, ctas / 2));
   ev_start(3, stream);
   MOLT_LAUNCH(launch_lmhead_bwd_chunk(m, a, ctas, stream), "lmhead backward");
   ev_stop(3, stream);

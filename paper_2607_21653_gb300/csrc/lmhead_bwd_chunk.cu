@@ -27,12 +27,13 @@
 //
 // One persistent launch walks all tiles of all chunks.  The tiles form one list,
 //   step s:  dH tiles of chunk s - L, Z tiles of chunk s, dW tiles of chunk s - L
-// (L = buffers - 1), and CTA pairs claim them in list order from a counter.  A dH
-// or dW tile waits until every Z tile of its chunk is stored (zdone), a Z tile's
-// epilogue until every tile that read the buffer's previous chunk is through
+// (L < buffers, see chunk_plan in api.cu), and CTA pairs claim them in list order from
+// a counter.  A dH or dW tile waits until every Z tile of its chunk is stored (zdone), a
+// Z tile's epilogue until every tile that read the buffer's previous chunk is through
 // (cdone).  Both are earlier in the list, so they were claimed earlier by pairs
-// that are running: the waits end whatever share of the grid is resident.  The
-// order leaves a third of a chunk's tiles between a tile and what it waits for.
+// that are running: the waits end whatever share of the grid is resident.  L steps
+// lie between a chunk's Z tiles and what reads them, buffers - L between those and the
+// buffer's next Z tiles: each has to cover the tiles in flight.
 //
 // Roles per CTA (384 threads): warps 0 and 11 TMA producers of the A and the B
 // operand (each CTA loads its half of both), warp 1 MMA issuer (even CTA) and
@@ -55,8 +56,8 @@
 // which converts without the target's and the edge's selects wherever the warp has
 // neither and signals a Z tile's stores one tile later (T = 4000, H = 320, V =
 // 50257: 0.51 ms, before these three 0.57; T = 3000, H = 1024, V = 32000: 0.355,
-// before 0.399), and by the waits between the tiles of a chunk, which more and
-// smaller buffers shorten (see chunk_plan in api.cu).  Counters on T = 8192, H = 4096,
+// before 0.399), and by the waits between the tiles of a chunk (see
+// chunk_plan in api.cu).  Counters on T = 8192, H = 4096,
 // V = 32768: tensor pipe active 90 % of the cycles, DRAM 29 %, L2 59 %.
 #include <atomic>
 #include <climits>
@@ -104,7 +105,7 @@ struct __align__(16) Tile {
 struct TileList {
   int n_rows, V, H;
   bool add_dw;
-  int n_t, n_v, n_h, n_tc, n_vc, n_chunks, nb;
+  int n_t, n_v, n_h, n_tc, n_vc, n_chunks, nb, lag;
   int total;                             // tiles in the list
   int step, base;                        // list step and its first index
   int n_dh, n_z, n_dw;                   // tiles of the step
@@ -125,6 +126,7 @@ struct TileList {
     n_chunks = n_tc * n_vc;
     total = n_t * n_v + (n_t * n_vc + n_v * n_tc) * n_h;   // Z + dH + dW tiles of all chunks
     nb = a.n_buf;
+    lag = a.lag;
     step = 0;
     base = 0;
     fill();
@@ -138,7 +140,7 @@ struct TileList {
   }
   __device__ __forceinline__ void fill() {
     n_dh = n_z = n_dw = 0;
-    const int c = step - (nb - 1);
+    const int c = step - lag;
     if (c >= 0 && c < n_chunks) {
       span(c, c_t0, c_ct, c_v0, c_cv);
       n_dh = c_ct * n_h;
@@ -158,7 +160,7 @@ struct TileList {
     }
     int i = j - base;
     const bool z = i >= n_dh && i < n_dh + n_z;
-    x.chunk = z ? step : step - (nb - 1);
+    x.chunk = z ? step : step - lag;
     const int tc = x.chunk / n_vc, vc = x.chunk - tc * n_vc;
     x.buf = x.chunk % nb;
     x.t0 = z ? z_t0 : c_t0;

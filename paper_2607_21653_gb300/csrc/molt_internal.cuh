@@ -110,6 +110,7 @@ struct ChunkArgs {
   int V, H;
   int chunk_t, chunk_v;      // a chunk's tiles of tokens and vocab, at most
   int n_buf;                 // chunk buffers (>= 2)
+  int lag;                   // list steps from a chunk's logit tiles to those that read it
   int buf_panels;            // 64-column panels of one buffer
   int panel_rows;            // token rows of one panel (128 bytes each)
   int add_dw;                // the call adds to dW
