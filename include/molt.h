@@ -233,11 +233,14 @@ molt_status molt_policy_loss_fwd_bwd(const uint16_t* hidden, const uint16_t* W, 
  *   deterministic 1: dW and dhidden are bitwise reproducible for the same inputs
  *                 (no paper counterpart).  The backward then fixes the order of
  *                 every partial-sum reduction: the contributions to dW are added
- *                 in token order and those to dhidden in vocabulary order, chunk by
- *                 chunk (of up to 4096 x 4096; 512 x 512 blocks for short hidden
- *                 sizes), each [32 x 128] slab waiting its turn on a counter in
- *                 the workspace.  The order does not depend on the number of SMs
- *                 the backward runs on (see det_clusters).  For short hidden sizes
+ *                 in token order, 512 tokens with a gradient at a time, and those to
+ *                 dhidden in vocabulary order, 512 columns at a time, each
+ *                 [32 x 128] slab waiting its turn on a counter in the workspace.
+ *                 The order depends neither on the kernel that the sizes select nor
+ *                 on the number of SMs it runs on (see det_clusters), and a row's
+ *                 log-probability is summed in a fixed order of its own, so that the
+ *                 bits of all outputs also stay the same from one version of the
+ *                 library to the next.  For short hidden sizes
  *                 its clusters wait on one another and must be resident together.
  *                 If other work keeps SMs busy for seconds, a wait gives up after
  *                 about 4 s, the call's backward returns early with dW and dhidden

@@ -173,6 +173,10 @@ struct ChunkPlan {
 //     would be faster already (V = 19000 0.051 and 0.044); the line lies above
 //     because tests/test_gpu_shapes.py holds the cluster kernel's vocab split there.
 //   H < 256: none (H = 64, T = 512, V = 19000 0.021 and 0.033).
+//   Reproducible calls (the same bits from either kernel): with H up to 512 and more than
+//     256 rows the cluster kernel from 25600 columns on, where adding a term at a time
+//     costs it less (T = 16384, H = 384, V = 100000 5.65 and 6.45; T = 4096, H = 512, V =
+//     20000 0.409 and 0.367; T = 64, H = 512, V = 100000 0.744 and 0.590).
 //
 // Chunk size and buffers (64 MB together, half of L2).  16 x 16 tiles (4096 x 4096) in
 // two buffers drain least and win where the power cap binds and a chunk holds many times
@@ -191,9 +195,11 @@ struct ChunkPlan {
 // 50257 (8 x 8 in eight): 0.52 ms at a lag of 3, 0.489 at 4, 0.493 at 5, 0.565 at 7; T =
 // 12000, H = 768, V = 40000 1.42 at 3, 1.55 at 4; T = 32768, H = 1024, V = 50000 7.05 at
 // 2, 6.88 at 3; a step too short costs up to half.
-ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
+ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V, bool det) {
   ChunkPlan p;
-  if (T <= 0 || H < 256 || (H == 256 && T <= 768 && V > 4096 && V <= 20480) || (H > 256 && H < 512 && T < 512)) return p;
+  if (T <= 0 || H < 256 || (H == 256 && T <= 768 && V > 4096 && V <= 20480) || (H > 256 && H < 512 && T < 512) ||
+      (det && H <= 512 && T > 256 && V >= 25600))
+    return p;
   p.n_t = (T + 255) / 256;
   p.n_v = (V + 255) / 256;
   p.n_h = (H + 255) / 256;
@@ -211,6 +217,7 @@ ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V) {
   } else {
     p.chunk_t = p.chunk_v = 8;
   }
+  if (det) p.chunk_v += p.chunk_v % 2;   // whole terms of 512 columns (chunk_t is even)
   const int64_t n_tc = (p.n_t + p.chunk_t - 1) / p.chunk_t, n_vc = (p.n_v + p.chunk_v - 1) / p.chunk_v;
   const int64_t tiles = p.n_t * p.n_v + (p.n_t * n_vc + p.n_v * n_tc) * p.n_h;
   p.use = tiles < (int64_t(1) << 30);   // claimed with a 32-bit counter
@@ -272,7 +279,7 @@ Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = 
   L.tile_list = take(ntile * 4);
   L.red = take(Tcap / kRedRows * kRedSlots * 8);
   L.dh32 = with_bwd ? take(static_cast<size_t>(Tcap) * H * 4) : o;
-  const ChunkPlan cp = chunk_plan(T, H, V);
+  const ChunkPlan cp = chunk_plan(T, H, V, det);
   L.turns = (with_bwd && det)
                 ? take(static_cast<size_t>(cp.use ? cp.turn_words() : turn_layout(Tcap, H, V).words) * 4)
                 : kNoRegion;
@@ -341,7 +348,7 @@ Layout vp_backward_layout(int64_t T, int64_t H, int64_t V) {
   L.lse_l = take(Tcap * 4);
   L.coef_l = take(Tcap * 4);
   L.dh32 = take(static_cast<size_t>(Tcap) * H * 4);
-  const ChunkPlan cp = chunk_plan(T, H, V);
+  const ChunkPlan cp = chunk_plan(T, H, V, false);
   L.g = take(cp.g_bytes());
   L.ctl = take(static_cast<size_t>(cp.ctl_words()) * 4);
   L.row_map = L.pos = L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.coef = L.red =
@@ -548,11 +555,12 @@ struct ZeroJoin {
 
 // Shared front half of the LM-head calls: the active rows packed and the
 // forward kernel (tensor maps already encoded by the caller).
-// tok_shift is subtracted from the tokens (a vocabulary shard's first column).
+// tok_shift is subtracted from the tokens (a vocabulary shard's first column);
+// ordered: the reproducible call's sums.
 molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int32_t* tokens, const uint8_t* mask,
                         const float* b, const float* adv, int64_t T, int64_t H, int64_t V, int S,
                         const Workspace& w, const CUtensorMap& tm_h, const CUtensorMap& tm_w, cudaStream_t s,
-                        const ZeroRows& zero, int64_t ctl_words = 0, int tok_shift = 0) {
+                        const ZeroRows& zero, int64_t ctl_words = 0, int tok_shift = 0, bool ordered = false) {
   const int64_t Tcap = round_tiles(T);
   ev_start(0, s);
   MOLT_LAUNCH(launch_pack(mask, static_cast<int>(T), static_cast<int>(H), hidden, tokens, b, adv, tok_shift, w, zero,
@@ -567,6 +575,7 @@ molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int3
   fa.H = static_cast<int>(H);
   fa.n_split = S;
   fa.n_vtiles = static_cast<int>((V + kFwdBN - 1) / kFwdBN);
+  fa.ordered = ordered;
   fa.next_unit = w.counts + 4;
   fa.part = w.part;
   fa.zx = w.zx;
@@ -584,7 +593,7 @@ molt_status run_forward(const DeviceInfo* di, const uint16_t* hidden, const int3
 molt_status zero_backward_targets(const Workspace& w, int64_t T, int64_t H, int64_t V, bool det, float* dW_out,
                                   int accumulate_dW, cudaStream_t s) {
   const int64_t Tcap = round_tiles(T);
-  const ChunkPlan cp = chunk_plan(T, H, V);
+  const ChunkPlan cp = chunk_plan(T, H, V, det);
   if (det) {
     const int64_t words = cp.use ? cp.turn_words() : turn_layout(Tcap, H, V).words;
     MOLT_CUDA(cudaMemsetAsync(w.turns, 0, static_cast<size_t>(words) * 4, s), "memset turns");
@@ -653,7 +662,7 @@ molt_status run_backward(const DeviceInfo* di, const uint16_t* W, int64_t T, int
                          const Workspace& w, bool det, int n_det, bool with_ecoef, float* dW_out, int accumulate_dW,
                          bool zeroed, cudaStream_t stream) {
   if (!zeroed) MOLT_TRY(zero_backward_targets(w, T, H, V, det, dW_out, accumulate_dW, stream));
-  if (const ChunkPlan cp = chunk_plan(T, H, V); cp.use)
+  if (const ChunkPlan cp = chunk_plan(T, H, V, det); cp.use)
     return run_backward_chunk(di, cp, W, T, H, V, w, det, n_det, with_ecoef, dW_out, accumulate_dW, stream);
   const int64_t Tcap = round_tiles(T);
   const bool pair_bwd = (H % 128) == 0;   // the cluster backward
@@ -790,7 +799,7 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
     return MOLT_OK;
   }
   const int64_t Tcap = round_tiles(T);
-  const int S = forward_splits(Tcap, H, V, di->n_sm);
+  const int S = det ? ordered_splits(Tcap, V, di->n_sm) : forward_splits(Tcap, H, V, di->n_sm);
   // deterministic schedule: n_det clusters (a multiple of 4), all resident at
   // once, whose reduce-adds take turns
   int n_det = det ? lmhead_bwd_quad_det_clusters(di->n_sm) : 0;
@@ -814,7 +823,7 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
   // the caller's stream waits for them before the backward, or on any early
   // return before the workspace is released
   ZeroJoin zj;
-  const ChunkPlan cp = chunk_plan(T, H, V);
+  const ChunkPlan cp = chunk_plan(T, H, V, det);
   if (const SideLane* zl = cp.use ? nullptr : side_lane(stream)) {
     MOLT_CUDA(cudaEventRecord(zl->fork, stream), "zero fork");
     MOLT_CUDA(cudaStreamWaitEvent(zl->side, zl->fork, 0), "zero fork");
@@ -831,17 +840,17 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
     if (zs != MOLT_OK) return zs;
   }
   MOLT_TRY(run_forward(di, hidden, tokens, mask, behavior_logp, adv, T, H, V, S, w, tm_h, tm_w, stream,
-                       ZeroRows{{logp_out, entropy_out, token_loss_out}}, cp.ctl_words()));
+                       ZeroRows{{logp_out, entropy_out, token_loss_out}}, cp.ctl_words(), 0, det));
   ev_start(2, stream);
   if (opts) {
-    MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
+    MOLT_LAUNCH(launch_merge(false, det, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
                            entropy_out, nullptr, w.lp_p, w.ent_p, di->status, stream),
               "merge");
     MOLT_LAUNCH(launch_seq_gate(static_cast<int>(T), static_cast<int>(Tcap), ex, w, di->status, stream), "gate");
     MOLT_LAUNCH(launch_loss_rows_ex(static_cast<int>(Tcap), denom, clip_lo, clip_hi, ex, w, token_loss_out, stream),
               "loss rows");
   } else {
-    MOLT_LAUNCH(launch_merge(true, static_cast<int>(Tcap), static_cast<int>(V), S, denom, clip_lo, clip_hi, w,
+    MOLT_LAUNCH(launch_merge(true, false, static_cast<int>(Tcap), static_cast<int>(V), S, denom, clip_lo, clip_hi, w,
                            logp_out, entropy_out, token_loss_out, nullptr, nullptr, di->status, stream),
               "merge");
   }
@@ -894,6 +903,13 @@ int forward_splits(int64_t Tcap, int64_t H, int64_t V, int n_sm) {
   auto waves = [&](int64_t w) { return (w * pairs + n_mt - 1) / n_mt; };
   const int64_t S = std::min(waves(24), std::max(waves(4), n_vt * (H / kBK) / 64));
   return static_cast<int>(std::max<int64_t>(1, std::min(S, n_vt)));
+}
+
+// 16 waves of 128-row units on all SMs.  The splits decide how a row's sums are
+// rounded, so this rule stays as it is.
+int ordered_splits(int64_t Tcap, int64_t V, int n_sm) {
+  const int64_t n_vt = (V + kFwdBN - 1) / kFwdBN, n_mt = Tcap / kTileM;
+  return static_cast<int>(std::max<int64_t>(1, std::min((int64_t(16) * n_sm + n_mt - 1) / n_mt, n_vt)));
 }
 
 molt_status encode_tmap_2d(CUtensorMap* m, CUtensorMapDataType dt, int elem_bytes, const void* base, uint64_t rows,
@@ -1047,7 +1063,8 @@ size_t molt_policy_loss_workspace_bytes_ex(int64_t T, int64_t H, int64_t V, cons
   const DeviceInfo* di = device_info(&st);
   const int n_sm = di ? di->n_sm : 152;
   const int64_t Tcap = round_tiles(T);
-  return layout(T, H, V, forward_splits(Tcap > 0 ? Tcap : kTileM, H, V, n_sm), true, det).total;
+  const int64_t rows = std::max<int64_t>(Tcap, kTileM);
+  return layout(T, H, V, det ? ordered_splits(rows, V, n_sm) : forward_splits(rows, H, V, n_sm), true, det).total;
 }
 
 molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, const int32_t* tokens,
@@ -1073,7 +1090,7 @@ molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, c
   MOLT_TRY(run_forward(di, hidden, tokens, mask, nullptr, nullptr, T, H, V, S, w, tm_h, tm_w, stream,
                        ZeroRows{{logp_out, entropy_out}}));
   ev_start(2, stream);
-  MOLT_LAUNCH(launch_merge(false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
+  MOLT_LAUNCH(launch_merge(false, false, static_cast<int>(Tcap), static_cast<int>(V), S, 0.0, 0.f, 0.f, w, logp_out,
                          entropy_out, nullptr, nullptr, nullptr, di->status, stream),
             "merge");
   ev_stop(2, stream);
@@ -1221,7 +1238,7 @@ molt_status molt_vp_backward(const uint16_t* hidden, const uint16_t* W_shard, co
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
   ev_start(2, stream);
-  const ChunkPlan cp = chunk_plan(T, H, V_shard);
+  const ChunkPlan cp = chunk_plan(T, H, V_shard, false);
   MOLT_LAUNCH(launch_vp_pack(static_cast<int>(T), static_cast<int>(H), cp.use ? kBK : kTileM, hidden, tokens, lse, coef,
                              static_cast<int>(v_begin), w, cp.ctl_words(), di->n_sm, stream),
               "shard rows");

@@ -24,6 +24,7 @@
 // through its SMs' path to L2, and those drains held the operand loads back.
 // A chunk is eight times wider in both directions, so the drains fall to an
 // eighth, and no tile waits for a chain Z -> g -> dH -> dW inside one cluster.
+// (Reproducible sums keep the drains: see kDetK.)
 //
 // One persistent launch walks all tiles of all chunks.  The tiles form one list,
 //   step s:  dH tiles of chunk s - L, Z tiles of chunk s, dW tiles of chunk s - L
@@ -80,6 +81,12 @@ constexpr int kEpiWarps = 8;
 constexpr int kThreads = 128 + 32 * kEpiWarps;
 constexpr int kSmemBytes = 1024 + kOffBox + kEpiWarps * kBoxBytes;
 constexpr int kSlots = 2;                         // tiles handed from the claiming warp to the other roles
+// Tokens (columns) per term of a reproducible sum.  The mode's results stay the same
+// bits from one version of the library to the next, so a term is what the cluster
+// kernel adds at a time, and the two kernels give the same bits.  A whole chunk to a
+// term, an eighth of the additions into global memory, takes 14.8 ms for the call at
+// T = 16384, H = 4096, V = 65536 (30 % masked), terms of 512 18.2, the cluster kernel 23.1.
+constexpr int kDetK = 512;
 constexpr float kLog2e = 1.4426950408889634f;
 
 enum TileKind : int { kTileZ = 0, kTileDH = 1, kTileDW = 2 };
@@ -102,6 +109,8 @@ struct __align__(16) Tile {
 };
 
 // The tile list, walked forwards by the claiming thread: claimed indices only grow.
+// kAlign: chunks begin at a multiple of so many tiles.
+template <int kAlign>
 struct TileList {
   int n_rows, V, H;
   bool add_dw;
@@ -133,10 +142,15 @@ struct TileList {
   }
   __device__ __forceinline__ void span(int c, int& t0, int& ct, int& v0, int& cv) const {
     const int tc = c / n_vc, vc = c - tc * n_vc;
-    t0 = static_cast<int>(static_cast<int64_t>(tc) * n_t / n_tc);
-    ct = static_cast<int>(static_cast<int64_t>(tc + 1) * n_t / n_tc) - t0;
-    v0 = static_cast<int>(static_cast<int64_t>(vc) * n_v / n_vc);
-    cv = static_cast<int>(static_cast<int64_t>(vc + 1) * n_v / n_vc) - v0;
+    t0 = begin(tc, n_tc, n_t);
+    ct = begin(tc + 1, n_tc, n_t) - t0;
+    v0 = begin(vc, n_vc, n_v);
+    cv = begin(vc + 1, n_vc, n_v) - v0;
+  }
+  // first of n tiles, cut evenly into `parts`, that part i holds
+  __device__ __forceinline__ int begin(int i, int parts, int n) const {
+    const int64_t blocks = (n + kAlign - 1) / kAlign;
+    return min(n, static_cast<int>(i * blocks / parts) * kAlign);
   }
   __device__ __forceinline__ void fill() {
     n_dh = n_z = n_dw = 0;
@@ -220,7 +234,8 @@ __device__ __forceinline__ void write_box32(uint32_t box, int lane, const float 
   }
 }
 
-template <bool kEnt>
+// kEnt: with an entropy bonus; kDet: reproducible sums
+template <bool kEnt, bool kDet>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     lmhead_bwd_chunk_kernel(const __grid_constant__ ChunkMaps m, const ChunkArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -316,6 +331,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     return x.kind >= 0;
   };
 
+  // K blocks that one accumulator sums: all of a tile's, or in a reproducible sum one
+  // term's, which a chunk's begin is a multiple of
+  auto term_k = [&](const Tile& x) -> int { return kDet && x.kind != kTileZ ? kDetK / kBK : INT_MAX / 2; };
+
   if (warp == 0) {
     // A: 128 rows of h (Z) or g (dH), or 64 token rows of two panels of g (dW)
     if (lane == 0) {
@@ -395,50 +414,57 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     if (lane == 0 && leader) {
-      uint32_t st = 0, ph = 0;
+      uint32_t st = 0, ph = 0, ai = 0;
       bool ok = true;
       Tile x;
-      for (uint32_t ji = 0; next_tile(ji, x); ++ji) {
-        const int nk = x.nk;
-        const uint32_t buf = ji & 1u;
-        if (!mbar_wait(smem_u32(&acce_bar[buf]), ((ji >> 1) & 1u) ^ 1u, abort_flag, a.err)) break;
-        tc_fence_after();
-        const uint32_t d = tmem_base + buf * 256;
+      for (uint32_t ji = 0; ok && next_tile(ji, x); ++ji) {
+        const int nk = x.nk, kt = term_k(x);
         // K-major operands advance 32 bytes per K = 16, MN-major ones 16 rows of 128
         const bool a_mn = x.kind == kTileDW, b_mn = x.kind != kTileZ;
         const uint32_t idesc = idesc_bf16_f32(256, b_mn ? mma_n(x.h) : 256, a_mn, b_mn);
         const uint32_t a_step = a_mn ? 128u : 2u, b_step = b_mn ? 128u : 2u;
         const uint64_t ad0 = sdesc_sw128(smem0, a_mn ? 8192u : 16u, 1024);
         const uint64_t bd0 = sdesc_sw128(smem0 + kHalf, b_mn ? 8192u : 16u, 1024);
+        uint32_t d = 0;
         auto issue = [&](uint32_t stage, uint32_t accumulate) {
           umma4_bf16_pair(d, ad0 + stage * (kStageBytes >> 4), bd0 + stage * (kStageBytes >> 4), a_step, b_step,
                           idesc, accumulate);
           umma_commit_pair_mc(smem_u32(&empty_bar[stage]), 3);
         };
-        // two stages per turn: one wait of the issuing thread for eight products.
-        // The copies' complete_tx makes both CTAs' bytes visible to the MMAs
-        // issued after the phase flips; a CTA-scope wait is enough.
-        for (int kb = 0; kb < nk; kb += 2) {
-          const bool two = kb + 1 < nk;
-          const uint32_t st0 = st;
-          if (!(ok = mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag, a.err))) break;
-          if (++st == kStages) {
-            st = 0;
-            ph ^= 1u;
-          }
-          if (two && !(ok = mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag, a.err))) break;
+        // one accumulator after the other: one to a tile, or to a term
+        int kb = 0;
+        do {
+          const uint32_t buf = ai & 1u;
+          if (!(ok = mbar_wait(smem_u32(&acce_bar[buf]), ((ai >> 1) & 1u) ^ 1u, abort_flag, a.err))) break;
           tc_fence_after();
-          issue(st0, kb != 0 ? 1u : 0u);
-          if (two) {
-            issue(st, 1u);
+          d = tmem_base + buf * 256;
+          // two stages per turn: one wait of the issuing thread for eight products.
+          // The copies' complete_tx makes both CTAs' bytes visible to the MMAs
+          // issued after the phase flips; a CTA-scope wait is enough.
+          const int k0 = kb, k1 = min(nk, kb + kt);
+          for (; kb < k1; kb += 2) {
+            const bool two = kb + 1 < k1;
+            const uint32_t st0 = st;
+            if (!(ok = mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag, a.err))) break;
             if (++st == kStages) {
               st = 0;
               ph ^= 1u;
             }
+            if (two && !(ok = mbar_wait(smem_u32(&full_bar[st]), ph, abort_flag, a.err))) break;
+            tc_fence_after();
+            issue(st0, kb != k0 ? 1u : 0u);
+            if (two) {
+              issue(st, 1u);
+              if (++st == kStages) {
+                st = 0;
+                ph ^= 1u;
+              }
+            }
           }
-        }
-        if (!ok) break;
-        umma_commit_pair_mc(smem_u32(&accf_bar[buf]), 3);
+          if (!ok) break;
+          umma_commit_pair_mc(smem_u32(&accf_bar[buf]), 3);
+          ++ai;
+        } while (kb < nk);
       }
       umma_commit_pair_mc(smem_u32(&done_bar), 1);
       mbar_wait_drain(smem_u32(&done_bar), 0, a.err);
@@ -447,7 +473,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (lane == 0 && leader) {
       const uint32_t tile_peer0 = mapa_shared(smem_u32(&tile_sh[0]), 1);
       const uint32_t jfull_peer0 = mapa_shared(smem_u32(&jfull_bar[0]), 1);
-      TileList list;
+      TileList<kDet ? kDetK / 256 : 1> list;
       list.init(a, n_rows);
       Tile x{};
       for (uint32_t i = 0; x.kind >= 0; ++i) {
@@ -511,9 +537,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       return __shfl_sync(0xffffffffu, good, 0) != 0;
     };
     int seen_dh = -1, seen_dw = -1;   // last first chunks seen stored
-    // the tile's products, in order of ji
-    auto acc_full = [&](uint32_t ji) -> bool {
-      const uint32_t bar = smem_u32(&accf_bar[ji & 1u]), ph = (ji >> 1) & 1u;
+    uint32_t ai = 0;   // accumulators read
+    // the next accumulator's products
+    auto acc_full = [&]() -> bool {
+      const uint32_t bar = smem_u32(&accf_bar[ai & 1u]), ph = (ai >> 1) & 1u;
       if (pending != nullptr && !__all_sync(0xffffffffu, mbar_test_wait(bar, ph))) raise();
       const bool full = mbar_wait(bar, ph, abort_flag, a.err);
       tc_fence_after();
@@ -521,14 +548,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     };
     Tile x;
     for (uint32_t ji = 0; ok && next_tile(ji, x, true); ++ji) {
-      const uint32_t buf = ji & 1u;
-      const uint32_t taddr = tmem_base + lane_off + buf * 256 + hf * 128;
       const int r0 = static_cast<int>(rank) * 128 + q * 32;   // this warp's first row of the tile
+      auto taddr = [&]() -> uint32_t { return tmem_base + lane_off + (ai & 1u) * 256 + hf * 128; };
       // accumulator read out: one arrival per warp hands it back
       auto release_acc = [&]() {
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster_relaxed(acce_lead0 + buf * 8);
+        if (lane == 0) mbar_arrive_cluster_relaxed(acce_lead0 + (ai & 1u) * 8);
+        ++ai;
       };
       if (x.kind == kTileZ) {
         const int row = x.t * 256 + r0 + lane;
@@ -547,7 +574,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int nvalid = in ? V - vbase : 0;
         // the buffer's previous chunk must have been read
         if (x.need > 0 && !(ok = wait_count(cdone + x.chunk - a.n_buf, x.need))) break;
-        if (!(ok = acc_full(ji))) break;
+        if (!(ok = acc_full())) break;
         const int p0 = (x.v - x.v0) * 4 + hf * 2;
         const int gy = (x.buf * a.buf_panels + p0) * a.panel_rows + (x.t - x.t0) * 256 + r0;
 #pragma unroll 1
@@ -556,7 +583,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             float v[32];
-            tmem_ld32(taddr + c * 64 + u * 32, v);
+            tmem_ld32(taddr() + c * 64 + u * 32, v);
             const int lxc = lx - c * 64 - u * 32;
             const int nv = nvalid - c * 64 - u * 32;
             auto p_of = [&](int j) -> float {   // g without the target's term
@@ -600,9 +627,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
       const bool dh = x.kind == kTileDH;
       const bool empty = !dh && n_rows == 0;   // dW of no rows: zeros, no products
-      if (!(ok = acc_full(ji))) break;
-      // the products have read the chunk buffer
-      if (leader && warp == 2 && lane == 0) red_add_release_gpu(cdone + x.chunk, 1u);
       const int w = tile_w(x.h);
       const int y = (dh ? x.t : x.v) * 256 + r0;
       const bool rows_in = y < (dh ? n_rows : V);
@@ -612,48 +636,71 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       // step, so the wait is a formality
       const bool first = x.order == 0 && (dh || !a.add_dw);
       uint32_t* turn = nullptr;
-      if (a.det_turns) {
-        // reproducible sums: the contributions to a slab take turns in chunk order
-        const int n_h = (H + 255) / 256;
-        const int64_t tile = static_cast<int64_t>(dh ? x.t : a.max_t + x.v) * n_h + x.h;
-        turn = a.det_turns + tile * (2 * kEpiWarps) + slab;
-        if (!(ok = wait_count(turn, x.order))) break;
-      } else if (x.first > 0) {
-        const int c0 = dh ? x.chunk - x.order : x.chunk - x.order * n_vc;
-        int& seen = dh ? seen_dh : seen_dw;
-        if (seen != c0) {
-          if (!(ok = wait_count((dh ? dh_first : dw_first) + c0, x.first))) break;
-          seen = c0;
+      const int n_term = kDet ? max(1, (x.nk + kDetK / kBK - 1) / (kDetK / kBK)) : 1;
+      for (int term = 0; ok && term < n_term; ++term) {
+        if (!(ok = acc_full())) break;
+        // the products have read the chunk buffer
+        if (term == n_term - 1 && leader && warp == 2 && lane == 0) red_add_release_gpu(cdone + x.chunk, 1u);
+        if (term == 0) {
+          if constexpr (kDet) {
+            // reproducible sums: the contributions to a slab take turns in chunk order
+            const int n_h = (H + 255) / 256;
+            const int64_t tile = static_cast<int64_t>(dh ? x.t : a.max_t + x.v) * n_h + x.h;
+            turn = a.det_turns + tile * (2 * kEpiWarps) + slab;
+            if (!(ok = wait_count(turn, x.order))) break;
+          } else if (x.first > 0) {
+            const int c0 = dh ? x.chunk - x.order : x.chunk - x.order * n_vc;
+            int& seen = dh ? seen_dh : seen_dw;
+            if (seen != c0) {
+              if (!(ok = wait_count((dh ? dh_first : dw_first) + c0, x.first))) break;
+              seen = c0;
+            }
+          }
         }
-      }
+        const bool store = first && term == 0;
 #pragma unroll 1
-      for (int s = 0; s < 4; ++s) {
-        const int col = hf * 128 + s * 32;
-        if (col >= w) break;
-        float v[32];
-        tmem_ld32(taddr + s * 32, v);
-        if (empty) {
+        for (int s = 0; s < 4; ++s) {
+          const int col = hf * 128 + s * 32;
+          if (col >= w) break;
+          float v[32];
+          tmem_ld32(taddr() + s * 32, v);
+          if (empty) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = 0.f;
+            for (int j = 0; j < 32; ++j) v[j] = 0.f;
+          }
+          if (kDet && store) {
+            // what adding to +0 would leave: no negative zeros
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = __fadd_rn(v[j], 0.f);
+          }
+          if (s == 3 || col + 32 >= w) release_acc();
+          if (s == 0) raise();
+          box_free();
+          write_box32(box, lane, v);
+          fence_proxy_async_smem();
+          if (term > 0 && lane == 0) {
+            // this warp's box of the term before is in the sum
+            if (w - hf * 128 >= 128)
+              bulk_wait_group<3>();
+            else
+              bulk_wait_group<0>();
+            fence_proxy_async_global();
+          }
+          __syncwarp();
+          if (lane == 0 && rows_in) {
+            if (store)
+              tma_store_2d(map, box, x.h * 256 + col, y);
+            else
+              tma_reduce_add_2d(map, box, x.h * 256 + col, y);
+          }
+          if (lane == 0) bulk_commit_group();
         }
-        if (s == 3 || col + 32 >= w) release_acc();
-        if (s == 0) raise();
-        box_free();
-        write_box32(box, lane, v);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0 && rows_in) {
-          if (first)
-            tma_store_2d(map, box, x.h * 256 + col, y);
-          else
-            tma_reduce_add_2d(map, box, x.h * 256 + col, y);
-        }
-        if (lane == 0) bulk_commit_group();
+        if (hf * 128 >= w) release_acc();   // no columns for this warp
       }
-      if (hf * 128 >= w) release_acc();   // no columns for this warp
+      if (!ok) break;
       raise();
-      if (turn == nullptr && first) pending = dh ? dh_first + x.chunk : dw_first + x.chunk;
-      if (turn != nullptr) {
+      if (!kDet && first) pending = dh ? dh_first + x.chunk : dw_first + x.chunk;
+      if constexpr (kDet) {
         if (lane == 0) {
           bulk_wait_group<0>();
           fence_proxy_async_global();
@@ -680,7 +727,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 }  // namespace
 
 cudaError_t launch_lmhead_bwd_chunk(const ChunkMaps& m, const ChunkArgs& a, int n_ctas, cudaStream_t s) {
-  auto* k = a.ecoef != nullptr ? &lmhead_bwd_chunk_kernel<true> : &lmhead_bwd_chunk_kernel<false>;
+  const bool ent = a.ecoef != nullptr;
+  auto* k = a.det_turns != nullptr ? (ent ? &lmhead_bwd_chunk_kernel<true, true> : &lmhead_bwd_chunk_kernel<false, true>)
+                                   : (ent ? &lmhead_bwd_chunk_kernel<true, false> : &lmhead_bwd_chunk_kernel<false, false>);
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
   k<<<n_ctas / 2 * 2, kThreads, kSmemBytes, s>>>(m, a);

@@ -55,15 +55,21 @@ constexpr uint32_t kIdesc = idesc_bf16_f32(256, 256, false, false);
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
+template <bool kOrdered>
 __device__ __forceinline__ void split_range(int s, int S, int n_vt, int& vt0, int& vt1) {
-  const int per = n_vt / S, more = n_vt - per * S;   // the first `more` splits take one tile more
-  vt0 = s * per + min(s, more);
-  vt1 = vt0 + per + (s < more ? 1 : 0);
+  if constexpr (kOrdered) {
+    vt0 = static_cast<int>(static_cast<int64_t>(s) * n_vt / S);
+    vt1 = static_cast<int>(static_cast<int64_t>(s + 1) * n_vt / S);
+  } else {
+    const int per = n_vt / S, more = n_vt - per * S;   // the first `more` splits take one tile more
+    vt0 = s * per + min(s, more);
+    vt1 = vt0 + per + (s < more ? 1 : 0);
+  }
 }
 
 // Running statistics of one row.  q2 is in log2 units: q2 = sum e (z - m) log2(e).
 // s is summed with its rounding carried along in c (Kahan), so that log s hardly
-// depends on how the columns are split.
+// depends on how the columns are split; in the ordered sums it is not (c stays 0).
 struct Stats {
   float m = -INFINITY, s = 0.f, c = 0.f, q2 = 0.f;
   __device__ __forceinline__ void raise(float cmax) {
@@ -78,33 +84,44 @@ struct Stats {
       m = cmax;
     }
   }
+  template <bool kOrdered>
   __device__ __forceinline__ void add(float ds, float dq) {
-    const float y = ds - c, t = s + y;
-    c = (t - s) - y;
-    s = t;
+    if constexpr (kOrdered) {
+      s += ds;
+    } else {
+      const float y = ds - c, t = s + y;
+      c = (t - s) - y;
+      s = t;
+    }
     q2 += dq;
   }
 };
 
 // fold 32 logits (all columns valid) into the row's statistics
+template <bool kOrdered>
 __device__ __forceinline__ void fold_full(const float (&v)[32], Stats& r) {
   float cm[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
   for (int j = 4; j < 32; ++j) cm[j & 3] = fmaxf(cm[j & 3], v[j]);
   r.raise(fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3])));
   const float mL = r.m * kLog2e;
+  constexpr int kSums = kOrdered ? 2 : 4;
   float s[4] = {0.f, 0.f, 0.f, 0.f}, q[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
     const float y = fmaf(v[j], kLog2e, -mL);
     const float e = ex2_approx(y);
-    s[j & 3] += e;
-    q[j & 3] = fmaf(e, y, q[j & 3]);
+    s[j % kSums] += e;
+    q[j % kSums] = fmaf(e, y, q[j % kSums]);
   }
-  r.add((s[0] + s[1]) + (s[2] + s[3]), (q[0] + q[1]) + (q[2] + q[3]));
+  if constexpr (kOrdered)
+    r.add<true>(s[0] + s[1], q[0] + q[1]);
+  else
+    r.add<false>((s[0] + s[1]) + (s[2] + s[3]), (q[0] + q[1]) + (q[2] + q[3]));
 }
 
 // same for a chunk where only the first `nv` (1..31) columns are valid
+template <bool kOrdered>
 __device__ __forceinline__ void fold_partial(const float (&v)[32], int nv, Stats& r) {
   float cmax = v[0];
 #pragma unroll
@@ -112,7 +129,7 @@ __device__ __forceinline__ void fold_partial(const float (&v)[32], int nv, Stats
     if (j < nv) cmax = fmaxf(cmax, v[j]);
   r.raise(cmax);
   const float mL = r.m * kLog2e;
-  float s = 0.f, q = 0.f;
+  float s = kOrdered ? r.s : 0.f, q = kOrdered ? r.q2 : 0.f;
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
     if (j < nv) {
@@ -122,7 +139,12 @@ __device__ __forceinline__ void fold_partial(const float (&v)[32], int nv, Stats
       q = fmaf(e, y, q);
     }
   }
-  r.add(s, q);
+  if constexpr (kOrdered) {
+    r.s = s;
+    r.q2 = q;
+  } else {
+    r.add<false>(s, q);
+  }
 }
 
 // unit u of the list: 256-row token tile and vocab split
@@ -134,6 +156,14 @@ __device__ __forceinline__ void unit_of(int u, int n_mt, int S, int& mt, int& s)
   mt = g * kGroup + (r - s * g_mt);
 }
 
+// kOrdered: the sums of the reproducible loss call.  Its results stay the same bits
+// from one version of the library to the next, so a row's columns are summed one
+// after the other by one thread (the four warps of the lower column half take all
+// 256 columns, the others none), uncompensated, in the splits of ordered_splits
+// (api.cu) and merged in their order.  T = 16384, V = 65536: 0.49 against
+// 0.38 ms at H = 256, 0.73 and 0.62 at H = 512, 1.33 and 1.21 at H = 1024; at H = 4096
+// the products hide it (4.94 and 4.93).
+template <bool kOrdered>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     lmhead_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
                       const FwdArgs a) {
@@ -141,7 +171,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) uint64_t full_bar[kStages];    // even CTA: both CTAs' bytes land here
   __shared__ __align__(8) uint64_t empty_bar[kStages];   // both CTAs
   __shared__ __align__(8) uint64_t accf_bar[2];          // both CTAs: accumulator full
-  __shared__ __align__(8) uint64_t acce_bar[2];          // even CTA: one arrival per epilogue warp of the pair
+  __shared__ __align__(8) uint64_t acce_bar[2];          // even CTA: one arrival per reading warp of the pair
   __shared__ __align__(8) uint64_t ufull_bar[kSlots];    // both CTAs: unit index written
   __shared__ __align__(8) uint64_t uempty_bar[kSlots];   // even CTA: every reader of both CTAs has it
   __shared__ __align__(8) uint64_t hfull_bar[4], hempty_bar[4];   // the upper column half's (m, s, q) written / read
@@ -164,7 +194,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&accf_bar[b]), 1);
-      mbar_init(smem_u32(&acce_bar[b]), 2 * kEpiWarps);
+      mbar_init(smem_u32(&acce_bar[b]), kOrdered ? kEpiWarps : 2 * kEpiWarps);
     }
     for (int s = 0; s < kSlots; ++s) {
       mbar_init(smem_u32(&ufull_bar[s]), 1);
@@ -219,7 +249,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (uint32_t ui = 0; u >= 0 && ok; ++ui) {
         int mt, s, vt0, vt1;
         unit_of(u, n_mt, S, mt, s);
-        split_range(s, S, a.n_vtiles, vt0, vt1);
+        split_range<kOrdered>(s, S, a.n_vtiles, vt0, vt1);
         for (int vt = vt0; vt < vt1 && ok; ++vt) {
           const int y = (is_a ? mt : vt) * 256 + static_cast<int>(rank) * 128;
           for (int kb = 0; kb < kblocks; ++kb) {
@@ -252,7 +282,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (uint32_t ui = 0; u >= 0 && ok; ++ui) {
         int mt, s, vt0, vt1;
         unit_of(u, n_mt, S, mt, s);
-        split_range(s, S, a.n_vtiles, vt0, vt1);
+        split_range<kOrdered>(s, S, a.n_vtiles, vt0, vt1);
         for (int vt = vt0; vt < vt1 && ok; ++vt) {
           const uint32_t buf = acc_it & 1u;
           if (!(ok = mbar_wait(smem_u32(&acce_bar[buf]), ((acc_it >> 1) & 1u) ^ 1u, abort_flag, a.err))) break;
@@ -313,6 +343,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // epilogue: warp w may read TMEM lanes [32 (w % 4), 32 (w % 4) + 32)
     const int q = warp & 3;
     const int hf = (warp - 2) >> 2;
+    constexpr int kCols = kOrdered ? 256 : 128;   // columns of a tile that one warp reads
     const int r_in_tile = static_cast<int>(rank) * 128 + q * 32 + lane;
     const uint32_t acce_lead0 = mapa_shared(smem_u32(&acce_bar[0]), 0);
     uint32_t acc_it = 0;
@@ -322,9 +353,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (lane == 0) u = next_unit(ui);
       u = __shfl_sync(0xffffffffu, u, 0);
       if (u < 0) break;
+      if (kOrdered && hf == 1) continue;
       int mt, s, vt0, vt1;
       unit_of(u, n_mt, S, mt, s);
-      split_range(s, S, a.n_vtiles, vt0, vt1);
+      split_range<kOrdered>(s, S, a.n_vtiles, vt0, vt1);
       const int row = mt * 256 + r_in_tile;
       const bool valid = row < n_rows;
       const int x = valid ? a.tok_p[row] : -1;
@@ -336,11 +368,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (!(ok = mbar_wait(smem_u32(&accf_bar[buf]), (acc_it >> 1) & 1u, abort_flag, a.err))) break;
         tc_fence_after();
         const int col0 = vt * 256 + hf * 128;
-        const int ncols = min(128, a.V - col0);   // may be <= 0 in the last tile
+        const int ncols = min(kCols, a.V - col0);   // may be <= 0 in the last tile
         const int lx = x - col0;
         const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * 256 + hf * 128;
 #pragma unroll 1
-        for (int c0 = 0; c0 < 128; c0 += 32) {
+        for (int c0 = 0; c0 < kCols; c0 += 32) {
           if (c0 >= ncols) break;
           float v[32];
           tmem_ld32(taddr + c0, v);
@@ -352,9 +384,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             found = true;
           }
           if (c0 + 32 <= ncols)
-            fold_full(v, st);
+            fold_full<kOrdered>(v, st);
           else
-            fold_partial(v, ncols - c0, st);
+            fold_partial<kOrdered>(v, ncols - c0, st);
         }
         // every lane's TMEM reads are complete: one arrival per warp hands it back
         tc_fence_before();
@@ -364,6 +396,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
       if (valid && found) a.zx[row] = zxv;
+      if constexpr (kOrdered) {
+        if (valid) a.part[static_cast<int64_t>(s) * a.rows_cap + row] = make_float4(st.m, st.s, st.q2 * kLn2, 0.f);
+        continue;
+      }
       // the two warps of a lane quarter put their column halves together
       if (hf == 1) {
         if (!(ok = mbar_wait(smem_u32(&hempty_bar[q]), (ui & 1u) ^ 1u, abort_flag, a.err))) break;
@@ -409,17 +445,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 cudaError_t launch_lmhead_fwd(const CUtensorMap& tm_h, const CUtensorMap& tm_w, const FwdArgs& a, int grid,
                               cudaStream_t s) {
   // the shared-memory attribute is per device: set it on each device once
-  static std::atomic<unsigned long long> attr_set{0};
+  static std::atomic<unsigned long long> attr_set[2] = {};
+  auto* const k = a.ordered ? &lmhead_fwd_kernel<true> : &lmhead_fwd_kernel<false>;
+  auto& set = attr_set[a.ordered ? 1 : 0];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
-  if ((attr_set.load(std::memory_order_acquire) & bit) == 0) {
-    e = cudaFuncSetAttribute(lmhead_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+  if ((set.load(std::memory_order_acquire) & bit) == 0) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    attr_set.fetch_or(bit, std::memory_order_release);
+    set.fetch_or(bit, std::memory_order_release);
   }
-  lmhead_fwd_kernel<<<grid / 2 * 2, kThreads, kSmemBytes, s>>>(tm_h, tm_w, a);
+  k<<<grid / 2 * 2, kThreads, kSmemBytes, s>>>(tm_h, tm_w, a);
   return cudaGetLastError();
 }
 

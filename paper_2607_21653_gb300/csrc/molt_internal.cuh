@@ -63,6 +63,7 @@ struct FwdArgs {
   int V, H;
   int n_split;
   int n_vtiles;
+  bool ordered;         // the reproducible loss call's sums: columns in order, by ordered_splits
   int32_t* next_unit;   // zeroed
   float4* part;         // [n_split, rows_cap]
   float* zx;
@@ -139,6 +140,7 @@ unsigned* device_status_word(molt_status* st);   // current device's status word
 int device_sm_count();                           // current device's SM count
 // vocab splits of the forward pass over Tcap packed rows
 int forward_splits(int64_t Tcap, int64_t H, int64_t V, int n_sm);
+int ordered_splits(int64_t Tcap, int64_t V, int n_sm);   // the reproducible loss call's
 molt_status encode_tmap_2d(CUtensorMap* m, CUtensorMapDataType dt, int elem_bytes, const void* base, uint64_t rows,
                            uint64_t cols, uint32_t box_cols, uint32_t box_rows);
 
@@ -162,8 +164,9 @@ struct ZeroRows {
 cudaError_t launch_pack(const uint8_t* mask, int T, int H, const uint16_t* hidden, const int32_t* tokens, const float* b,
                         const float* adv, int tok_shift, const Workspace& ws, const ZeroRows& z, int64_t ctl_words,
                         int n_sm, cudaStream_t s);
-// lp_p, ent_p: packed log-probs and entropies for the extended objective, or nullptr
-cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
+// ordered: a row's splits are merged one after the other; lp_p, ent_p: packed
+// log-probs and entropies for the extended objective, or nullptr
+cudaError_t launch_merge(bool loss_mode, bool ordered, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
                          const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, float* lp_p,
                          float* ent_p, unsigned* err, cudaStream_t s);
 // the loss and stats, and the list of the rows with a gradient, with pad > 0 packed

@@ -590,13 +590,30 @@ __device__ __forceinline__ void reduce_loss(int n, double denom, const int32_t* 
                                             unsigned* err) {
   static_assert(kFinSlots == kPackThreads / 32, "a warp to each slot");
   __shared__ double tot[kFinSlots];
-  const int n_rt = (n + kRedRows - 1) / kRedRows;
+  const int n_rt = (n + kRedRows - 1) / kRedRows, n_tiles = (n_rt + 3) / 4;
   const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  // In the order in which these sums have always been taken, so that the loss and
+  // the stats stay the same bits: four sets of rows to a tile of 128, tile i to
+  // column i % 1024, the columns 32 at a time by a shuffle tree (here 32 kBatch at
+  // a time), and those 32 totals by another.
+  auto join = [&](double x, double y) { return q == 3 ? fmax(x, y) : x + y; };
+  auto part = [&](int r) { return r < n_rt ? red[(int64_t)r * kRedSlots + q] : 0.0; };
+  constexpr int kBatch = 4;
   double a = 0.0;
-#pragma unroll 8
-  for (int b = lane; b < n_rt; b += 32) {
-    const double x = red[(int64_t)b * kRedSlots + q];
-    a = (q == 3) ? fmax(a, x) : a + x;
+  for (int w = 0; w < 32 && 32 * w < n_tiles; w += kBatch) {
+    double x[kBatch] = {};
+    for (int base = 32 * w + lane; base < n_tiles; base += 1024) {
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int r = 4 * (base + 32 * i);
+        x[i] = join(x[i], join(join(part(r), part(r + 1)), join(part(r + 2), part(r + 3))));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const double total = q == 3 ? warp_max(x[i]) : warp_sum(x[i]);
+      if (lane == w + i) a = total;
+    }
   }
   a = (q == 3) ? warp_max(a) : warp_sum(a);
   if (lane == 0) tot[q] = a;
@@ -777,13 +794,15 @@ cudaError_t launch_pack(const uint8_t* mask, int T, int H, const uint16_t* hidde
   return cudaGetLastError();
 }
 
-cudaError_t launch_merge(bool loss_mode, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
+cudaError_t launch_merge(bool loss_mode, bool ordered, int Tcap, int V, int n_parts, double denom, float clip_lo, float clip_hi,
                          const Workspace& ws, float* logp_out, float* ent_out, float* tokloss_out, float* lp_p,
                          float* ent_p, unsigned* err, cudaStream_t s) {
   const int blocks = Tcap / kRedRows;
   if (blocks == 0) return cudaSuccess;
-  const int groups = merge_groups(n_parts);
-  auto* k = groups == kMergeGroupsMany ? &merge_kernel<kMergeGroupsMany> : &merge_kernel<kMergeGroupsFew>;
+  const int groups = ordered ? 1 : merge_groups(n_parts);
+  auto* k = groups == 1                  ? &merge_kernel<1>
+            : groups == kMergeGroupsMany ? &merge_kernel<kMergeGroupsMany>
+                                         : &merge_kernel<kMergeGroupsFew>;
   k<<<blocks, kRedRows * groups, 0, s>>>(loss_mode ? 1 : 0, Tcap, V, n_parts, denom, clip_lo, clip_hi, ws.counts,
                                          ws.row_map, ws.tok_p, ws.b_p, ws.adv_p, ws.part, ws.zx, ws.lse, ws.coef,
                                          ws.red, logp_out, ent_out, tokloss_out, lp_p, ent_p, err);
