@@ -17,7 +17,9 @@
  *     mask, unsorted group ids, a pipeline wait that timed out) set bits of a
  *     per-device status word that molt_device_status() reads and clears.
  *   - Workspace: calls that need scratch memory take (workspace, bytes).  The
- *     size comes from the matching *_workspace_bytes() query.  Passing NULL
+ *     size comes from the matching *_workspace_bytes() query and does not fall as
+ *     T grows (other arguments the same): a buffer for the largest T serves every
+ *     smaller one.  Passing NULL
  *     makes the call allocate and free it stream-ordered (cudaMallocAsync).
  *   - The library keeps no state between calls except cached device
  *     properties, the per-device status word, the kernel-launch counter, the

@@ -145,7 +145,6 @@ struct ChunkPlan {
   int64_t panel_rows = 0, buf_panels = 0;   // of one chunk buffer: token rows of a panel, 64-column panels
   int n_buf = 0;
   int64_t g_rows() const { return n_buf * buf_panels * panel_rows; }
-  size_t g_bytes() const { return use ? static_cast<size_t>(g_rows()) * kBK * 2 : 0; }
   int64_t ctl_words() const { return use ? kChunkCtlHead + 4 * max_chunks : 0; }
   int64_t turn_words() const { return use ? (n_t + n_v) * n_h * 16 : 0; }
   // list steps between a chunk's logit tiles and those that read them
@@ -230,14 +229,6 @@ ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V, bool det) {
   return p;
 }
 
-struct Layout {
-  size_t counts, row_map, pos, tok_p, b_p, adv_p, h_p, part, zx, lse, coef, tile_list, red, dh32, turns, g, ctl;
-  size_t lp_p, ent_p, ecoef, mu, gate_p;
-  size_t live_of, h_l, tok_l, lse_l, coef_l, ecoef_l, mu_l, total;
-};
-
-constexpr size_t kNoRegion = ~size_t(0);   // a Layout region that is not allocated
-
 // turn counters of the deterministic schedule: an abort word (padded to 64
 // words), then [token quads, H jobs, 32] for dhidden and [vocab blocks, H jobs,
 // 32] for dW
@@ -255,7 +246,45 @@ TurnLayout turn_layout(int64_t Tcap, int64_t H, int64_t V) {
   return t;
 }
 
-Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = false) {
+// What the workspace holds for the backward over chunks.  Chunk shapes and buffers
+// follow the call's size, so what a call uses can shrink as T or V grows; what is
+// reserved never does, so that a workspace for the largest T serves every smaller one.
+// (Up to 16 buffers of at most 16 x 16 tiles, 512 tiles together; chunks of at least
+// 4 x 4.  Calls of other sizes than chunk_plan takes reserve nothing, except the
+// reproducible ones that it sends to the cluster kernel from a T on.)
+struct ChunkReserve {
+  size_t g = 0, ctl = 0, turns = 0;   // bytes
+};
+ChunkReserve chunk_reserve(int64_t T, int64_t H, int64_t V, bool det) {
+  ChunkReserve r;
+  const int64_t n_t = (T + 255) / 256, n_v = (V + 255) / 256;
+  const ChunkPlan plain = chunk_plan(T, H, V, false), p = chunk_plan(T, H, V, det);
+  if (plain.use || p.use) {
+    r.g = static_cast<size_t>(std::min<int64_t>(512, 16 * std::min<int64_t>(n_t, 16) * std::min<int64_t>(n_v, 16))) *
+          (256 * 256 * 2);
+    r.ctl = static_cast<size_t>(kChunkCtlHead + 4 * ((n_t + 3) / 4) * ((n_v + 3) / 4)) * 4;
+  }
+  if (det)
+    r.turns = static_cast<size_t>(std::max(plain.turn_words(), turn_layout(round_tiles(T), H, V).words)) * 4;
+  return r;
+}
+
+// Rows of split partials that a workspace holds: no fewer than the splits of
+// forward_splits or ordered_splits times their rows, and never fewer for a larger T.
+int64_t part_rows(int64_t Tcap, int64_t V, int n_sm) {
+  const int64_t n_vt = (V + kFwdBN - 1) / kFwdBN, n_mt = (Tcap + 255) / 256;
+  return std::min(n_vt * n_mt, 24 * int64_t(n_sm / 2) + n_mt) * 256;
+}
+
+struct Layout {
+  size_t counts, row_map, pos, tok_p, b_p, adv_p, h_p, part, zx, lse, coef, tile_list, red, dh32, turns, g, ctl;
+  size_t lp_p, ent_p, ecoef, mu, gate_p;
+  size_t live_of, h_l, tok_l, lse_l, coef_l, ecoef_l, mu_l, total;
+};
+
+constexpr size_t kNoRegion = ~size_t(0);   // a Layout region that is not allocated
+
+Layout layout(int64_t T, int64_t H, int64_t V, int n_sm, bool with_bwd, bool det = false) {
   const int64_t Tcap = round_tiles(T);
   const int64_t ntile = Tcap / kTileM;
   Layout L{};
@@ -272,19 +301,17 @@ Layout layout(int64_t T, int64_t H, int64_t V, int S, bool with_bwd, bool det = 
   L.b_p = take(Tcap * 4);
   L.adv_p = take(Tcap * 4);
   L.h_p = take(Tcap * H * 2);
-  L.part = take(static_cast<size_t>(S) * Tcap * 16);
+  L.part = take(static_cast<size_t>(part_rows(Tcap, V, n_sm)) * 16);
   L.zx = take(Tcap * 4);
   L.lse = take(Tcap * 4);
   L.coef = take(Tcap * 4);
   L.tile_list = take(ntile * 4);
   L.red = take(Tcap / kRedRows * kRedSlots * 8);
   L.dh32 = with_bwd ? take(static_cast<size_t>(Tcap) * H * 4) : o;
-  const ChunkPlan cp = chunk_plan(T, H, V, det);
-  L.turns = (with_bwd && det)
-                ? take(static_cast<size_t>(cp.use ? cp.turn_words() : turn_layout(Tcap, H, V).words) * 4)
-                : kNoRegion;
-  L.g = with_bwd ? take(cp.g_bytes()) : o;
-  L.ctl = with_bwd ? take(static_cast<size_t>(cp.ctl_words()) * 4) : o;
+  const ChunkReserve cr = chunk_reserve(T, H, V, det);
+  L.turns = (with_bwd && det) ? take(cr.turns) : kNoRegion;
+  L.g = with_bwd ? take(cr.g) : o;
+  L.ctl = with_bwd ? take(cr.ctl) : o;
   L.lp_p = with_bwd ? take(Tcap * 4) : o;
   L.ent_p = with_bwd ? take(Tcap * 4) : o;
   L.ecoef = with_bwd ? take(Tcap * 4) : o;
@@ -348,9 +375,9 @@ Layout vp_backward_layout(int64_t T, int64_t H, int64_t V) {
   L.lse_l = take(Tcap * 4);
   L.coef_l = take(Tcap * 4);
   L.dh32 = take(static_cast<size_t>(Tcap) * H * 4);
-  const ChunkPlan cp = chunk_plan(T, H, V, false);
-  L.g = take(cp.g_bytes());
-  L.ctl = take(static_cast<size_t>(cp.ctl_words()) * 4);
+  const ChunkReserve cr = chunk_reserve(T, H, V, false);
+  L.g = take(cr.g);
+  L.ctl = take(cr.ctl);
   L.row_map = L.pos = L.tok_p = L.b_p = L.adv_p = L.h_p = L.part = L.zx = L.lse = L.coef = L.red =
       L.lp_p = L.ent_p = L.ecoef = L.mu = L.gate_p = L.ecoef_l = L.mu_l = o;
   L.turns = kNoRegion;
@@ -812,7 +839,7 @@ molt_status policy_loss_impl(const uint16_t* hidden, const uint16_t* W, const in
                   "det_clusters must be 0 or a multiple of 4 from 4 to " + std::to_string(n_det));
     n_det = want;
   }
-  const Layout L = layout(T, H, V, S, true, det);
+  const Layout L = layout(T, H, V, di->n_sm, true, det);
   Scratch sc;
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
@@ -1042,8 +1069,7 @@ size_t molt_token_logprobs_workspace_bytes(int64_t T, int64_t H, int64_t V) {
   molt_status st;
   const DeviceInfo* di = device_info(&st);
   const int n_sm = di ? di->n_sm : 152;
-  const int64_t Tcap = round_tiles(T);
-  return layout(T, H, V, forward_splits(Tcap > 0 ? Tcap : kTileM, H, V, n_sm), false).total;
+  return layout(T, H, V, n_sm, false).total;
 }
 
 size_t molt_policy_loss_workspace_bytes(int64_t T, int64_t H, int64_t V) {
@@ -1051,8 +1077,7 @@ size_t molt_policy_loss_workspace_bytes(int64_t T, int64_t H, int64_t V) {
   molt_status st;
   const DeviceInfo* di = device_info(&st);
   const int n_sm = di ? di->n_sm : 152;
-  const int64_t Tcap = round_tiles(T);
-  return layout(T, H, V, forward_splits(Tcap > 0 ? Tcap : kTileM, H, V, n_sm), true).total;
+  return layout(T, H, V, n_sm, true).total;
 }
 
 size_t molt_policy_loss_workspace_bytes_ex(int64_t T, int64_t H, int64_t V, const molt_loss_options* opts) {
@@ -1062,9 +1087,7 @@ size_t molt_policy_loss_workspace_bytes_ex(int64_t T, int64_t H, int64_t V, cons
   molt_status st;
   const DeviceInfo* di = device_info(&st);
   const int n_sm = di ? di->n_sm : 152;
-  const int64_t Tcap = round_tiles(T);
-  const int64_t rows = std::max<int64_t>(Tcap, kTileM);
-  return layout(T, H, V, det ? ordered_splits(rows, V, n_sm) : forward_splits(rows, H, V, n_sm), true, det).total;
+  return layout(T, H, V, n_sm, true, det).total;
 }
 
 molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, const int32_t* tokens,
@@ -1080,7 +1103,7 @@ molt_status molt_token_logprobs_fwd(const uint16_t* hidden, const uint16_t* W, c
   if (!di) return st;
   const int64_t Tcap = round_tiles(T);
   const int S = forward_splits(Tcap, H, V, di->n_sm);
-  const Layout L = layout(T, H, V, S, false);
+  const Layout L = layout(T, H, V, di->n_sm, false);
   Scratch sc;
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);
@@ -1145,7 +1168,7 @@ molt_status molt_vp_partials(const uint16_t* hidden, const uint16_t* W_shard, co
   if (!di) return st;
   const int64_t Tcap = round_tiles(T);
   const int S = forward_splits(Tcap, H, V_shard, di->n_sm);
-  const Layout L = layout(T, H, V_shard, S, false);
+  const Layout L = layout(T, H, V_shard, di->n_sm, false);
   Scratch sc;
   MOLT_TRY(get_scratch(sc, workspace, workspace_bytes, L.total, stream));
   const Workspace w = carve(sc.ptr, L);

@@ -107,6 +107,28 @@ def test_workspace_query_with_options(lib):
     assert lib.molt_policy_loss_workspace_bytes_ex(1000, 192, 5000, ctypes.byref(det)) == 0
 
 
+# the lines of the rules that choose a kernel and its buffers lie at these H and V, and
+# between these T: chunk shapes, buffers and splits change there
+@pytest.mark.parametrize("H", [64, 128, 256, 320, 384, 512, 640, 1024, 1536, 4096])
+def test_workspace_never_shrinks_as_tokens_grow(lib, H):
+    """A buffer for the largest batch serves every smaller one."""
+    det = molt.LossOptions(0.0, 0.0, None, None, 0.0, 0.0, 1)
+    tokens = sorted({max(0, 128 * k + d) for k in (*range(0, 64), *range(64, 600, 7)) for d in (-1, 0, 1)})
+    for V in (1, 1000, 4096, 5000, 20480, 25600, 32000, 151936):
+        queries = {
+            "logprobs": lambda T: lib.molt_token_logprobs_workspace_bytes(T, H, V),
+            "loss": lambda T: lib.molt_policy_loss_workspace_bytes(T, H, V),
+            "loss, deterministic": lambda T: lib.molt_policy_loss_workspace_bytes_ex(T, H, V, ctypes.byref(det)),
+            "partials": lambda T: lib.molt_vp_partials_workspace_bytes(T, H, V),
+            "shard backward": lambda T: lib.molt_vp_backward_workspace_bytes(T, H, V),
+            "shard loss": lambda T: lib.molt_vp_loss_workspace_bytes(T),
+        }
+        for name, query in queries.items():
+            sizes = [query(T) for T in tokens]
+            falls = [(a, b) for a, b, x, y in zip(tokens, tokens[1:], sizes, sizes[1:]) if y < x]
+            assert not falls, (name, H, V, falls[:3])
+
+
 def test_header_compiles_as_c(tmp_path):
     """include/molt.h is a C header: it compiles with a C11 compiler and -pedantic."""
     import shutil
