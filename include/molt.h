@@ -87,6 +87,26 @@ int molt_version(void);
  * enqueue).  For launch accounting in benchmarks and tests. */
 uint64_t molt_kernel_launches(void);
 
+/* The backward that a loss call of this size runs on the current device (a shard's
+ * backward with V = V_shard and deterministic = 0), for benchmarks and tests.
+ *   kernel   one of MOLT_BWD_*: a single CTA per 128 x 256 unit, clusters of four per
+ *            512 x 512 unit (beside them, on some sizes, the former on the SMs that no
+ *            cluster can use), or CTA pairs over chunks of the plane
+ *   chunk_tokens, chunk_columns, buffers, lag   (MOLT_BWD_CHUNKS, else 0) the most that
+ *            a chunk holds, the ring's buffers, and how many chunks the products that
+ *            read a chunk stand behind those that form it */
+#define MOLT_BWD_SINGLE 0
+#define MOLT_BWD_CLUSTERS 1
+#define MOLT_BWD_CHUNKS 2
+typedef struct {
+  int kernel;
+  int chunk_tokens;
+  int chunk_columns;
+  int buffers;
+  int lag;
+} molt_backward_info;
+molt_status molt_backward_plan(int64_t T, int64_t H, int64_t V, int deterministic, molt_backward_info* out);
+
 /* Self-test of the device-side wait bound (no paper counterpart).  One warp
  * waits, exactly as the deterministic backward's turn waits do, on a counter
  * that nothing raises: the wait gives up after its time limit (about 4 s),

@@ -19,7 +19,7 @@ from concurrent.futures import ThreadPoolExecutor
 __all__ = [
     "build", "load", "lib_path", "MoltError", "STATUS", "DEV_FLAGS", "group_advantages",
     "broadcast_advantages", "mask_count", "token_logprobs", "policy_loss_fwd_bwd", "device_status",
-    "token_logprobs_workspace_bytes", "policy_loss_workspace_bytes", "header_functions",
+    "token_logprobs_workspace_bytes", "policy_loss_workspace_bytes", "header_functions", "backward_plan",
     "vp_partials", "vp_loss", "vp_backward", "vocab_shard_bounds", "gather_shard_partials", "sum_dhidden",
     "policy_loss_vocab_parallel",
 ]
@@ -93,6 +93,12 @@ class MoltError(RuntimeError):
         self.status = status
 
 
+class BackwardInfo(ctypes.Structure):
+    """molt_backward_info: the backward kernel of a size and, over chunks, their plan."""
+    _fields_ = [(n, ctypes.c_int) for n in ("kernel", "chunk_tokens", "chunk_columns", "buffers", "lag")]
+
+
+BACKWARD_KERNELS = ("lmhead_bwd_kernel", "lmhead_bwd_quad_kernel", "lmhead_bwd_chunk_kernel")   # by MOLT_BWD_*
 _lib = None
 
 
@@ -126,6 +132,7 @@ def load():
         "molt_policy_loss_fwd_bwd_ex": (I32, [P, P, P, P, P, P, I64, I64, I64, F, F, D, P, P, P, P, I32, P, P,
                                                P, P, P, SZ, P]),
         "molt_set_timing_events": (None, [P, P, I32]),
+        "molt_backward_plan": (I32, [I64, I64, I64, I32, ctypes.POINTER(BackwardInfo)]),
         "molt_token_logprobs_fwd_noalloc": (I32, [P, P, P, P, I64, I64, I64, P, P, P]),
         "molt_vp_partials_workspace_bytes": (SZ, [I64, I64, I64]),
         "molt_vp_partials": (I32, [P, P, P, P, I64, I64, I64, I64, P, P, SZ, P]),
@@ -295,6 +302,15 @@ def selftest_wait_timeout(stream=None) -> None:
 def kernel_launches() -> int:
     """Process-wide number of kernels the library has enqueued so far."""
     return int(load().molt_kernel_launches())
+
+
+def backward_plan(T, H, V, deterministic=False) -> dict:
+    """The backward that a loss call of this size runs (molt_backward_plan); `kernel` by name."""
+    info = BackwardInfo()
+    _check(load().molt_backward_plan(T, H, V, 1 if deterministic else 0, ctypes.byref(info)))
+    out = {n: getattr(info, n) for n, _ in info._fields_}
+    out["kernel"] = BACKWARD_KERNELS[info.kernel]
+    return out
 
 
 def group_advantages(rewards, group_ids, eps: float = 1e-6, out=None, stream=None):

@@ -972,6 +972,23 @@ int molt_version(void) { return 1; }
 
 uint64_t molt_kernel_launches(void) { return molt::g_kernel_launches.load(std::memory_order_relaxed); }
 
+molt_status molt_backward_plan(int64_t T, int64_t H, int64_t V, int deterministic, molt_backward_info* out) {
+  if (!out) return fail(MOLT_ERR_INVALID_ARG, "out is NULL");
+  MOLT_TRY(check_shape(T, H, V));
+  if (deterministic && H % 128 != 0) return fail(MOLT_ERR_UNSUPPORTED_SHAPE, "deterministic mode needs H % 128 == 0");
+  molt_status st;
+  const DeviceInfo* di = device_info(&st);
+  const ChunkPlan p = chunk_plan(T, H, V, deterministic != 0);
+  *out = molt_backward_info{};
+  out->kernel = p.use ? MOLT_BWD_CHUNKS : H % 128 == 0 ? MOLT_BWD_CLUSTERS : MOLT_BWD_SINGLE;
+  if (!p.use) return MOLT_OK;
+  out->chunk_tokens = static_cast<int>(p.chunk_t * 256);
+  out->chunk_columns = static_cast<int>(p.chunk_v * 256);
+  out->buffers = p.n_buf;
+  out->lag = p.lag(H, (di ? di->n_sm : 152) / 2);
+  return MOLT_OK;
+}
+
 void molt_set_timing_events(cudaEvent_t* starts, cudaEvent_t* stops, int n) {
   t_ev_start = starts;
   t_ev_stop = stops;
