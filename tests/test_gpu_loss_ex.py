@@ -1,7 +1,7 @@
 """GPU parity of the extended objective (KL to a reference policy, entropy
 bonus, sequence-level importance gate; Sec. 4.5) against the fp64 oracle,
-through molt_policy_loss_fwd_bwd_ex, on both backward kernels (H a multiple of
-256 runs on CTA pairs, other H on single CTAs).
+through molt_policy_loss_fwd_bwd_ex, on the backward kernels that these sizes select:
+over chunks from H = 256 on, clusters of four at H = 128, single CTAs at H = 192.
 
 Gate cases are built so that no decision sits near a boundary: each sequence's
 mean log-ratio is placed at least 0.3 (in log space) from the band edges, and
@@ -226,9 +226,9 @@ def test_bad_options_rejected():
 
 
 # ----------------------------------------------------------- deterministic mode
-# (5000, 256, 9000): about 7 token quads (two groups of four) and 18 vocab
-# blocks (two per residue class on a GB300), so both reduction orders of the
-# schedule have more than one step
+# All on the backward over chunks (the cluster kernel's: test_gpu_bwd_cluster.py).
+# (5000, 256, 9000): about seven terms of 512 tokens in two chunks and 18 of 512
+# columns in nine, so both reduction orders have more than one step
 DET_SHAPES = [(1000, 256, 5000), (513, 512, 4133), (640, 768, 2304), (1, 256, 7), (5000, 256, 9000),
               (900, 384, 3000)]
 
@@ -260,10 +260,10 @@ def test_deterministic_mode_is_bitwise_reproducible(T, H, V):
 @pytest.mark.parametrize("T,H,V", [(5000, 256, 9000), (2100, 640, 20000)])
 def test_deterministic_mode_does_not_depend_on_the_cluster_count(T, H, V):
     """The reduction order of the deterministic schedule is fixed by the turn
-    counters (dW in token-quad order, dhidden in vocab-block order), not by which
-    cluster runs which unit: 4, 8 and 16 clusters give the bits of the default
-    count, although units, timing and the clusters' waits all change.  (2100,
-    640, 20000) has a 128-column last job and 40 vocab blocks."""
+    counters (dW in token order, dhidden in vocab order), not by which CTA pair runs
+    which tile: 4, 8 and 16 clusters' worth of SMs give the bits of the default
+    count, although tiles, timing and the waits all change.  (2100, 640, 20000) has a
+    128-column last H tile and ten chunks of the vocabulary."""
     rng = np.random.default_rng(T + H)
     h, W, x, m = random_problem(rng, T, H, V, mask_frac=0.25, w_std=0.05)
     m[0] = 1

@@ -1,8 +1,8 @@
 """Seeded shape fuzzing of the policy-loss call against the fp64 oracle: token
-counts that leave 1-3 tiles of the last quad empty, vocabularies with ragged
-512-column blocks, H from 256 (two jobs per unit) upward, both the cluster
-backward (H % 128 == 0, a last 128-column job when H % 256 == 128) and the
-single-CTA one, the deterministic schedule, and caller-provided workspaces."""
+counts and vocabularies that leave ragged tiles, terms and chunks, H from 256 upward
+(a last H tile of 128 columns when H % 256 == 128), whichever backward kernel a size
+selects (mostly the one over chunks), the deterministic schedule, the cluster kernel's
+vocabulary split, and caller-provided workspaces."""
 import ctypes
 
 import numpy as np
@@ -121,10 +121,10 @@ def test_vocab_split_with_side_kernel(V):
 
 @pytest.mark.parametrize("H,V", [(384, 3000), (640, 4133), (896, 18986)])
 def test_half_width_last_job(H, V):
-    """H % 256 == 128: the cluster backward's last dH / dW job is 128 columns
-    wide.  Parity with the oracle on the raster schedule (V = 18986 also splits
-    the vocabulary with the side kernel) and on the deterministic one, which is
-    bitwise reproducible."""
+    """H % 256 == 128: the last dH / dW tile is 128 columns wide.  Parity with the
+    oracle, reduce-adds in arrival order and in the reproducible one, on the backward
+    over chunks, which takes these sizes (the cluster kernel's last job:
+    test_gpu_bwd_cluster.py)."""
     T = 900
     rng = np.random.default_rng(H + V)
     h, W, x, m = random_problem(rng, T, H, V, mask_frac=0.25, w_std=0.05)
