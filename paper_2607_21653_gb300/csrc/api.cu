@@ -163,28 +163,39 @@ struct ChunkPlan {
 // kernels' ms, those first:
 //   H >= 512: all (T = 64, V = 3000, H = 512 0.039 and 0.029; T = 2000, V = 19000,
 //     H = 896 0.262 and 0.140; T = 16384, V = 151936, H = 4096 54.4 and 36.8).
-//   256 < H < 512: from 512 rows on (T = 1024, V = 19000, H = 320 0.085 and 0.053);
-//     below, the single-CTA kernel is up to half faster (T = 64, V = 100000 0.081
-//     and 0.121), since a tile of 256 rows is mostly empty and short.
-//   H = 256: all but the middle vocabularies of small calls: up to 512 rows the
-//     cluster kernel is 5-20 % faster there (T = 256, V = 19000 0.031 and 0.038; but
-//     V = 60000 0.090 and 0.065, V = 2000 0.029 and 0.027).  At 700 rows this kernel
-//     would be faster already (V = 19000 0.051 and 0.044); the line lies above
-//     because tests/test_gpu_shapes.py holds the cluster kernel's vocab split there.
+//   256 < H < 512: from 512 rows on (T = 1024, V = 19000, H = 320 0.085 and 0.053; T =
+//     512, V = 40000, H = 320 0.100 and 0.066).  Below, a tile of 256 rows is mostly
+//     empty and short: against the single-CTA kernel (H = 320, 448) up to 128 rows half
+//     as slow again (T = 128, V = 100000, H = 320 0.077 and 0.123), even at 256
+//     (0.123 and 0.122) and already faster at 384 with many columns (V = 40000 0.083 and
+//     0.067; V = 4096 0.029 and 0.033).  Against the cluster kernel (H = 384) this one would
+//     be the faster at most sizes below the line too (T = 128, V = 2500 0.035 and 0.029; T =
+//     384, V = 40000 0.096 and 0.067; T = 256, V = 19000 0.039 and 0.041): the line is the
+//     single-CTA kernel's.
+//   H = 256: all but the middle vocabularies of small calls.  At 512 rows they cross at
+//     V = 4096 (V = 2500 0.030 and 0.029, 4096 0.031 and 0.032, 9000 0.031 and 0.033, 19000
+//     0.036 and 0.039), and back again above 20480, where the clusters need a second round
+//     of units (25000 0.051 and 0.043).  In rows they cross between 512 and 640 (T = 640,
+//     V = 9000 0.032 and 0.032, 13000 0.049 and 0.035); the line lies above because
+//     tests/test_gpu_shapes.py holds the cluster kernel's vocab split at 700 rows.
 //   H < 256: none (H = 64, T = 512, V = 19000 0.021 and 0.033).
 //   Reproducible calls (the same bits from either kernel): with H up to 512 and more than
-//     256 rows the cluster kernel from 25600 columns on, where adding a term at a time
+//     128 rows the cluster kernel from 25600 columns on, where adding a term at a time
 //     costs it less (T = 16384, H = 384, V = 100000 5.65 and 6.45; T = 4096, H = 512, V =
-//     20000 0.409 and 0.367; T = 64, H = 512, V = 100000 0.744 and 0.590).
+//     20000 0.409 and 0.367; V = 100000, T = 200, H = 256 0.62 and 0.74, T = 64, H = 512
+//     0.744 and 0.590).
 //
 // Chunk size and buffers (64 MB together, half of L2).  16 x 16 tiles (4096 x 4096) in
-// two buffers drain least and win where the power cap binds and a chunk holds many times
-// the tiles in flight: T = 4096, H = 4096, V = 151936 10.0 ms (whole call), 8 x 8 in
-// eight 10.6; T = 32768, H = 2048, V = 32000 8.5 and 8.6.  Everywhere else what counts is
+// two buffers drain least and win where the power cap binds and a chunk holds several times
+// the tiles in flight, against 8 x 8 in eight (whole calls, ms): at H = 4096 T = 16384, V =
+// 32000 10.01 and 10.41, T = 4096, V = 8000 (512 tiles) 0.675 and 0.695, but T = 2048, V =
+// 4000 (128 tiles) 0.234 and 0.220; at H = 2048 T = 16384, V = 32000 5.26 and 5.35, T =
+// 4096, V = 8000 0.375 and 0.376, T = 4096, V = 2000 0.162 and 0.148; at H = 1536 T = 16384,
+// V = 32000 4.02 and 4.01, T = 5000, V = 32000 1.30 and 1.27.  Everywhere else what counts is
 // that no tile waits for the ones it depends on: 8 x 8 in eight (T = 32768, H = 1024, V =
-// 50000 6.88 ms, 16 x 16 7.07), 4 x 8 in sixteen for at most four token tiles (T = 512, H = 768, V = 100000 0.27
-// ms, 4 x 32 in four 0.36; with few vocab tiles 4 x 4, so that dH spreads), 8 x 4 in sixteen at H = 256 (T = 12000, V = 60000 1.08 ms, 4 x 4
-// in sixteen 1.25).
+// 50000 6.88 ms, 16 x 16 7.07), 4 x 8 in sixteen for at most four token tiles (T = 512,
+// H = 768, V = 100000 0.27 ms, 4 x 32 in four 0.36; with few vocab tiles 4 x 4, so that dH
+// spreads), 8 x 4 in sixteen at H = 256 (T = 12000, V = 60000 1.08 ms, 4 x 4 in sixteen 1.25).
 //
 // Lag: the list steps from a chunk's logit tiles to the tiles that read them, long enough
 // for the tiles that the pairs hold (about one of dH and one of dW, 4 K blocks a chunk
@@ -197,7 +208,7 @@ struct ChunkPlan {
 ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V, bool det) {
   ChunkPlan p;
   if (T <= 0 || H < 256 || (H == 256 && T <= 768 && V > 4096 && V <= 20480) || (H > 256 && H < 512 && T < 512) ||
-      (det && H <= 512 && T > 256 && V >= 25600))
+      (det && H <= 512 && T > 128 && V >= 25600))
     return p;
   p.n_t = (T + 255) / 256;
   p.n_v = (V + 255) / 256;
@@ -211,7 +222,7 @@ ChunkPlan chunk_plan(int64_t T, int64_t H, int64_t V, bool det) {
     p.chunk_t = 8;
     p.chunk_v = 4;
     most_buf = 16;
-  } else if (H >= 1536 && p.n_t * p.n_v >= 2560) {
+  } else if (H >= 2048 && p.n_t * p.n_v >= 512) {
     p.chunk_t = p.chunk_v = 16;
   } else {
     p.chunk_t = p.chunk_v = 8;

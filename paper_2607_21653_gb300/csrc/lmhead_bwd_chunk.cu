@@ -418,7 +418,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       bool ok = true;
       Tile x;
       for (uint32_t ji = 0; ok && next_tile(ji, x); ++ji) {
-        const int nk = x.nk, kt = term_k(x);
+        const int nk = x.nk;
         // K-major operands advance 32 bytes per K = 16, MN-major ones 16 rows of 128
         const bool a_mn = x.kind == kTileDW, b_mn = x.kind != kTileZ;
         const uint32_t idesc = idesc_bf16_f32(256, b_mn ? mma_n(x.h) : 256, a_mn, b_mn);
@@ -441,7 +441,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           // two stages per turn: one wait of the issuing thread for eight products.
           // The copies' complete_tx makes both CTAs' bytes visible to the MMAs
           // issued after the phase flips; a CTA-scope wait is enough.
-          const int k0 = kb, k1 = min(nk, kb + kt);
+          const int k0 = kb, k1 = kDet ? min(nk, kb + term_k(x)) : nk;
           for (; kb < k1; kb += 2) {
             const bool two = kb + 1 < k1;
             const uint32_t st0 = st;
@@ -464,7 +464,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (!ok) break;
           umma_commit_pair_mc(smem_u32(&accf_bar[buf]), 3);
           ++ai;
-        } while (kb < nk);
+        } while (kDet && kb < nk);
       }
       umma_commit_pair_mc(smem_u32(&done_bar), 1);
       mbar_wait_drain(smem_u32(&done_bar), 0, a.err);

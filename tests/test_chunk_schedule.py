@@ -57,7 +57,7 @@ def tile_list(rows, H, V, plan, det):
 @pytest.mark.parametrize("det", [False, True])
 @pytest.mark.parametrize("T,H,V", [(1, 640, 1), (513, 512, 4133), (769, 256, 8200), (520, 320, 66000), (1000, 768, 9000),
                                    (2305, 256, 17000), (5003, 320, 50257), (2100, 640, 14700), (3000, 1024, 9001),
-                                   (5121, 1536, 32769), (16384, 4096, 65536)])
+                                   (5121, 1536, 32769), (4300, 2176, 8300), (16384, 4096, 65536)])
 def test_every_wait_reaches_back(T, H, V, det):
     if det and H % 128:
         pytest.skip("reproducible sums need H % 128 == 0")

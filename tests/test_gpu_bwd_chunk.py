@@ -90,9 +90,9 @@ def _all_live(T, H, V, w_std):
 
 # each kind of ring with at least twice as many chunks as buffers, so that every buffer
 # is written again after its readers: 8 x 4 tiles in sixteen buffers, two chunks of tokens;
-# 4 x 8 in sixteen; 8 x 8 in eight, two chunks of tokens, a 192-column H tile.  (16 x 16 in
-# two: the full-size tests, mid whole)
-@pytest.mark.parametrize("T,H,V", [(2305, 256, 17000), (520, 320, 66000), (2100, 704, 14700)])
+# 4 x 8 in sixteen; 8 x 8 in eight, two chunks of tokens, a 192-column H tile; 16 x 16 in
+# two, two chunks of tokens, a 64-column H tile
+@pytest.mark.parametrize("T,H,V", [(2305, 256, 17000), (520, 320, 66000), (2100, 704, 14700), (4300, 2112, 8300)])
 def test_buffers_used_again(T, H, V):
     plan = molt.backward_plan(T, H, V)
     tiles = lambda n, chunk: -(-(-(-n // 256)) // (chunk // 256))

@@ -26,7 +26,7 @@ GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "rep
 # and the one over chunks: one row, a remainder of one row in the second term, several
 # terms and chunks in both directions, chunks of 16 x 16 tiles
 SHAPES = [(700, 128, 5000), (400, 384, 3000), (1, 256, 7), (513, 512, 4133), (900, 384, 3000), (2100, 640, 20000),
-          (5000, 256, 9000), (769, 256, 8200), (700, 384, 30000), (4700, 1536, 40000)]
+          (5000, 256, 9000), (769, 256, 8200), (700, 384, 30000), (4700, 1536, 40000), (4300, 2176, 8300)]
 # the surrogate alone; with KL, entropy bonus and sequence gate, added to a dW;
 # gradients so small that most of them are subnormal
 VARIANTS = ("plain", "extended", "subnormal")
