@@ -574,7 +574,7 @@ def run_ours(args):
         "frac": achieved_bwd / peak,
         "traffic": traffic,
         "traffic_source": traffic_note,
-        "limiter": limiter(executed / peak, clk),
+        "limiter": limiter(executed / peak, clk, args.deterministic),
         "peak_source": f"{peaks['source']} bf16 sustained (kernel timed inside a long step)",
         "kernels_per_step": launches / args.steps,
         "algorithmic_flops_per_launch": 4.0 * tp * H * V_work / max(1, len(mine)),
@@ -634,12 +634,13 @@ def run_ours(args):
     return 0
 
 
-def limiter(executed_frac, clk):
+def limiter(executed_frac, clk, deterministic):
     """What bounds the backward in this run: the logits are formed again in it, so it
     executes 6 T_p H V where 4 T_p H V are counted."""
     at = f"{100 * executed_frac:.0f}% of the sustained cuBLAS rate on what is executed (6 T_p H V; 4 T_p H V counted)"
     if executed_frac < 0.8:
-        return f"not the tensor cores: {at}; launches and waits between tiles"
+        why = "additions of 512-token and 512-column terms to the sums" if deterministic else "waits between tiles"
+        return f"not the tensor cores alone: {at}; {why}"
     cap = "sw_power_cap" in (clk or {}).get("reasons", [])
     return f"tensor cores{' under the board power cap' if cap else ''}: {at}"
 
