@@ -1,8 +1,9 @@
 // Backward pass of the fused LM-head + policy loss on clusters of four CTAs
 // (two tcgen05 CTA pairs), used for short hidden sizes that are multiples of 128
 // where the backward over chunks (lmhead_bwd_chunk.cu) is slower: H = 128, the middle
-// vocabularies of small calls at H = 256, and H = 384 below 512 rows (chunk_plan in
-// api.cu has the rule and the times).  g never leaves the cluster here, so a small
+// vocabularies of small calls at H = 256, H = 384 below 512 rows, and reproducible calls
+// with H up to 512 and many columns, which get the same bits from either kernel
+// (chunk_plan in api.cu has the rule and the times).  g never leaves the cluster here, so a small
 // call needs no round trip through L2 between its products.
 //
 //   g_tv = coef_t (softmax(z_t)_v - [v == x_t]),  coef_t = m_t c_t / D   (Eq. 2)

@@ -8,7 +8,7 @@
 // A chunk is up to 4096 tokens x 4096 vocab columns.  Its g (bf16, at most
 // 32 MB) passes from the products that form it to the products that read it
 // through a ring of a few chunk buffers, 64 MB together, that the 129 MB L2 holds
-// while they are used (as any store it is also written back: 3.5 of the 57.6 GB of
+// while they are used (as any store it is also written back: 3.5 of the 52.9 GB of
 // DRAM traffic at T = 11626 rows, H = 4096, V = 151936); neither the logits nor g of
 // the whole plane exist anywhere.  All three products are then plain 256 x 256
 // tiles on CTA pairs (tcgen05 cta_group::2):
@@ -59,7 +59,7 @@
 // 50257: 0.51 ms, before these three 0.57; T = 3000, H = 1024, V = 32000: 0.355,
 // before 0.399), and by the waits between the tiles of a chunk (see
 // chunk_plan in api.cu).  Counters on T = 8192, H = 4096,
-// V = 32768: tensor pipe active 90 % of the cycles, DRAM 29 %, L2 59 %.
+// V = 32768: tensor pipe active 93 % of the cycles, DRAM 28 %, L2 61 %.
 #include <atomic>
 #include <climits>
 #include <cstdint>
